@@ -3199,9 +3199,13 @@ __global__ void k_t_fill(int64_t n_rows, int64_t ld, int k, const int32_t* __res
     }
 }
 
-// order each transposed row by forward row; pad with (self, -1)
-__global__ void k_t_sort_pad(int64_t n_cols, int64_t ldt, int width, const int* __restrict__ counts,
-                             int32_t* __restrict__ tidx, int32_t* __restrict__ tslot) {
+// order each transposed row by forward row; pad with slot -1 (weight 0) and a
+// valid forward row, since the products read x at every index: column c where
+// the forward operator has such a row, its last row otherwise (D^(P,V) has
+// three times as many columns as rows)
+__global__ void k_t_sort_pad(int64_t n_rows, int64_t n_cols, int64_t ldt, int width,
+                             const int* __restrict__ counts, int32_t* __restrict__ tidx,
+                             int32_t* __restrict__ tslot) {
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_cols;
        c += (int64_t)gridDim.x * blockDim.x) {
     const int m = counts[c];
@@ -3217,7 +3221,7 @@ __global__ void k_t_sort_pad(int64_t n_cols, int64_t ldt, int width, const int* 
       tslot[b * ldt + c] = q;
     }
     for (int a = m; a < width; ++a) {
-      tidx[a * ldt + c] = (int32_t)c;
+      tidx[a * ldt + c] = (int32_t)(c < n_rows ? c : n_rows - 1);
       tslot[a * ldt + c] = -1;
     }
   }
@@ -3478,7 +3482,7 @@ int build_transpose(rbffd_ctx* ctx, AdjointPlan* a, const int32_t* idx, int64_t 
   rc = check_cuda(ctx, cudaMemsetAsync(cursor, 0, sizeof(int) * n_cols, st), "memset");
   if (rc) return rc;
   k_t_fill<<<grid, 256, 0, st>>>(n_rows, ld, k, idx, cursor, t->ld, t->idx, t->slot);
-  k_t_sort_pad<<<grid, 256, 0, st>>>(n_cols, t->ld, t->width, t->counts, t->idx, t->slot);
+  k_t_sort_pad<<<grid, 256, 0, st>>>(n_rows, n_cols, t->ld, t->width, t->counts, t->idx, t->slot);
   return check_cuda(ctx, cudaGetLastError(), "transpose kernels");
 }
 
