@@ -341,25 +341,59 @@ void amg_free(Amg* a) {
   delete a;
 }
 
-int amg_build(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
-              Amg** out, cudaStream_t st) {
-  *out = nullptr;
+namespace {
+
+// The P-node edge graph of a flow: *G, and the boundary conditions *bc.
+int load_graph(rbffd_ctx* ctx, const rbffd_flow& f, HostCsr* G, std::vector<uint8_t>* bc,
+               cudaStream_t st) {
   if (!f.p_edges || f.n_edges <= 0 || !f.p_x || !f.p_y)
     return set_error(ctx, RBFFD_ERR_INVALID_ARG,
                      "precond = 1 needs the P-node edges (p_edges, n_edges) and p_x, p_y");
   const int64_t M = f.M;
   std::vector<int32_t> e;
   std::vector<double> x, y;
-  std::vector<uint8_t> bc;
   int rc = download(ctx, f.p_edges, (size_t)(2 * f.n_edges), &e, st);
   if (!rc) rc = download(ctx, f.p_x, (size_t)M, &x, st);
   if (!rc) rc = download(ctx, f.p_y, (size_t)M, &y, st);
-  if (!rc) rc = download(ctx, f.p_bc, (size_t)M, &bc, st);
+  if (!rc) rc = download(ctx, f.p_bc, (size_t)M, bc, st);
   if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "multigrid download");
   if (rc) return rc;
-  std::vector<HostCsr> L(1);
-  std::string why = edge_graph(M, f.n_edges, e, x, y, bc, &L[0]);
+  std::string why = edge_graph(M, f.n_edges, e, x, y, *bc, G);
   if (!why.empty()) return set_error(ctx, RBFFD_ERR_INVALID_ARG, "pressure graph: %s", why.c_str());
+  return RBFFD_OK;
+}
+
+bool has_dirichlet(const std::vector<uint8_t>& bc) {
+  return std::find(bc.begin(), bc.end(), (uint8_t)RBFFD_PBC_DIRICHLET) != bc.end();
+}
+
+}  // namespace
+
+int amg_check(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
+              cudaStream_t st) {
+  HostCsr G;
+  std::vector<uint8_t> bc;
+  const int rc = load_graph(ctx, f, &G, &bc, st);
+  if (rc) return rc;
+  double ces = 0.0;
+  for (int64_t i = 0; i < f.M; ++i) {
+    if (!std::isfinite(G.diag[i]))
+      return set_error(ctx, RBFFD_ERR_INVALID_ARG, "coarsest pressure graph matrix is not positive");
+    ces += (diag_a[i] != 0.0 ? G.diag[i] / diag_a[i] : G.diag[i]) * es[i];
+  }
+  if (!has_dirichlet(bc) && (!(ces != 0.0) || !std::isfinite(ces)))
+    return set_error(ctx, RBFFD_ERR_INVALID_ARG, "pressure rank-one column is zero");
+  return RBFFD_OK;
+}
+
+int amg_build(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
+              Amg** out, cudaStream_t st) {
+  *out = nullptr;
+  const int64_t M = f.M;
+  std::vector<uint8_t> bc;
+  std::vector<HostCsr> L(1);
+  int rc = load_graph(ctx, f, &L[0], &bc, st);
+  if (rc) return rc;
   std::vector<std::vector<int32_t>> aggs;
   while (L.back().n > kAmgCoarse && (int)L.size() < kAmgMaxLevels) {
     const HostCsr& A = L.back();
@@ -378,8 +412,7 @@ int amg_build(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const d
     return set_error(ctx, RBFFD_ERR_INVALID_ARG,
                      "pressure graph does not coarsen below %lld nodes (disconnected?)",
                      (long long)L.back().n);
-  bool pdir = false;
-  for (int64_t i = 0; i < M; ++i) pdir = pdir || bc[i] == RBFFD_PBC_DIRICHLET;
+  const bool pdir = has_dirichlet(bc);
   std::vector<double> Xd;
   if (!coarse_inverse(L.back(), &Xd, !pdir))
     return set_error(ctx, RBFFD_ERR_INVALID_ARG, "coarsest pressure graph matrix is not positive");

@@ -107,5 +107,10 @@ struct Amg {
 int amg_build(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
               Amg** out, cudaStream_t st);
 void amg_free(Amg* a);
+// The checks amg_build makes of the flow's edge graph, without building
+// anything (a plan that solves small systems directly still refuses the
+// descriptions that the hierarchy refuses).
+int amg_check(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
+              cudaStream_t st);
 
 }  // namespace rbffd

@@ -1,0 +1,406 @@
+// Direct pressure solve of small systems (Section 3, Eq. pressure_Poisson; the
+// paper factorises its implicit matrices once, too): the dense inverse of the
+// scaled operator A_f = A + es 1^T is built once per plan, and a solve is a
+// product with it inside iterative refinement on the sparse operator, in one
+// cooperative launch.
+#include <algorithm>
+#include <cmath>
+
+#include "gridsync.cuh"
+#include "psolve.cuh"
+
+namespace rbffd {
+
+namespace {
+
+constexpr int kMaxSweeps = 8;
+constexpr int kOwn = 32;  // rows a block of the inversion owns, at most
+
+// T = A + es 1^T, one block per row
+__global__ void __launch_bounds__(256)
+    k_dense_fill(int n, int64_t ld, int k, const int32_t* __restrict__ idx,
+                 const double* __restrict__ w, const double* __restrict__ es,
+                 double* __restrict__ T, int ldt) {
+  const int i = blockIdx.x;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) T[(int64_t)i * ldt + j] = es[i];
+  __syncthreads();
+  if (threadIdx.x == 0)  // a padded row may repeat a column
+    for (int s = 0; s < k; ++s) T[(int64_t)i * ldt + idx[s * ld + i]] += w[s * ld + i];
+}
+
+struct InvArgs {
+  int n, ldt;
+  double* T;
+  int* prow;             // [n] pivot row of step k
+  double* cand_v;        // [2][gridDim.x] each block's best pivot candidate
+  int* cand_r;           // [2][gridDim.x]
+  double* partials;
+  unsigned int* arrivals;  // zero at launch
+  int* status;             // 0 on entry; 1: singular, 2: non-finite
+};
+
+// Gauss-Jordan exchange with partial pivoting, in place: step k exchanges
+// row p (the largest |T[i][k]| among the rows not yet used) with column k.
+// Block b owns rows b, b + gridDim.x, ...; rows are never moved.  One barrier
+// per step: every block reads row p as step k - 1 left it, and its owner
+// rescales it while it applies step k + 1.
+//
+// What bounds it: n^2 FP64 FMAs and one pass over the matrix (in L2 up to about
+// n = 3,500) per step: 6 us a step at n = 1,600 and 13 us at 2,700, of which
+// the barrier and the pivot search are 4 us.  A blocked form would save memory
+// traffic, not FP64 instructions, which are the larger part on this GPU.
+__global__ void __launch_bounds__(kPT, 1) k_dense_invert(const __grid_constant__ InvArgs a) {
+  __shared__ double sh[kNVMax * kPT];
+  __shared__ double part[kNVMax * 4];
+  __shared__ double f[kOwn], cv[kOwn], s_inv;
+  __shared__ int used[kOwn], okf, s_p, s_bad;
+  Grid g{sh, part, &okf, a.partials, a.arrivals};
+  const int tid = threadIdx.x, n = a.n, nb = gridDim.x, blk = blockIdx.x;
+  const int own = blk < n ? (n - blk + nb - 1) / nb : 0;
+  if (tid < kOwn) {
+    used[tid] = 0;
+    cv[tid] = tid < own ? fabs(a.T[(int64_t)(blk + tid * nb) * a.ldt]) : -1.0;
+  }
+  if (tid == 0) s_bad = 0;
+  int pend = -1, kprev = 0;  // own row still to be rescaled by the last step's pivot
+  double inv_prev = 0.0;
+  for (int k = 0; k < n; ++k) {
+    __syncthreads();
+    if (tid < 32) {  // this block's candidate: largest magnitude, lowest row on ties
+      double v = tid < own && !used[tid] ? cv[tid] : -1.0;
+      if (!(v == v)) v = INFINITY;  // NaN: picked, then caught below
+      int r = blk + tid * nb;
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int orr = __shfl_xor_sync(0xffffffffu, r, o);
+        if (ov > v || (ov == v && orr < r)) {
+          v = ov;
+          r = orr;
+        }
+      }
+      if (tid == 0) {
+        a.cand_v[(k & 1) * nb + blk] = v;
+        a.cand_r[(k & 1) * nb + blk] = r;
+      }
+    }
+    if (!g.sync()) return;
+    if (tid < 32) {
+      double v = -2.0;
+      int r = n;
+      for (int b = tid; b < nb; b += 32) {
+        const double ov = a.cand_v[(k & 1) * nb + b];
+        const int orr = a.cand_r[(k & 1) * nb + b];
+        if (ov > v || (ov == v && orr < r)) {
+          v = ov;
+          r = orr;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int orr = __shfl_xor_sync(0xffffffffu, r, o);
+        if (ov > v || (ov == v && orr < r)) {
+          v = ov;
+          r = orr;
+        }
+      }
+      if (tid == 0) {
+        s_p = r;
+        // rows are scaled to a unit diagonal: a pivot this small is rounding
+        s_bad = !isfinite(v) ? 2 : (v > 1e-13 ? 0 : 1);
+        if (!s_bad) s_inv = 1.0 / a.T[(int64_t)r * a.ldt + k];
+      }
+    }
+    // the multipliers of the own rows in column k, before it is overwritten
+    if (tid >= 32 && tid < 32 + own) {
+      const int q = tid - 32;
+      double v = a.T[(int64_t)(blk + q * nb) * a.ldt + k];
+      if (q == pend) v = -v * inv_prev;  // k != kprev
+      f[q] = v;
+    }
+    __syncthreads();
+    if (s_bad) {
+      if (blk == 0 && tid == 0) *a.status = s_bad;
+      return;
+    }
+    const int p = s_p;
+    const double inv = s_inv;
+    const int qp = p % nb == blk ? p / nb : -1;
+    const double* Tp = a.T + (int64_t)p * a.ldt;
+    for (int j = tid; j < n; j += kPT) {
+      const double t = j == k ? inv : -Tp[j] * inv;
+      double* col = a.T + (int64_t)blk * a.ldt + j;
+      const int64_t step = (int64_t)nb * a.ldt;
+#pragma unroll 4
+      for (int q = 0; q < own; ++q) {
+        if (q == qp) continue;
+        double old = j == k ? 0.0 : col[q * step];
+        if (q == pend && j != k) old = j == kprev ? inv_prev : -old * inv_prev;
+        const double v = fma(f[q], t, old);
+        col[q * step] = v;
+        if (j == k + 1) cv[q] = fabs(v);
+      }
+    }
+    if (tid == 0) {
+      if (qp >= 0) used[qp] = 1;
+      if (blk == 0) a.prow[k] = p;
+    }
+    pend = qp;
+    inv_prev = inv;
+    kprev = k;
+  }
+  if (!g.sync()) return;  // the other blocks still read the last pivot row in their last step
+  if (pend >= 0) {
+    double* row = a.T + (int64_t)(blk + pend * nb) * a.ldt;
+    for (int j = tid; j < n; j += kPT) row[j] = j == kprev ? inv_prev : -row[j] * inv_prev;
+  }
+}
+
+// out[k][prow[j]] = T[prow[k]][j], rows padded with zeros to ldt
+__global__ void __launch_bounds__(256)
+    k_dense_order(int n, int ldt, const int* __restrict__ prow, const double* __restrict__ T,
+                  double* __restrict__ out) {
+  const int k = blockIdx.x;
+  const double* row = T + (int64_t)prow[k] * ldt;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) out[(int64_t)k * ldt + prow[j]] = row[j];
+}
+
+struct DArgs {
+  int M, rows, k, ldt;
+  int64_t ld;
+  const int32_t* idx;
+  const double *w, *es, *inv;
+  const double* b;
+  double *x, *r;  // r: ldt values, zero beyond M
+  double tol2;
+  double* partials;
+  unsigned int* arrivals;
+  PSolveResult* res;
+};
+
+// Refinement: r = b - A_f x, x += A_f^-1 r until (r, r) <= tol^2 (b, b).  A
+// block owns `rows` consecutive rows, in the residual (one thread per row) and
+// in the product (one warp per row, r in shared memory).  What bounds it: the
+// product's M^2 FP64 FMAs (4.1 us at 1,600 rows on the FP64 pipe) and the
+// latency of its four phases.
+template <int K>
+__global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs a) {
+  __shared__ __align__(16) double sh[kNVMax * kPT];
+  static_assert(kNVMax * kPT >= kDenseMax, "the residual is staged in sh");
+  __shared__ double part[kNVMax * 4];
+  __shared__ double s_sig, s_rr, s_bb;
+  __shared__ int okf;
+  Grid g{sh, part, &okf, a.partials, a.arrivals};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = min(a.M, a.rows * (int)blockIdx.x), r1 = min(a.M, r0 + a.rows);
+  const int active = min(kPT, (a.rows + 31) / 32 * 32);
+  {
+    double sx = 0.0;
+    for (int i = r0 + tid; i < r1; i += kPT) sx += a.x[i];
+    const double v[1] = {sx};
+    if (!g.reduce<1>(v, active, [&](const double* t) { s_sig = t[0]; })) return;
+  }
+  double prev = INFINITY;
+  for (int sweep = 0;; ++sweep) {
+    double d0 = 0.0, d1 = 0.0;
+    const double sig = s_sig;
+    for (int i = r0 + tid; i < r1; i += kPT) {
+      double ax = 0.0;
+      if constexpr (K > 0) {
+#pragma unroll
+        for (int s = 0; s < K; ++s)
+          ax += __ldg(a.w + s * a.ld + i) * a.x[__ldg(a.idx + s * a.ld + i)];
+      } else {
+#pragma unroll 4
+        for (int s = 0; s < a.k; ++s)
+          ax += __ldg(a.w + s * a.ld + i) * a.x[__ldg(a.idx + s * a.ld + i)];
+      }
+      const double bi = a.b[i], ri = bi - (ax + __ldg(a.es + i) * sig);
+      a.r[i] = ri;
+      d0 += ri * ri;
+      d1 += bi * bi;
+    }
+    const double v[2] = {d0, d1};
+    const bool ok = g.reduce<2>(v, active, [&](const double* t) {
+      s_rr = t[0];
+      s_bb = t[1];
+    });
+    if (!ok) return;
+    const double rr = s_rr, bb = s_bb;
+    const bool conv = rr <= a.tol2 * bb, fin = isfinite(rr);
+    // a sweep that does not halve the residual has reached the rounding level
+    const bool stalled = sweep > 0 && !(rr < 0.25 * prev);
+    if (conv || !fin || stalled || sweep >= kMaxSweeps) {
+      if (blockIdx.x == 0 && tid == 0) {
+        a.res->iters = sweep;
+        a.res->status = conv ? 0 : (fin ? 5 : 2);
+        a.res->relres = bb > 0 ? sqrt(rr / bb) : sqrt(rr);
+        a.res->converged = conv;
+      }
+      return;
+    }
+    prev = rr;
+    // x += inv r: the rows' products need all of r, read once per block
+    for (int j = tid; j < a.ldt; j += kPT) sh[j] = a.r[j];
+    __syncthreads();
+    double sx = 0.0;
+    for (int i = r0 + warp; i < r1; i += kPW) {
+      const double2* row = reinterpret_cast<const double2*>(a.inv + (int64_t)i * a.ldt);
+      const double2* r2 = reinterpret_cast<const double2*>(sh);
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+      for (int j = lane; j < a.ldt / 2; j += 32) {
+        const double2 u = __ldg(row + j), q = r2[j];
+        s0 = fma(u.x, q.x, s0);
+        s1 = fma(u.y, q.y, s1);
+      }
+      const double s = warp_sum(s0 + s1);
+      if (lane == 0) {
+        const double xi = a.x[i] + s;
+        a.x[i] = xi;
+        sx += xi;
+      }
+    }
+    __syncthreads();  // sh is reused by the reduction
+    const double vx[1] = {sx};
+    if (!g.reduce<1>(vx, kPT, [&](const double* t) { s_sig = t[0]; })) return;
+  }
+}
+
+}  // namespace
+
+struct DSolve {
+  std::vector<void*> allocs;
+  int grid = 0;
+  DArgs a{};
+};
+
+void dsolve_free(DSolve* d) {
+  if (!d) return;
+  for (void* q : d->allocs) cudaFree(q);
+  delete d;
+}
+
+namespace {
+
+template <typename T>
+int d_alloc(rbffd_ctx* ctx, DSolve* d, T** out, size_t count, cudaStream_t st) {
+  void* ptr = nullptr;
+  const int rc = check_cuda(ctx, cudaMalloc(&ptr, sizeof(T) * count), "direct solve alloc");
+  if (rc) return rc;
+  d->allocs.push_back(ptr);
+  *out = (T*)ptr;
+  return check_cuda(ctx, cudaMemsetAsync(ptr, 0, sizeof(T) * count, st), "memset");
+}
+
+int invert(rbffd_ctx* ctx, DSolve* d, const InvArgs& in, const double* es, double* out, int* h_status,
+           cudaStream_t st) {
+  DArgs& a = d->a;
+  k_dense_fill<<<a.M, 256, 0, st>>>(a.M, a.ld, a.k, a.idx, a.w, es, in.T, a.ldt);
+  int rc = check_cuda(ctx, cudaGetLastError(), "dense operator");
+  if (rc) return rc;
+  InvArgs arg = in;
+  void* args[] = {&arg};
+  rc = check_cuda(ctx, cudaLaunchCooperativeKernel((const void*)k_dense_invert, dim3(d->grid),
+                                                   dim3(kPT), args, 0, st), "dense inverse");
+  if (rc) return rc;
+  int* h = (int*)ctx->host_pinned;
+  unsigned int* arrived = (unsigned int*)(h + 1);
+  rc = check_cuda(ctx, cudaMemcpyAsync(h, in.status, sizeof(int), cudaMemcpyDeviceToHost, st),
+                  "inverse status");
+  if (!rc)
+    rc = check_cuda(ctx, cudaMemcpyAsync(arrived, in.arrivals, sizeof(unsigned int),
+                                         cudaMemcpyDeviceToHost, st), "inverse status");
+  if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "dense inverse sync");
+  if (rc) return rc;
+  *h_status = *h;
+  if (*h == 0 && *arrived != (unsigned int)d->grid * ((unsigned int)a.M + 1u))
+    return set_error(ctx, RBFFD_ERR_CUDA, "dense inverse: grid barrier not reached (bounded wait)");
+  if (*h == 0) {
+    k_dense_order<<<a.M, 256, 0, st>>>(a.M, a.ldt, in.prow, in.T, out);
+    rc = check_cuda(ctx, cudaGetLastError(), "dense inverse order");
+  }
+  return rc;
+}
+
+}  // namespace
+
+int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* idx,
+                 const double* w, const double* es, DSolve** out, cudaStream_t st) {
+  *out = nullptr;
+  DSolve* d = new DSolve();
+  d->grid = sm_count();
+  DArgs& a = d->a;
+  a.M = (int)M;
+  a.rows = (int)((M + d->grid - 1) / d->grid);
+  a.k = k;
+  a.ld = ld;
+  a.ldt = (int)round_up(M, 2);
+  a.idx = idx;
+  a.w = w;
+  a.es = es;
+  InvArgs in{};
+  in.n = a.M;
+  in.ldt = a.ldt;
+  const size_t nn = (size_t)M * a.ldt;
+  double* inv = nullptr;
+  int rc = 0, bad = 0;
+  if (a.rows > kOwn)  // fewer SMs than the ownership tables assume
+    rc = -1;
+  if (!rc) rc = d_alloc(ctx, d, &inv, nn, st);
+  if (!rc) rc = d_alloc(ctx, d, &in.T, nn, st);
+  void* work = in.T;
+  if (!rc) rc = d_alloc(ctx, d, &in.prow, (size_t)M, st);
+  if (!rc) rc = d_alloc(ctx, d, &in.cand_v, (size_t)2 * d->grid, st);
+  if (!rc) rc = d_alloc(ctx, d, &in.cand_r, (size_t)2 * d->grid, st);
+  if (!rc) rc = d_alloc(ctx, d, &in.status, 1, st);
+  if (!rc) rc = d_alloc(ctx, d, &a.partials, (size_t)2 * kNVMax * d->grid, st);
+  if (!rc) rc = d_alloc(ctx, d, &a.arrivals, 1, st);
+  if (!rc) rc = d_alloc(ctx, d, &a.res, 1, st);
+  if (!rc) rc = d_alloc(ctx, d, &a.r, (size_t)a.ldt, st);
+  in.partials = a.partials;
+  in.arrivals = a.arrivals;
+  a.inv = inv;
+  if (!rc) rc = invert(ctx, d, in, es, inv, &bad, st);
+  if (!rc && !bad) rc = check_cuda(ctx, cudaStreamSynchronize(st), "dense inverse sync");
+  if (rc || bad) {
+    cudaStreamSynchronize(st);
+    dsolve_free(d);
+    // singular to working precision, or no room: the Krylov solve takes over
+    return rc == RBFFD_ERR_CUDA ? rc : RBFFD_OK;
+  }
+  for (void*& q : d->allocs)  // the inversion's matrix is not needed any more
+    if (q == work) {
+      cudaFree(q);
+      q = nullptr;
+    }
+  *out = d;
+  return RBFFD_OK;
+}
+
+int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
+               PSolveResult* res, int64_t* launches, cudaStream_t st) {
+  DArgs a = d->a;
+  a.x = x;
+  a.b = b;
+  a.tol2 = tol * tol;
+  PSolveResult* h = (PSolveResult*)ctx->host_pinned;
+  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, sizeof(unsigned int), st), "memset");
+  if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
+  if (rc) return rc;
+  const void* fn = a.k == 28 ? (const void*)k_dsolve<28> : (const void*)k_dsolve<0>;
+  void* args[] = {&a};
+  rc = check_cuda(ctx, cudaLaunchCooperativeKernel(fn, dim3(d->grid), dim3(kPT), args, 0, st),
+                  "direct pressure solve");
+  if (!rc)
+    rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(PSolveResult), cudaMemcpyDeviceToHost, st),
+                    "direct solve result");
+  if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "direct solve sync");
+  if (rc) return rc;
+  *launches += 1;
+  if (h->iters < 0)  // the kernel gave up before it could write its result
+    return set_error(ctx, RBFFD_ERR_CUDA, "direct solve: grid barrier not reached (bounded wait)");
+  *res = *h;
+  return RBFFD_OK;
+}
+
+}  // namespace rbffd

@@ -1,0 +1,66 @@
+// The preconditioned pressure solve as one resident kernel (psolve.cu), and
+// the direct solve of small systems (dsolve.cu).
+#pragma once
+
+#include "amg.cuh"
+#include "common.cuh"
+
+namespace rbffd {
+
+struct PSolve;
+
+// Up to this many rows the resident kernel is the faster form; beyond it the
+// phases are long enough to hide their launches, and the graph of separate
+// launches, whose products and level-0 sweeps have more warps in flight, is
+// (FP64 step at 1M rows: 33.7 ms a step as launches, 34.2 resident; at 100k
+// rows 9.9 against 7.9, MIXED at 250k rows 17.3 against 15.5).
+constexpr int64_t kResidentMax = 1 << 19;
+
+struct PSolveResult {
+  int iters = 0;
+  int status = 0;  // as KScal::status of step.cu
+  double relres = 0.0;
+  bool converged = false;
+};
+
+// Build the solve's copies for one plan: the scaled pressure operator (idx, w
+// [k][ld], rank-one column es, row sums a1; M rows) in the hierarchy's level-0
+// order, in FP64, or in FP32 when `mix` is set, and its work vectors.
+int psolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* idx,
+                 const double* w, const double* es, const double* a1, const Amg* amg, bool mix,
+                 PSolve** out, cudaStream_t st);
+void psolve_free(PSolve* p);
+
+// Right-preconditioned BiCGSTAB on the scaled pressure system, x (in: the
+// initial iterate, not read when x_zero; out: the solution) and b in P-node
+// order; T = float or double as the plan was built.  Synchronises `st`.
+// `launches` is increased by the kernels launched.
+template <typename T>
+int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxit, uint32_t seed,
+               bool x_zero, PSolveResult* res, int64_t* launches, cudaStream_t st);
+
+// Small systems (M <= kDenseMax) are solved directly: the dense FP64 inverse
+// of the scaled pressure operator, built once per plan, applied with iterative
+// refinement.
+//
+// Where the line lies: a solve takes one product with the inverse and two
+// residuals, 16 us at 1,600 rows, 30 us at 2,700 and about 60 us at 4,096
+// (16.8 M FP64 FMAs, and an inverse of 134 MB that no longer stays in L2),
+// against 40 to 55 us for EACH of the 40 to 500 Krylov iterations that these
+// sizes take; beyond it the inversion (n^3 FP64 FMAs, 0.2 s at 4,096) would
+// cost a first pass more than the hierarchy it replaces.
+constexpr int kDenseMax = 4096;
+struct DSolve;
+
+// *out stays null when the operator is numerically singular (the caller then
+// takes the Krylov solve).  Synchronises `st`.
+int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* idx,
+                 const double* w, const double* es, DSolve** out, cudaStream_t st);
+void dsolve_free(DSolve* d);
+// x (in: the initial iterate, out: the solution) and b in P-node order.
+// Refines until the relative residual is at most tol; res->iters counts the
+// products with the inverse.  status 5: the refinement stalled above tol.
+int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
+               PSolveResult* res, int64_t* launches, cudaStream_t st);
+
+}  // namespace rbffd

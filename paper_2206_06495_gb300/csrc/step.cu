@@ -37,6 +37,7 @@
 
 #include "amg.cuh"
 #include "common.cuh"
+#include "psolve.cuh"
 
 namespace rbffd {
 
@@ -1919,6 +1920,9 @@ struct StepPlan {
   double* dscal = nullptr;  // [0]: sum, [1..6]: residual norms
   struct AdjointPlan* adj = nullptr;  // transposed operators, built on first use
   Amg* amg = nullptr;                 // pressure preconditioner (precond = 1)
+  PSolve* ps = nullptr;               // the preconditioned solve's resident kernel
+  DSolve* ds = nullptr;               // small systems: the direct solve (amg and ps are then
+                                      // built when something needs the Krylov solve)
   double* a1 = nullptr;    // row sums of the FP64 pressure operator
   float* a1_32 = nullptr;  // the same in FP32 (complement of the difference-form FP32 rows)
   // tile records of the pressure and viscous operators the Krylov solves
@@ -1965,6 +1969,8 @@ void adjoint_plan_free(struct AdjointPlan* a);
 void step_plan_free(StepPlan* p) {
   if (!p) return;
   adjoint_plan_free(p->adj);
+  psolve_free(p->ps);
+  dsolve_free(p->ds);
   amg_free(p->amg);
   for (auto& g : p->graphs) cudaGraphExecDestroy(g.exec);
   if (p->cap) cudaStreamDestroy(p->cap);
@@ -2001,6 +2007,72 @@ rbffd_flow plan_key(const rbffd_flow& f) {
   k.tol = k.inner_tol = 0.0;
   k.max_iter = k.km_mode = k.overwrite_bc = k.profile = k.cn_form = 0;
   return k;
+}
+
+// tile records of an operator in the solves' precision
+int tile_records(rbffd_ctx* ctx, StepPlan* p, int64_t rows, int64_t ld, const int32_t* idx,
+                 const double* w64, const float* w32, unsigned char** out, cudaStream_t st) {
+  const size_t wsz = p->mix ? sizeof(float) : sizeof(double);
+  const size_t rec = (size_t)p->k * kTileRows * (sizeof(int32_t) + wsz);
+  const int64_t ntiles = (rows + kTileRows - 1) / kTileRows;
+  const int rc = palloc(ctx, p, out, rec * (size_t)ntiles);
+  if (rc) return rc;
+  if (p->mix)
+    k_tile_records<float><<<p->grid, kThreads, 0, st>>>(ld, p->k, ntiles, idx, w32, *out);
+  else
+    k_tile_records<double><<<p->grid, kThreads, 0, st>>>(ld, p->k, ntiles, idx, w64, *out);
+  return check_cuda(ctx, cudaGetLastError(), "tile records");
+}
+
+// host copies of the scaled pressure operator's diagonal and rank-one column
+int pressure_diag(rbffd_ctx* ctx, StepPlan* p, const rbffd_flow& f, std::vector<double>* hd,
+                  std::vector<double>* hes, cudaStream_t st) {
+  hd->resize(f.M);
+  hes->resize(f.M);
+  k_diag<<<p->grid, kThreads, 0, st>>>(f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->kw64[0][0]);
+  int rc = check_cuda(ctx, cudaGetLastError(), "diagonal");
+  if (!rc)
+    rc = check_cuda(ctx, cudaMemcpyAsync(hd->data(), p->kw64[0][0], sizeof(double) * f.M,
+                                         cudaMemcpyDeviceToHost, st),
+                    "diagonal copy");
+  if (!rc)
+    rc = check_cuda(ctx, cudaMemcpyAsync(hes->data(), p->es, sizeof(double) * f.M,
+                                         cudaMemcpyDeviceToHost, st),
+                    "rank-one column copy");
+  if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "diagonal sync");
+  return rc;
+}
+
+// The multigrid hierarchy of the P-node edge graph, scaled to the pressure
+// rows, and the preconditioned Krylov solve on it.
+int build_precond(rbffd_ctx* ctx, StepPlan* p, const rbffd_flow& f, const std::vector<double>& hd,
+                  const std::vector<double>& hes, cudaStream_t st) {
+  int rc = 0;
+  if (!p->a1) {
+    if ((rc = palloc(ctx, p, &p->a1, f.M))) return rc;
+    k_rowsum<double><<<p->grid, kThreads, 0, st>>>(f.M, f.ld_p, p->kL, p->Lw, p->a1);
+    if ((rc = check_cuda(ctx, cudaGetLastError(), "row sums"))) return rc;
+    // the FP32 pressure rows are applied in difference form with the FP64
+    // row sums (near zero) as their diagonal complement (see k_spmv_pc)
+    if (p->mix && (rc = to32(ctx, p, p->a1, f.M, &p->a1_32, st))) return rc;
+    // the composed operator's width is not the staged tiles' k: its SpMVs
+    // read rows directly, as the FP64 ones do
+    if (p->mix && !p->proj &&
+        (rc = tile_records(ctx, p, f.M, f.ld_p, p->Lidx, p->Lw, p->Lw32, &p->Lt, st)))
+      return rc;
+  }
+  if ((rc = amg_build(ctx, f, hd.data(), hes.data(), &p->amg, st))) return rc;
+  if (f.M > kResidentMax) return RBFFD_OK;
+  return psolve_build(ctx, f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->es, p->a1, p->amg, p->mix,
+                      &p->ps, st);
+}
+
+// the same for a plan whose direct solve has made do without it so far
+int need_precond(rbffd_ctx* ctx, StepPlan* p, const rbffd_flow& f, cudaStream_t st) {
+  if (p->amg) return RBFFD_OK;
+  std::vector<double> hd, hes;
+  const int rc = pressure_diag(ctx, p, f, &hd, &hes, st);
+  return rc ? rc : build_precond(ctx, p, f, hd, hes, st);
 }
 
 int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t st) {
@@ -2145,28 +2217,8 @@ int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t
               set_error(ctx, RBFFD_ERR_INVALID_ARG,
                         "exact projection needs wall V-nodes with normals (v_bc, v_nx, v_ny)"));
   }
-  if (f.precond) {
-    // multigrid hierarchy of the P-node edge graph, scaled to the pressure rows
-    std::vector<double> hd(f.M), hes(f.M);
-    k_diag<<<p->grid, kThreads, 0, st>>>(f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->kw64[0][0]);
-    TRY(check_cuda(ctx, cudaGetLastError(), "diagonal"));
-    TRY(check_cuda(ctx, cudaMemcpyAsync(hd.data(), p->kw64[0][0], sizeof(double) * f.M,
-                                        cudaMemcpyDeviceToHost, st),
-                   "diagonal copy"));
-    TRY(check_cuda(ctx, cudaMemcpyAsync(hes.data(), p->es, sizeof(double) * f.M,
-                                        cudaMemcpyDeviceToHost, st),
-                   "rank-one column copy"));
-    TRY(check_cuda(ctx, cudaStreamSynchronize(st), "diagonal sync"));
-    TRY(amg_build(ctx, f, hd.data(), hes.data(), &p->amg, st));
-    TRY(palloc(ctx, p, &p->a1, f.M));
-    k_rowsum<double><<<p->grid, kThreads, 0, st>>>(f.M, f.ld_p, p->kL, p->Lw, p->a1);
-    TRY(check_cuda(ctx, cudaGetLastError(), "row sums"));
-  }
   if (p->mix) {
     TRY(to32(ctx, p, p->Lw, np, &p->Lw32, st));
-    // the FP32 pressure rows are applied in difference form with the FP64
-    // row sums (near zero) as their diagonal complement (see k_spmv_pc)
-    if (f.precond) TRY(to32(ctx, p, p->a1, f.M, &p->a1_32, st));
     TRY(to32(ctx, p, p->es, f.M, &p->es32, st));
     TRY(to32(ctx, p, p->Hw, nv, &p->Hw32, st));
     if (p->open) TRY(to32(ctx, p, p->Hw_v, nv, &p->Hw32_v, st));
@@ -2192,29 +2244,20 @@ int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t
       TRY(palloc(ctx, p, &p->r64[b], nmax));
     }
   }
-  {
-    const size_t wsz = p->mix ? sizeof(float) : sizeof(double);
-    const size_t rec = (size_t)p->k * kTileRows * (sizeof(int32_t) + wsz);
-    auto records = [&](int64_t rows, int64_t ld, const int32_t* idx, const double* w64,
-                       const float* w32, unsigned char** out) -> int {
-      const int64_t ntiles = (rows + kTileRows - 1) / kTileRows;
-      int rc = palloc(ctx, p, out, rec * (size_t)ntiles);
-      if (rc) return rc;
-      if (p->mix)
-        k_tile_records<float><<<p->grid, kThreads, 0, st>>>(ld, p->k, ntiles, idx, w32, *out);
-      else
-        k_tile_records<double><<<p->grid, kThreads, 0, st>>>(ld, p->k, ntiles, idx, w64, *out);
-      return check_cuda(ctx, cudaGetLastError(), "tile records");
-    };
-    if (p->open) {
-      TRY(records(f.N, f.ld_v, p->Hidx, p->Hw, p->Hw32, &p->Ht));
-      TRY(records(f.N, f.ld_v, p->Hidx, p->Hw_v, p->Hw32_v, &p->Ht_v));
-    } else {
-      TRY(records(f.N, f.ld_v, f.vv_idx, p->Hw, p->Hw32, &p->Ht));
+  if (p->open) {
+    TRY(tile_records(ctx, p, f.N, f.ld_v, p->Hidx, p->Hw, p->Hw32, &p->Ht, st));
+    TRY(tile_records(ctx, p, f.N, f.ld_v, p->Hidx, p->Hw_v, p->Hw32_v, &p->Ht_v, st));
+  } else {
+    TRY(tile_records(ctx, p, f.N, f.ld_v, f.vv_idx, p->Hw, p->Hw32, &p->Ht, st));
+  }
+  if (f.precond) {
+    std::vector<double> hd, hes;
+    TRY(pressure_diag(ctx, p, f, &hd, &hes, st));
+    if (f.M <= kDenseMax) {
+      TRY(amg_check(ctx, f, hd.data(), hes.data(), st));
+      TRY(dsolve_build(ctx, f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->es, &p->ds, st));
     }
-    // the composed operator's width is not the staged tiles' k: its SpMVs
-    // read rows directly
-    if (f.precond && !p->proj) TRY(records(f.M, f.ld_p, p->Lidx, p->Lw, p->Lw32, &p->Lt));
+    if (!p->ds) TRY(build_precond(ctx, p, f, hd, hes, st));
   }
 #undef TRY
   *out = p;
@@ -2751,6 +2794,24 @@ int bicgstab(rbffd_ctx* ctx, StepPlan* P, const KOp<TW, TV>& op, TV* const* x,
   return RBFFD_OK;
 }
 
+// The preconditioned pressure solve in its resident kernel (psolve.cu).
+template <typename T>
+int resident_solve(rbffd_ctx* ctx, StepPlan* P, T* x, const T* b, double tol, int maxit,
+                   SolveResult* res, cudaStream_t st, uint32_t seed = 0, bool x_zero = false) {
+  PSolveResult r;
+  const int rc = psolve_run<T>(ctx, P->ps, x, b, tol, maxit, seed, x_zero, &r, &P->launches, st);
+  if (rc) return rc;
+  res->iters = r.iters;
+  res->status = r.status;
+  res->relres = r.relres;
+  res->converged = r.converged;
+  res->resumable = false;
+  if (trace_on())
+    fprintf(stderr, "[rbffd] pressure %s iters=%d relres=%.3e status=%d\n",
+            sizeof(T) == 8 ? "fp64" : "fp32", r.iters, r.relres, r.status);
+  return RBFFD_OK;
+}
+
 // FP64 iterative refinement: the residual uses the FP64 operator; each
 // correction solves the FP32 copy of the operator in FP32 (FP32 weights,
 // vectors and recurrences; the pressure solves with the FP32 V-cycle) to a
@@ -2839,9 +2900,13 @@ int refine(rbffd_ctx* ctx, StepPlan* P, const KOp<double, double>& op64,
     const double resume =
         resumable && nrm[0] > 0.0 && last_nrm[0] > 0.0 ? last_nrm[0] / nrm[0] : 0.0;
     SolveResult inner;
-    rc = bicgstab<K, NRHS, RANK1, float, float>(ctx, P, op32, E32.v, R32.v, P->kw32, inner_tol,
-                                                maxit - used, &inner, st, prof, retries,
-                                                RANK1 ? P->amg : nullptr, true, resume);
+    if (RANK1 && P->ps && !prof)
+      rc = resident_solve<float>(ctx, P, E32.v[0], R32.v[0], inner_tol, maxit - used, &inner, st,
+                                 retries, true);
+    else
+      rc = bicgstab<K, NRHS, RANK1, float, float>(ctx, P, op32, E32.v, R32.v, P->kw32, inner_tol,
+                                                  maxit - used, &inner, st, prof, retries,
+                                                  RANK1 ? P->amg : nullptr, true, resume);
     if (rc) return rc;
     resumable = inner.resumable;
     used += inner.iters > 0 ? inner.iters : 1;
@@ -2890,13 +2955,21 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
                              "flags");
     if (rc) return rc;
   }
+  // the direct solve of a small pressure system stands in for the Krylov one,
+  // except where the launches of that one are profiled or its iterations
+  // capped below a single cycle
+  const bool direct = P->ds && !f.profile && f.max_iter >= kRestartLen;
+  if (f.precond && !direct) {
+    const int rc = need_precond(ctx, P, f, st);
+    if (rc) return rc;
+  }
   KOp<double, double> H64{f.vv_idx, P->Hw, f.ld_v, f.N, k, 1, nullptr};
   KOp<double, double> L64{P->Lidx, P->Lw, f.ld_p, f.M, P->kL, 0, P->es, nullptr, P->a1};
   KOp<float, float> H32{f.vv_idx, P->Hw32, f.ld_v, f.N, k, 1, nullptr, nullptr};
   KOp<float, float> L32{P->Lidx, P->Lw32, f.ld_p, f.M, P->kL, 0, P->es32, nullptr, P->a1_32};
   L32.diff = P->a1_32 ? 1 : 0;
   const bool proj = P->proj != 0;
-  if (f.precond && !proj) (MIX ? L32.tiles : L64.tiles) = P->Lt;
+  if (MIX && f.precond && !proj) L32.tiles = P->Lt;
   (MIX ? H32.tiles : H64.tiles) = P->Ht;
   // open flows: one viscous operator per component on the shared index array
   KOp<double, double> Hu64{P->Hidx, P->Hw, f.ld_v, f.N, k, 1, nullptr};
@@ -3030,16 +3103,34 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     const double* pbv[1] = {P->pb};
     SolveResult pr;
     const bool prof = f.profile != 0;
-    if (proj) {  // the composed operator's rows are read directly (runtime width)
+    if (direct) {
+      PSolveResult dr;
+      rc = dsolve_run(ctx, P->ds, P->px, P->pb, f.tol, &dr, &P->launches, st);
+      if (rc) return rc;
+      pr.iters = dr.iters;
+      pr.status = dr.status;
+      pr.relres = dr.relres;
+      pr.converged = dr.converged;
+      sweeps = dr.iters;
+      // refinement at its rounding level above the tolerance: Krylov from here
+      if (!pr.converged && pr.status != 2) rc = need_precond(ctx, P, f, st);
+      if (rc) return rc;
+    }
+    if (direct && (pr.converged || pr.status == 2)) {
+    } else if (proj) {  // the composed operator's rows are read directly (runtime width)
       if (MIX)
         rc = refine<0, 1, true>(ctx, P, L64, L32, px, pbv, f.tol, f.inner_tol, f.max_iter, &pr,
                                 &sweeps, st, prof);
+      else if (P->ps && !prof)
+        rc = resident_solve<double>(ctx, P, P->px, P->pb, f.tol, f.max_iter, &pr, st);
       else
         rc = bicgstab<0, 1, true, double, double>(ctx, P, L64, px, pbv, P->kw64, f.tol,
                                                   f.max_iter, &pr, st, prof, 0, P->amg);
     } else if (MIX) {
       rc = refine<K, 1, true>(ctx, P, L64, L32, px, pbv, f.tol, f.inner_tol, f.max_iter, &pr,
                               &sweeps, st, prof);
+    } else if (P->ps && !prof) {
+      rc = resident_solve<double>(ctx, P, P->px, P->pb, f.tol, f.max_iter, &pr, st);
     } else {
       rc = bicgstab<K, 1, true, double, double>(ctx, P, L64, px, pbv, P->kw64, f.tol, f.max_iter,
                                                 &pr, st, prof, 0, P->amg);
