@@ -4,11 +4,14 @@
 // step and differ in their Reynolds number and wall data.  All vectors are
 // member-contiguous: entry (i, e) of a field lives at [i * E + e] (the
 // viscous work vectors hold u and v of every member, C = 2E columns, at
-// [i * C + c]).  A thread owns one (row, column) pair and keeps its column
-// under grid striding (the stride is a multiple of 256 and C divides 256), so
-// every stencil weight and index is read once per row and broadcast to the
-// row's columns, and every gather of a neighbour's values is one contiguous
-// run of C entries: the operator stream is shared by all members.
+// [i * C + c]).  A thread of the solve kernels owns four consecutive columns
+// of a row (V = 4; V = 1 where a solve has fewer than four columns) and keeps
+// its columns under grid striding (C / V divides 256), so every stencil
+// weight and index is read once per row and broadcast to the row's columns,
+// and every gather of a neighbour's values is one contiguous run of C entries:
+// the operator stream is shared by all members.  With one column per thread
+// the products were bound by load instructions, 84 per row and 32 columns;
+// with four, 16 B loads bring that to 84 per row and 128.
 //
 // The step follows the MIXED design of step.cu: explicit stages with FP32
 // weights gathering split (hi, lo) FP32 copies of the FP64 fields (reading R9),
@@ -18,6 +21,7 @@
 // preconditioned by a batched V-cycle on the multigrid hierarchy of step.cu
 // (amg.cuh), with the same rank-one completion of the constant mode per
 // column.  Per-column reductions are summed in a fixed order.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -48,65 +52,121 @@ struct EScal {
   int iters, maxit, done, C;
 };
 
+// Blocks of a grid are summed in kRG groups first (see col_reduce).
+constexpr int kRG = 16;
+
 struct EReduce {
-  double* partials;  // [grid][kRV][C]
-  unsigned int* counter;
+  double* partials;       // [grid][kRV][C]
+  double* groups;         // [kRG][kRV][C]
+  unsigned int* counter;  // [kRG + 1], zero between launches
 };
 
-// Per-column reduction of NV values (column = thread index mod C, fixed under
-// the loops; thread t is in group g = t / C of the kT / C groups).  In a block,
-// the groups are summed by a fixed tree into group 0, which stores the block
-// partials; the last block then has every thread sum the partials of blocks
-// g, g + G, ... for its column in block order, reduces the groups by the same
-// tree and runs fin(column, totals) for every column.  The order of every sum
-// is fixed, so the result does not depend on timing.
-template <int NV, typename Fin>
-__device__ __forceinline__ void col_reduce(double (&v)[NV], int C, EReduce rd, Fin fin) {
-  __shared__ double sh[NV][kT];
+// V consecutive columns of one row
+template <int V>
+struct alignas(4 * V) Fv {
+  float a[V];
+};
+template <int V>
+__device__ __forceinline__ Fv<V> ldv(const float* p) {
+  return *reinterpret_cast<const Fv<V>*>(p);
+}
+template <int V>
+__device__ __forceinline__ void stv(float* p, const Fv<V>& x) {
+  *reinterpret_cast<Fv<V>*>(p) = x;
+}
+
+// (double)x with integer instructions: the FP64 pipe, which converts at the
+// rate of its additions (2 lanes a cycle and SM), is what bounds the
+// reductions.  Exact; zeros, subnormals, infinities and NaN take the
+// conversion instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (double)x;
+  return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)),
+                          (int)(b << 29));
+}
+
+// Per-column reduction of NV values of each of a thread's V columns (columns
+// V (t mod C/V) ..., fixed under the loops; thread t is in row group
+// t / (C / V) of the block).  In a block, the groups are summed by a fixed
+// tree into group 0, which stores the block partials.  The blocks of a grid
+// form kRG groups: the last block of a group adds its group's partials, the
+// last group's adder adds the groups and runs fin(column, totals) for every
+// column.  The order of every sum is fixed, so the result does not depend on
+// timing.  One block adding all partials would issue grid x C x NV FP64 adds
+// alone on one SM's pipe (19 us for 608 blocks, 64 columns and two values, in
+// each of the five reductions of an iteration); in two steps it is 1.7 us.
+template <int NV, int V, typename Fin>
+__device__ __forceinline__ void col_reduce(double (&v)[NV][V], int C, EReduce rd, Fin fin) {
+  __shared__ double sh[NV * V * kT];
   __shared__ bool last;
-  const int t = threadIdx.x, G = kT / C, g = t / C;
-  auto tree = [&]() {  // sh[j][c] = sum over the groups of sh[j][g C + c]
-    for (int h = G / 2; h >= 1; h /= 2) {
-      if (g < h) {
+  const int t = threadIdx.x, CG = C / V, G = kT / CG, cg = t % CG, g = t / CG;
+  // sh[(j * V + u) * kT + t]: value j of column V cg + u, group g
 #pragma unroll
-        for (int j = 0; j < NV; ++j) sh[j][t] += sh[j][t + h * C];
+  for (int j = 0; j < NV; ++j)
+#pragma unroll
+    for (int u = 0; u < V; ++u) sh[(j * V + u) * kT + t] = v[j][u];
+  __syncthreads();
+  for (int h = G / 2; h >= 1; h /= 2) {
+    if (g < h) {
+#pragma unroll
+      for (int j = 0; j < NV * V; ++j) sh[j * kT + t] += sh[j * kT + t + h * CG];
+    }
+    __syncthreads();
+  }
+  if (g == 0) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+#pragma unroll
+      for (int u = 0; u < V; ++u)
+        rd.partials[((size_t)blockIdx.x * kRV + j) * C + cg * V + u] = sh[(j * V + u) * kT + t];
+  }
+  const int gs = ((int)gridDim.x + kRG - 1) / kRG;  // blocks per group
+  const int grp = blockIdx.x / gs, ngrp = ((int)gridDim.x + gs - 1) / gs;
+  const int b0 = grp * gs, b1 = min((int)gridDim.x, b0 + gs);
+  auto arrive = [&](unsigned int* cnt, int of) {  // true in the last of `of` blocks to come here
+    __syncthreads();
+    if (t == 0) {
+      __threadfence();
+      last = atomicAdd(cnt, 1u) == (unsigned int)of - 1u;
+      if (last) *cnt = 0u;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+  };
+  // sum of rows [p0, p1) of src ([row][kRV][C]) per column, in sh[j * kT + column]
+  const int c = t % C, G1 = kT / C, g1 = t / C;
+  auto add_rows = [&](const double* src, int p0, int p1) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      double a = 0.0;
+      for (int b = p0 + g1; b < p1; b += G1) a += ((volatile const double*)src)[((size_t)b * kRV + j) * C + c];
+      sh[j * kT + t] = a;
+    }
+    __syncthreads();
+    for (int h = G1 / 2; h >= 1; h /= 2) {
+      if (g1 < h) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) sh[j * kT + t] += sh[j * kT + t + h * C];
       }
       __syncthreads();
     }
   };
-#pragma unroll
-  for (int j = 0; j < NV; ++j) sh[j][t] = v[j];
-  __syncthreads();
-  tree();
+  if (!arrive(rd.counter + 1 + grp, b1 - b0)) return;
+  add_rows(rd.partials, b0, b1);
   if (t < C) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) rd.partials[((size_t)blockIdx.x * kRV + j) * C + t] = sh[j][t];
+    for (int j = 0; j < NV; ++j) rd.groups[((size_t)grp * kRV + j) * C + t] = sh[j * kT + t];
   }
-  __syncthreads();
-  if (t == 0) {
-    __threadfence();
-    last = atomicAdd(rd.counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  const int c = t % C;
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    double a = 0.0;
-    for (int b = g; b < (int)gridDim.x; b += G)
-      a += ((volatile double*)rd.partials)[((size_t)b * kRV + j) * C + c];
-    sh[j][t] = a;
-  }
-  __syncthreads();
-  tree();
+  if (!arrive(rd.counter, ngrp)) return;
+  add_rows(rd.groups, 0, ngrp);
   if (t < C) {
     double tot[NV];
 #pragma unroll
-    for (int j = 0; j < NV; ++j) tot[j] = sh[j][t];
+    for (int j = 0; j < NV; ++j) tot[j] = sh[j * kT + t];
     fin(t, tot);
   }
-  if (t == 0) *rd.counter = 0u;
 }
 
 // Items f = i C + c (row i, column c) of a contiguous share of the rows per
@@ -134,6 +194,25 @@ __device__ __forceinline__ void col_reduce(double (&v)[NV], int C, EReduce rd, F
   const int64_t es_sub = (es_share + es_groups - 1) / es_groups;                         \
   const int ef_c = (int)threadIdx.x % (C);                                               \
   const int64_t es_a = min(es_r1, es_r0 + es_sub * ((int)threadIdx.x / (C)));             \
+  const int64_t es_b = min(es_r1, es_a + es_sub);                                        \
+  for (int64_t I = es_a, f = es_a * (C) + ef_c; I < es_b; ++I, f += (C))
+
+// The two orders with V columns per thread, the first of them ef_c.
+#define EFORV(n, C, I)                                                                    \
+  const int64_t ef_share = ((int64_t)(n) + gridDim.x - 1) / gridDim.x;                   \
+  const int64_t ef_r1 = min((int64_t)(n), ef_share * (blockIdx.x + 1));                  \
+  const int ef_cg = (C) / V, ef_c = V * ((int)threadIdx.x % ef_cg), ef_step = kT / ef_cg; \
+  for (int64_t I = min((int64_t)(n), ef_share * blockIdx.x) + (int)threadIdx.x / ef_cg,   \
+               f = I * (C) + ef_c;                                                       \
+       I < ef_r1; I += ef_step, f += (int64_t)ef_step * (C))
+#define EFORV_SEQ(n, C, I)                                                                \
+  const int64_t es_share = ((int64_t)(n) + gridDim.x - 1) / gridDim.x;                   \
+  const int64_t es_r0 = min((int64_t)(n), es_share * blockIdx.x);                        \
+  const int64_t es_r1 = min((int64_t)(n), es_share * (blockIdx.x + 1));                  \
+  const int ef_cg = (C) / V, ef_c = V * ((int)threadIdx.x % ef_cg);                       \
+  const int es_groups = kT / ef_cg;                                                       \
+  const int64_t es_sub = (es_share + es_groups - 1) / es_groups;                         \
+  const int64_t es_a = min(es_r1, es_r0 + es_sub * ((int)threadIdx.x / ef_cg));           \
   const int64_t es_b = min(es_r1, es_a + es_sub);                                        \
   for (int64_t I = es_a, f = es_a * (C) + ef_c; I < es_b; ++I, f += (C))
 
@@ -324,9 +403,9 @@ __global__ void e_split(int64_t n, const double* __restrict__ x, float2* __restr
 // per-column sum of x (n rows, C columns) into out[c] / n (the mean)
 __global__ void __launch_bounds__(kT)
     e_colmean(int64_t n, int C, const double* __restrict__ x, EReduce rd, double* out) {
-  double v[1] = {0.0};
-  EFOR(n, C, row) v[0] += x[f];
-  col_reduce<1>(v, C, rd, [&](int c, double* t) { out[c] = t[0] / (double)n; });
+  double v[1][1] = {{0.0}};
+  EFOR(n, C, row) v[0][0] += x[f];
+  col_reduce<1, 1>(v, C, rd, [&](int c, double* t) { out[c] = t[0] / (double)n; });
 }
 
 // ---------------------------------------------------------- batched operators
@@ -342,33 +421,56 @@ struct EOp {
   const float* a1;      // pressure: row sums
 };
 
-template <int K>
-__device__ __forceinline__ float erow32(const EOp& op, const float* w, int64_t i, const float* x,
-                                      int C, int c) {
-  float acc = 0.f;
+// sum_s w_s x_j over row i for the thread's V columns, seven gathers in flight
+// per batch (28 registers of operands; all 28 at once left 2 blocks per SM)
+template <int K, int V>
+__device__ __forceinline__ Fv<V> erow32(const EOp& op, const float* w, int64_t i, const float* x,
+                                        int C, int c) {
+  Fv<V> acc{};
   const int kk = K > 0 ? K : op.k;
-#pragma unroll(K > 0 ? K : 1)
-  for (int s = 0; s < kk; ++s) acc += w[s * op.ld + i] * x[(int64_t)op.idx[s * op.ld + i] * C + c];
+#pragma unroll(K > 0 ? 7 : 1)
+  for (int s = 0; s < kk; ++s) {
+    const float ws = w[s * op.ld + i];
+    const Fv<V> xj = ldv<V>(x + (int64_t)op.idx[s * op.ld + i] * C + c);
+#pragma unroll
+    for (int u = 0; u < V; ++u) acc.a[u] += ws * xj.a[u];
+  }
   return acc;
 }
 
 // ---------------------------------------------------------- batched BiCGSTAB
+// A thread works while any of its columns is active.  What it writes for a
+// column that has ended is never read again, except x, which it leaves alone.
+template <int V>
+__device__ __forceinline__ bool any_active(const EScal* sc, int c0, bool (&act)[V]) {
+  bool any = false;
+#pragma unroll
+  for (int u = 0; u < V; ++u) any |= act[u] = sc->active[c0 + u] != 0;
+  return any;
+}
+
 // r = b (x0 = 0); rh = r; p = r; rho = (rh, r); rr; bb; (c . p) for the pressure
+template <int V>
 __global__ void __launch_bounds__(kT)
     e_init(int64_t n, int C, const float* __restrict__ b, float* __restrict__ r,
            float* __restrict__ rh, float* __restrict__ p, float* __restrict__ x,
            const float* __restrict__ cnode, EScal* sc, EReduce rd, double tol2, int maxit) {
-  double v[3] = {0.0, 0.0, 0.0};
-  EFOR(n, C, i) {
-    const float bi = b[f];
-    r[f] = bi;
-    rh[f] = bi;
-    p[f] = bi;
-    x[f] = 0.f;
-    v[0] += (double)bi * bi;
-    v[1] += cnode ? (double)cnode[i] * bi : 0.0;
+  double v[2][V] = {};
+  EFORV(n, C, i) {
+    const Fv<V> bi = ldv<V>(b + f);
+    stv<V>(r + f, bi);
+    stv<V>(rh + f, bi);
+    stv<V>(p + f, bi);
+    stv<V>(x + f, Fv<V>{});
+    const double cn = cnode ? widen(cnode[i]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const double d = widen(bi.a[u]);
+      v[0][u] += d * d;
+      if (cnode) v[1][u] += cn * d;
+    }
   }
-  col_reduce<3>(v, C, rd, [&](int c, double* t) {
+  col_reduce<2, V>(v, C, rd, [&](int c, double* t) {
     sc->rr[c] = t[0];
     sc->bb[c] = t[0];
     sc->rho[c] = t[0];
@@ -387,99 +489,104 @@ __global__ void __launch_bounds__(kT)
   });
 }
 
-// v = A zp (+ rank-one terms); reduce (rh, v) -> alpha
-template <int K>
+// One product of the batched method: y = A z (+ rank-one terms).  WHICH = 0:
+// v = A p^, reduce (rh, v) -> alpha (dot = rh).  WHICH = 1: t = A s^, reduce
+// (t, s), (t, t) -> omega (dot = s).
+template <int K, int V, int WHICH>
 __global__ void __launch_bounds__(kT)
-    e_spmv_v(EOp op, const float* __restrict__ w, const float* __restrict__ zp,
-             float* __restrict__ v, const float* __restrict__ rh, EScal* sc, EReduce rd) {
+    e_spmv(EOp op, const float* __restrict__ w, const float* __restrict__ z,
+           float* __restrict__ y, const float* __restrict__ dot, EScal* sc, EReduce rd) {
   if (sc->done) return;
   const int C = sc->C;
-  // this thread's column is fixed: its scalars are read once
-  const int c0 = (int)threadIdx.x % C;
-  const bool act = sc->active[c0] != 0;
-  const float ac = op.visc ? op.a[c0] : 0.f;
-  const float kap = op.visc ? 0.f : (float)sc->kap[0][c0];
-  const float sig = op.visc ? 0.f : (float)sc->sum_p[c0];
-  double acc[1] = {0.0};
-  if (act) {
-    EFOR_SEQ(op.n, C, i) {
-      float y = erow32<K>(op, w, i, zp, C, ef_c);
-      if (op.visc)
-        y = zp[f] - ac * y;
-      else
-        y += kap * op.a1[i] + op.es[i] * sig;
-      v[f] = y;
-      acc[0] += (double)rh[f] * y;
+  // this thread's columns are fixed: their scalars are read once
+  const int c0 = V * ((int)threadIdx.x % (C / V));
+  bool act[V];
+  const bool any = any_active<V>(sc, c0, act);
+  float ac[V], kap[V], sig[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+    ac[u] = op.visc ? op.a[c0 + u] : 0.f;
+    kap[u] = op.visc ? 0.f : (float)sc->kap[WHICH][c0 + u];
+    sig[u] = op.visc ? 0.f : (float)(WHICH ? sc->sum_s[c0 + u] : sc->sum_p[c0 + u]);
+  }
+  constexpr int NV = WHICH ? 2 : 1;
+  double acc[NV][V] = {};
+  if (any) {
+    EFORV_SEQ(op.n, C, i) {
+      Fv<V> yi = erow32<K, V>(op, w, i, z, C, ef_c);
+      if (op.visc) {
+        const Fv<V> zi = ldv<V>(z + f);
+#pragma unroll
+        for (int u = 0; u < V; ++u) yi.a[u] = zi.a[u] - ac[u] * yi.a[u];
+      } else {
+        const float a1 = op.a1[i], es = op.es[i];
+#pragma unroll
+        for (int u = 0; u < V; ++u) yi.a[u] += kap[u] * a1 + es * sig[u];
+      }
+      stv<V>(y + f, yi);
+      const Fv<V> di = ldv<V>(dot + f);
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const double yd = widen(yi.a[u]);
+        acc[0][u] += widen(di.a[u]) * yd;
+        if (WHICH) acc[NV - 1][u] += yd * yd;
+      }
     }
   }
-  col_reduce<1>(acc, C, rd, [&](int c, double* t) {
+  col_reduce<NV, V>(acc, C, rd, [&](int c, double* t) {
     if (!sc->active[c]) return;
-    if (t[0] == 0.0 || !isfinite(t[0])) {
-      sc->active[c] = 0;
-      sc->status[c] = isfinite(t[0]) ? 1 : 2;
-      return;
+    if (WHICH == 0) {
+      if (t[0] == 0.0 || !isfinite(t[0])) {
+        sc->active[c] = 0;
+        sc->status[c] = isfinite(t[0]) ? 1 : 2;
+        return;
+      }
+      sc->alpha[c] = sc->rho[c] / t[0];
+    } else {
+      const double t2 = t[NV - 1];
+      if (!(t2 > 0.0) || !isfinite(t[0])) {
+        sc->active[c] = 0;
+        sc->status[c] = isfinite(t2) ? 3 : 2;
+        return;
+      }
+      sc->omega[c] = t[0] / t2;
     }
-    sc->alpha[c] = sc->rho[c] / t[0];
   });
 }
 
 // s = r - alpha v; reduce (c . s) for the pressure
+template <int V>
 __global__ void __launch_bounds__(kT)
     e_update_s(int64_t n, const float* __restrict__ r, const float* __restrict__ v,
                float* __restrict__ s, const float* __restrict__ cnode, EScal* sc, EReduce rd) {
   if (sc->done) return;
   const int C = sc->C;
-  const int c0 = (int)threadIdx.x % C;
-  const bool act = sc->active[c0] != 0;
-  const float al = (float)sc->alpha[c0];
-  double acc[1] = {0.0};
-  if (act) {
-    EFOR(n, C, i) {
-      const float si = r[f] - al * v[f];
-      s[f] = si;
-      if (cnode) acc[0] += (double)cnode[i] * si;
+  const int c0 = V * ((int)threadIdx.x % (C / V));
+  bool act[V];
+  const bool any = any_active<V>(sc, c0, act);
+  float al[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) al[u] = (float)sc->alpha[c0 + u];
+  double acc[1][V] = {};
+  if (any) {
+    EFORV(n, C, i) {
+      Fv<V> si = ldv<V>(r + f);
+      const Fv<V> vi = ldv<V>(v + f);
+      const double cn = cnode ? widen(cnode[i]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        si.a[u] -= al[u] * vi.a[u];
+        if (cnode) acc[0][u] += cn * widen(si.a[u]);
+      }
+      stv<V>(s + f, si);
     }
   }
-  col_reduce<1>(acc, C, rd, [&](int c, double* t) { sc->cs[c] = t[0]; });
-}
-
-// t = A zs; reduce (t, s), (t, t) -> omega
-template <int K>
-__global__ void __launch_bounds__(kT)
-    e_spmv_t(EOp op, const float* __restrict__ w, const float* __restrict__ zs,
-             float* __restrict__ tv, const float* __restrict__ s, EScal* sc, EReduce rd) {
-  if (sc->done) return;
-  const int C = sc->C;
-  const int c0 = (int)threadIdx.x % C;
-  const bool act = sc->active[c0] != 0;
-  const float ac = op.visc ? op.a[c0] : 0.f;
-  const float kap = op.visc ? 0.f : (float)sc->kap[1][c0];
-  const float sig = op.visc ? 0.f : (float)sc->sum_s[c0];
-  double acc[2] = {0.0, 0.0};
-  if (act) {
-    EFOR_SEQ(op.n, C, i) {
-      float y = erow32<K>(op, w, i, zs, C, ef_c);
-      if (op.visc)
-        y = zs[f] - ac * y;
-      else
-        y += kap * op.a1[i] + op.es[i] * sig;
-      tv[f] = y;
-      acc[0] += (double)y * s[f];
-      acc[1] += (double)y * y;
-    }
-  }
-  col_reduce<2>(acc, C, rd, [&](int c, double* t) {
-    if (!sc->active[c]) return;
-    if (!(t[1] > 0.0) || !isfinite(t[0])) {
-      sc->active[c] = 0;
-      sc->status[c] = isfinite(t[1]) ? 3 : 2;
-      return;
-    }
-    sc->omega[c] = t[0] / t[1];
-  });
+  if (!cnode) return;  // viscous: nothing to reduce
+  col_reduce<1, V>(acc, C, rd, [&](int c, double* t) { sc->cs[c] = t[0]; });
 }
 
 // x += alpha zp + omega zs; r = s - omega t; reduce (rh, r), (r, r); beta
+template <int V>
 __global__ void __launch_bounds__(kT)
     e_update_xr(int64_t n, float* __restrict__ x, float* __restrict__ r,
                 const float* __restrict__ rh, const float* __restrict__ zp,
@@ -487,21 +594,37 @@ __global__ void __launch_bounds__(kT)
                 const float* __restrict__ tv, int pc, EScal* sc, EReduce rd) {
   if (sc->done) return;
   const int C = sc->C;
-  const int c0 = (int)threadIdx.x % C;
-  const bool act = sc->active[c0] != 0;
-  const float al = (float)sc->alpha[c0], om = (float)sc->omega[c0];
-  const float kp = pc ? (float)sc->kap[0][c0] : 0.f, ks = pc ? (float)sc->kap[1][c0] : 0.f;
-  double acc[2] = {0.0, 0.0};
-  if (act) {
-    EFOR(n, C, i) {
-      x[f] += al * (zp[f] + kp) + om * (zs[f] + ks);
-      const float ri = s[f] - om * tv[f];
-      r[f] = ri;
-      acc[0] += (double)rh[f] * ri;
-      acc[1] += (double)ri * ri;
+  const int c0 = V * ((int)threadIdx.x % (C / V));
+  bool act[V];
+  const bool any = any_active<V>(sc, c0, act);
+  float al[V], om[V], kp[V], ks[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+    al[u] = (float)sc->alpha[c0 + u];
+    om[u] = (float)sc->omega[c0 + u];
+    kp[u] = pc ? (float)sc->kap[0][c0 + u] : 0.f;
+    ks[u] = pc ? (float)sc->kap[1][c0 + u] : 0.f;
+  }
+  double acc[2][V] = {};
+  if (any) {
+    EFORV(n, C, i) {
+      Fv<V> xi = ldv<V>(x + f), ri = ldv<V>(s + f);
+      const Fv<V> pi = ldv<V>(zp + f), qi = ldv<V>(zs + f), ti = ldv<V>(tv + f),
+                  hi = ldv<V>(rh + f);
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const float xn = xi.a[u] + (al[u] * (pi.a[u] + kp[u]) + om[u] * (qi.a[u] + ks[u]));
+        if (act[u]) xi.a[u] = xn;
+        ri.a[u] -= om[u] * ti.a[u];
+        const double rd2 = widen(ri.a[u]);
+        acc[0][u] += widen(hi.a[u]) * rd2;
+        acc[1][u] += rd2 * rd2;
+      }
+      stv<V>(x + f, xi);
+      stv<V>(r + f, ri);
     }
   }
-  col_reduce<2>(acc, C, rd, [&](int c, double* t) {
+  col_reduce<2, V>(acc, C, rd, [&](int c, double* t) {
     if (sc->active[c]) {
       sc->rr[c] = t[1];
       const double rho_new = t[0];
@@ -523,77 +646,102 @@ __global__ void __launch_bounds__(kT)
 }
 
 // p = r + beta (p - omega v); reduce (c . p) for the pressure; done flag
+template <int V>
 __global__ void __launch_bounds__(kT)
     e_update_p(int64_t n, float* __restrict__ p, const float* __restrict__ r,
                const float* __restrict__ v, const float* __restrict__ cnode, EScal* sc,
                EReduce rd) {
   if (sc->done) return;
   const int C = sc->C;
-  const int c0 = (int)threadIdx.x % C;
-  const bool act = sc->active[c0] != 0;
-  const float be = (float)sc->alpha[c0], om = (float)sc->omega[c0];
-  double acc[1] = {0.0};
-  if (act) {
-    EFOR(n, C, i) {
-      const float pi = r[f] + be * (p[f] - om * v[f]);
-      p[f] = pi;
-      if (cnode) acc[0] += (double)cnode[i] * pi;
+  const int c0 = V * ((int)threadIdx.x % (C / V));
+  bool act[V];
+  const bool any = any_active<V>(sc, c0, act);
+  float be[V], om[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+    be[u] = (float)sc->alpha[c0 + u];
+    om[u] = (float)sc->omega[c0 + u];
+  }
+  double acc[1][V] = {};
+  if (any) {
+    EFORV(n, C, i) {
+      Fv<V> pi = ldv<V>(p + f);
+      const Fv<V> ri = ldv<V>(r + f), vi = ldv<V>(v + f);
+      const double cn = cnode ? widen(cnode[i]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        pi.a[u] = ri.a[u] + be[u] * (pi.a[u] - om[u] * vi.a[u]);
+        if (cnode) acc[0][u] += cn * widen(pi.a[u]);
+      }
+      stv<V>(p + f, pi);
     }
   }
-  col_reduce<1>(acc, C, rd, [&](int c, double* t) {
+  col_reduce<1, V>(acc, C, rd, [&](int c, double* t) {
     if (sc->active[c]) sc->cp[c] = t[0];
     if (c == sc->C - 1) {
-      int any = 0;
-      for (int q = 0; q < sc->C; ++q) any |= sc->active[q];
-      if (!any || sc->iters >= sc->maxit) sc->done = 1;
+      int any2 = 0;
+      for (int q = 0; q < sc->C; ++q) any2 |= sc->active[q];
+      if (!any2 || sc->iters >= sc->maxit) sc->done = 1;
     }
   });
 }
 
 // ------------------------------------------------------------ batched V-cycle
 // r0[p][c] = c_p v[perm0[p]][c] - mu_c ce_p,  mu_c = (c . v)_c / (c . es)
+template <int V>
 __global__ void __launch_bounds__(kT)
     e_pc_in(int64_t M, int C, const float* __restrict__ v, const float* __restrict__ cl,
             const float* __restrict__ ce, const int32_t* __restrict__ perm0, int which,
             double inv_ces, const EScal* sc, float* __restrict__ r0) {
   if (sc->done) return;
-  const int c0 = (int)threadIdx.x % C;
-  const float mu = (float)((which ? sc->cs[c0] : sc->cp[c0]) * inv_ces);
-  EFOR(M, C, p) r0[f] = cl[p] * v[(int64_t)perm0[p] * C + ef_c] - mu * ce[p];
+  const int c0 = V * ((int)threadIdx.x % (C / V));
+  float mu[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u)
+    mu[u] = (float)((which ? sc->cs[c0 + u] : sc->cp[c0 + u]) * inv_ces);
+  EFORV(M, C, p) {
+    Fv<V> vi = ldv<V>(v + (int64_t)perm0[p] * C + ef_c);
+    const float a = cl[p], b = ce[p];
+#pragma unroll
+    for (int u = 0; u < V; ++u) vi.a[u] = a * vi.a[u] - mu[u] * b;
+    stv<V>(r0 + f, vi);
+  }
 }
 
 // Pre-smoothing from zero (x = omega D^-1 r) and restriction of its residual
-// to the aggregates: thread (aggregate I, column c) takes I's rows in order.
-template <int W>
+// to the aggregates: thread (aggregate I, columns) takes I's rows in order.
+template <int W, int V>
 __global__ void __launch_bounds__(kT)
     e_pc_restrict(AmgLevel F, int64_t nagg, int C, const float* __restrict__ r,
                   float* __restrict__ x, float* __restrict__ rc, const EScal* sc) {
   if (sc->done) return;
-  EFOR_SEQ(nagg, C, I) {
+  EFORV_SEQ(nagg, C, I) {
     const int c = ef_c;
-    float acc = 0.f;
+    Fv<V> acc{};
     for (int32_t i = F.cptr[I]; i < F.cptr[I + 1]; ++i) {
-      const float ri = r[(int64_t)i * C + c];
-      const float xi = F.wd[i] * ri;
-      x[(int64_t)i * C + c] = xi;
-      float ax = F.diag[i] * xi;
-      if constexpr (W > 0) {  // every load of the row in flight at once
+      const Fv<V> ri = ldv<V>(r + (int64_t)i * C + c);
+      const float wi = F.wd[i], di = F.diag[i];
+      Fv<V> xi, ax;
 #pragma unroll
-        for (int s = 0; s < W; ++s) {
-          if (s < F.width) {
-            const int32_t j = F.idx[s * F.ld + i];
-            ax += F.val[s * F.ld + i] * (F.wd[j] * r[(int64_t)j * C + c]);
-          }
-        }
-      } else {
-        for (int s = 0; s < F.width; ++s) {
+      for (int u = 0; u < V; ++u) {
+        xi.a[u] = wi * ri.a[u];
+        ax.a[u] = di * xi.a[u];
+      }
+      stv<V>(x + (int64_t)i * C + c, xi);
+#pragma unroll(W > 0 ? W : 1)
+      for (int s = 0; s < (W > 0 ? W : F.width); ++s) {
+        if (W == 0 || s < F.width) {
           const int32_t j = F.idx[s * F.ld + i];
-          ax += F.val[s * F.ld + i] * (F.wd[j] * r[(int64_t)j * C + c]);
+          const float vs = F.val[s * F.ld + i], wj = F.wd[j];
+          const Fv<V> rj = ldv<V>(r + (int64_t)j * C + c);
+#pragma unroll
+          for (int u = 0; u < V; ++u) ax.a[u] += vs * (wj * rj.a[u]);
         }
       }
-      acc += ri - ax;
+#pragma unroll
+      for (int u = 0; u < V; ++u) acc.a[u] += ri.a[u] - ax.a[u];
     }
-    rc[f] = acc;
+    stv<V>(rc + f, acc);
   }
 }
 
@@ -674,53 +822,189 @@ __global__ void __launch_bounds__(kT)
   }
 }
 
+// The same product for four columns or more: split kCS ways along j, so that
+// its nc / TR tiles fill the chip (98 tiles of 16 rows for nc = 1,560 left a
+// third of the SMs idle and one block's latency bound: 185 us for 64 columns,
+// against 13 us).  A block takes TR rows and every column: thread t keeps
+// columns 4 (t mod C/4) .. + 3 and TR C / 1024 rows; X and r move through
+// shared memory in slabs of kCJ columns of X, the next slab's loads in
+// registers before the current one's products.  Part q of the sum over j goes
+// to zpart[q]; e_pc_prolong adds the parts.
+constexpr int kCS = 4;
+constexpr int kCRow = 36;  // stride of a staged row of X: 16 B aligned, conflict-free
+inline int coarse_rows(int C) { return std::max(32, 1024 / C); }  // TR
+
+template <int RP>  // rows per thread, TR C / 1024: 2 for C = 64, else 1
+__global__ void __launch_bounds__(kT)
+    e_pc_coarse4(int64_t nc, int C, int TR, const float* __restrict__ X,
+                 const float* __restrict__ r, float* __restrict__ zpart, const EScal* sc) {
+  if (sc->done) return;
+  extern __shared__ __align__(16) float csm[];
+  float* xs = csm;               // [TR][kCRow]
+  float* rs = csm + TR * kCRow;  // [kCJ][C]
+  const int t = threadIdx.x, CG = C / 4, cg = t % CG, rt = t / CG;
+  const int64_t row0 = (int64_t)blockIdx.x * TR;
+  const int64_t share = (nc + kCS * kCJ - 1) / (kCS * kCJ) * kCJ;
+  const int64_t j_a = min(nc, share * blockIdx.y), j_b = min(nc, j_a + share);
+  const int nx = TR * kCJ / kT;      // X values a thread moves per slab (4 to 32)
+  const int nr = (kCJ * CG + kT - 1) / kT;  // and 4-column groups of r (1 or 2)
+  float4 acc[RP];
+#pragma unroll
+  for (int q = 0; q < RP; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float px[8];
+  float4 pr[2];
+  auto load = [&](int64_t j0) {  // the first 8 X values; more rows than 64 load theirs in store
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int e = t + k * kT, rr = e / kCJ, jj = e % kCJ;
+      px[k] = (k < nx && row0 + rr < nc && j0 + jj < j_b) ? X[(row0 + rr) * nc + j0 + jj] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int e = t + k * kT, jj = e / CG;
+      pr[k] = (k < nr && jj < kCJ && j0 + jj < j_b)
+                  ? reinterpret_cast<const float4*>(r + (j0 + jj) * C)[e % CG]
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  auto store = [&](int64_t j0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int e = t + k * kT;
+      if (k < nx) xs[(e / kCJ) * kCRow + e % kCJ] = px[k];
+    }
+    for (int k = 8; k < nx; ++k) {
+      const int e = t + k * kT, rr = e / kCJ, jj = e % kCJ;
+      xs[rr * kCRow + jj] =
+          (row0 + rr < nc && j0 + jj < j_b) ? X[(row0 + rr) * nc + j0 + jj] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int e = t + k * kT;
+      if (k < nr && e < kCJ * CG) reinterpret_cast<float4*>(rs)[e] = pr[k];
+    }
+  };
+  if (j_a < j_b) load(j_a);
+  const int RT = kT / CG;  // row threads
+  for (int64_t j0 = j_a; j0 < j_b; j0 += kCJ) {
+    store(j0);
+    __syncthreads();
+    if (j0 + kCJ < j_b) load(j0 + kCJ);
+#pragma unroll
+    for (int jj = 0; jj < kCJ; jj += 4) {  // slabs are padded with zeros
+      float4 rv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) rv[k] = reinterpret_cast<const float4*>(rs)[(jj + k) * CG + cg];
+#pragma unroll
+      for (int q = 0; q < RP; ++q) {
+        const float4 x4 = *reinterpret_cast<const float4*>(xs + (rt + q * RT) * kCRow + jj);
+        const float xk[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          acc[q].x += xk[k] * rv[k].x;
+          acc[q].y += xk[k] * rv[k].y;
+          acc[q].z += xk[k] * rv[k].z;
+          acc[q].w += xk[k] * rv[k].w;
+        }
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < RP; ++q) {
+    const int64_t row = row0 + rt + q * RT;
+    if (row < nc)
+      reinterpret_cast<float4*>(zpart + ((int64_t)blockIdx.y * nc + row) * C)[cg] = acc[q];
+  }
+}
+
+// z = the sum of the parts; then the correction of the finer level's rows of
+// each aggregate (has_fine), or z itself
+__global__ void __launch_bounds__(kT)
+    e_pc_prolong(int64_t nc, int C, const float* __restrict__ zpart, float* __restrict__ z,
+                 AmgLevel Fine, float* __restrict__ xfine, int has_fine, const EScal* sc) {
+  if (sc->done) return;
+  constexpr int V = 4;
+  EFORV(nc, C, row) {
+    Fv<V> a = ldv<V>(zpart + f);
+#pragma unroll
+    for (int q = 1; q < kCS; ++q) {
+      const Fv<V> b = ldv<V>(zpart + (int64_t)q * nc * C + f);
+#pragma unroll
+      for (int u = 0; u < V; ++u) a.a[u] += b.a[u];
+    }
+    if (!has_fine) {
+      stv<V>(z + f, a);
+      continue;
+    }
+    for (int32_t i = Fine.cptr[row]; i < Fine.cptr[row + 1]; ++i) {
+      Fv<V> x = ldv<V>(xfine + (int64_t)i * C + ef_c);
+#pragma unroll
+      for (int u = 0; u < V; ++u) x.a[u] += kAmgCoarseScale * a.a[u];
+      stv<V>(xfine + (int64_t)i * C + ef_c, x);
+    }
+  }
+}
+
+// B v = z + kap with kap = (mu - sum(z)) / M, per column
+__device__ __forceinline__ void e_finish(EScal* sc, int which, int c, double zsum, double inv_ces,
+                                         double inv_R) {
+  const double mu = (which ? sc->cs[c] : sc->cp[c]) * inv_ces;
+  sc->kap[which][c] = (mu - zsum) * inv_R;
+  if (which)
+    sc->sum_s[c] = mu;
+  else
+    sc->sum_p[c] = mu;
+}
+
 // Post-smoothing z = x + omega D^-1 (r - G x) on a level whose x holds the
 // coarse correction; above level 0 it corrects the finer level's rows of each
 // aggregate (x_fine += scale z), on level 0 it writes z in P-node order and
 // reduces its per-column sum (for B v = z - mean(z) + mu / M)
-template <int W>
+template <int W, int V, bool LEVEL0>
 __global__ void __launch_bounds__(kT)
     e_pc_up(AmgLevel F, int C, const float* __restrict__ r, const float* __restrict__ x,
-            AmgLevel Fine, float* __restrict__ xfine, int level0,
-            const int32_t* __restrict__ perm0, float* __restrict__ zout, int which,
-            double inv_ces, double inv_R, EScal* sc, EReduce rd) {
+            AmgLevel Fine, float* __restrict__ xfine, const int32_t* __restrict__ perm0,
+            float* __restrict__ zout, int which, double inv_ces, double inv_R, EScal* sc,
+            EReduce rd) {
   if (sc->done) return;
-  double acc[1] = {0.0};
-  EFOR_SEQ(F.n, C, i) {
+  double acc[1][V] = {};
+  EFORV_SEQ(F.n, C, i) {
     const int c = ef_c;
-    const float xi = x[f];
-    float ax = F.diag[i] * xi;
-    if constexpr (W > 0) {
+    const Fv<V> xi = ldv<V>(x + f), ri = ldv<V>(r + f);
+    const float di = F.diag[i], wi = F.wd[i];
+    Fv<V> ax;
 #pragma unroll
-      for (int s = 0; s < W; ++s) {
-        if (s < F.width) {
-          const int32_t j = F.idx[s * F.ld + i];
-          ax += F.val[s * F.ld + i] * x[(int64_t)j * C + c];
-        }
-      }
-    } else {
-      for (int s = 0; s < F.width; ++s) {
+    for (int u = 0; u < V; ++u) ax.a[u] = di * xi.a[u];
+#pragma unroll(W > 0 ? W : 1)
+    for (int s = 0; s < (W > 0 ? W : F.width); ++s) {
+      if (W == 0 || s < F.width) {
         const int32_t j = F.idx[s * F.ld + i];
-        ax += F.val[s * F.ld + i] * x[(int64_t)j * C + c];
+        const float vs = F.val[s * F.ld + i];
+        const Fv<V> xj = ldv<V>(x + (int64_t)j * C + c);
+#pragma unroll
+        for (int u = 0; u < V; ++u) ax.a[u] += vs * xj.a[u];
       }
     }
-    const float zi = xi + F.wd[i] * (r[f] - ax);
-    if (level0) {
-      zout[(int64_t)perm0[i] * C + c] = zi;
-      acc[0] += zi;
+    Fv<V> zi;
+#pragma unroll
+    for (int u = 0; u < V; ++u) zi.a[u] = xi.a[u] + wi * (ri.a[u] - ax.a[u]);
+    if (LEVEL0) {
+      stv<V>(zout + (int64_t)perm0[i] * C + c, zi);
+#pragma unroll
+      for (int u = 0; u < V; ++u) acc[0][u] += widen(zi.a[u]);
     } else {
-      const float v = kAmgCoarseScale * zi;
-      for (int32_t q = Fine.cptr[i]; q < Fine.cptr[i + 1]; ++q) xfine[(int64_t)q * C + c] += v;
+      for (int32_t q = Fine.cptr[i]; q < Fine.cptr[i + 1]; ++q) {
+        Fv<V> y = ldv<V>(xfine + (int64_t)q * C + c);
+#pragma unroll
+        for (int u = 0; u < V; ++u) y.a[u] += kAmgCoarseScale * zi.a[u];
+        stv<V>(xfine + (int64_t)q * C + c, y);
+      }
     }
   }
-  if (!level0) return;
-  col_reduce<1>(acc, C, rd, [&](int c, double* t) {
-    const double mu = (which ? sc->cs[c] : sc->cp[c]) * inv_ces;
-    sc->kap[which][c] = (mu - t[0]) * inv_R;
-    if (which)
-      sc->sum_s[c] = mu;
-    else
-      sc->sum_p[c] = mu;
+  if (!LEVEL0) return;
+  col_reduce<1, V>(acc, C, rd, [&](int c, double* t) {
+    e_finish(sc, which, c, t[0], inv_ces, inv_R);
   });
 }
 
@@ -731,19 +1015,14 @@ __global__ void __launch_bounds__(kT)
              float* __restrict__ zout, int which, double inv_ces, double inv_R, EScal* sc,
              EReduce rd) {
   if (sc->done) return;
-  double acc[1] = {0.0};
+  double acc[1][1] = {{0.0}};
   EFOR(M, C, q) {
     const int c = ef_c;
     zout[(int64_t)perm0[q] * C + c] = z0[f];
-    acc[0] += z0[f];
+    acc[0][0] += z0[f];
   }
-  col_reduce<1>(acc, C, rd, [&](int c, double* t) {
-    const double mu = (which ? sc->cs[c] : sc->cp[c]) * inv_ces;
-    sc->kap[which][c] = (mu - t[0]) * inv_R;
-    if (which)
-      sc->sum_s[c] = mu;
-    else
-      sc->sum_p[c] = mu;
+  col_reduce<1, 1>(acc, C, rd, [&](int c, double* t) {
+    e_finish(sc, which, c, t[0], inv_ces, inv_R);
   });
 }
 
@@ -755,7 +1034,7 @@ __global__ void __launch_bounds__(kT)
                  const double* __restrict__ esd, const double* __restrict__ x,
                  const double* __restrict__ b, double* __restrict__ r,
                  const double* __restrict__ xsum, int C, EReduce rd, double* out) {
-  double acc[2] = {0.0, 0.0};
+  double acc[2][1] = {{0.0}, {0.0}};
   EFOR_SEQ(op.n, C, i) {
     const int c = ef_c;
     double y = 0.0;
@@ -768,10 +1047,10 @@ __global__ void __launch_bounds__(kT)
       y += esd[i] * xsum[c];
     const double ri = b[f] - y;
     r[f] = ri;
-    acc[0] += ri * ri;
-    acc[1] += b[f] * b[f];
+    acc[0][0] += ri * ri;
+    acc[1][0] += b[f] * b[f];
   }
-  col_reduce<2>(acc, C, rd, [&](int c, double* t) {
+  col_reduce<2, 1>(acc, C, rd, [&](int c, double* t) {
     out[2 * c] = t[0];
     out[2 * c + 1] = t[1];
   });
@@ -780,9 +1059,9 @@ __global__ void __launch_bounds__(kT)
 // per-column sum of x (the rank-one term of the scaled pressure operator)
 __global__ void __launch_bounds__(kT)
     e_colsum(int64_t n, int C, const double* __restrict__ x, EReduce rd, double* out) {
-  double v[1] = {0.0};
-  EFOR(n, C, row) v[0] += x[f];
-  col_reduce<1>(v, C, rd, [&](int c, double* t) { out[c] = t[0]; });
+  double v[1][1] = {{0.0}};
+  EFOR(n, C, row) v[0][0] += x[f];
+  col_reduce<1, 1>(v, C, rd, [&](int c, double* t) { out[c] = t[0]; });
 }
 
 __global__ void e_to32(int64_t n, int C, const double* __restrict__ r, const double* __restrict__ sc,
@@ -835,6 +1114,7 @@ struct EnsPlan {
   float *aV32 = nullptr;
   float* kw[9] = {};  // x r rh p v s t zp zs (FP32, C columns)
   float *r32 = nullptr;
+  float* zpart = nullptr;  // [kCS][nc][E] parts of the coarse product
   // batched V-cycle work per level (r, x) and the coarse r, z
   float* lr[kAmgMaxLevels + 1] = {};
   float* lx[kAmgMaxLevels + 1] = {};
@@ -880,17 +1160,40 @@ int ealloc(rbffd_ctx* ctx, EnsPlan* p, T** out, size_t count) {
       kern<0><<<grid, kT, 0, st>>>(__VA_ARGS__);                 \
   } while (0)
 
-// kern<8> / kern<16> for graph rows of at most that width (slots unrolled
-// and predicated), kern<0> (plain loop) for wider ones
-#define EW(kern, width, ...)                                     \
+// kern<V> with the columns per thread of a solve with C columns
+#define EV(kern, grid, C, ...)                                   \
+  do {                                                           \
+    if ((C) % 4 == 0)                                            \
+      kern<4><<<grid, kT, 0, st>>>(__VA_ARGS__);                 \
+    else                                                         \
+      kern<1><<<grid, kT, 0, st>>>(__VA_ARGS__);                 \
+  } while (0)
+// the batched product for stencil size k and C columns
+#define ESPMV(which, grid, C, ...)                               \
+  do {                                                           \
+    if ((C) % 4 == 0) {                                          \
+      if (k == 28)                                               \
+        e_spmv<28, 4, which><<<grid, kT, 0, st>>>(__VA_ARGS__);  \
+      else                                                       \
+        e_spmv<0, 4, which><<<grid, kT, 0, st>>>(__VA_ARGS__);   \
+    } else if (k == 28) {                                        \
+      e_spmv<28, 1, which><<<grid, kT, 0, st>>>(__VA_ARGS__);    \
+    } else {                                                     \
+      e_spmv<0, 1, which><<<grid, kT, 0, st>>>(__VA_ARGS__);     \
+    }                                                            \
+  } while (0)
+// kern<8, V, ...> / kern<16, V, ...> for graph rows of at most that width
+// (slots unrolled and predicated), kern<0, V, ...> (plain loop) for wider ones
+#define EWV(kern, V, width, tail, ...)                           \
   do {                                                           \
     if ((width) <= 8)                                            \
-      kern<8><<<G, kT, 0, st>>>(__VA_ARGS__);                    \
+      kern<8, V tail><<<G, kT, 0, st>>>(__VA_ARGS__);            \
     else if ((width) <= 16)                                      \
-      kern<16><<<G, kT, 0, st>>>(__VA_ARGS__);                   \
+      kern<16, V tail><<<G, kT, 0, st>>>(__VA_ARGS__);           \
     else                                                         \
-      kern<0><<<G, kT, 0, st>>>(__VA_ARGS__);                    \
+      kern<0, V tail><<<G, kT, 0, st>>>(__VA_ARGS__);            \
   } while (0)
+#define ENS_COMMA ,
 
 int ens_to32(rbffd_ctx* ctx, EnsPlan* p, const double* src, int64_t n, float** dst,
              cudaStream_t st) {
@@ -1100,9 +1403,12 @@ int ens_build(rbffd_ctx* ctx, const rbffd_flow& f, int E, EnsPlan** out, cudaStr
   TRY(ealloc(ctx, p, &p->sc, 1));
   TRY(ealloc(ctx, p, &p->sc_t, 1));
   TRY(ealloc(ctx, p, &p->rd.partials, (size_t)p->grid * kRV * kCMax));
-  TRY(ealloc(ctx, p, &p->rd.counter, 1));
-  TRY(check_cuda(ctx, cudaMemsetAsync(p->rd.counter, 0, sizeof(unsigned int), st), "memset"));
+  TRY(ealloc(ctx, p, &p->rd.groups, (size_t)kRG * kRV * kCMax));
+  TRY(ealloc(ctx, p, &p->rd.counter, kRG + 1));
+  TRY(check_cuda(ctx, cudaMemsetAsync(p->rd.counter, 0, sizeof(unsigned int) * (kRG + 1), st),
+                 "memset"));
   if (const Amg* a = p->amg) {
+    TRY(ealloc(ctx, p, &p->zpart, (size_t)kCS * a->nc * E));
     // level l (0 <= l < nlev; the coarsest is lev[nlev - 1], nc rows)
     for (int l = 0; l < a->nlev; ++l) {
       TRY(ealloc(ctx, p, &p->lr[l], a->lev[l].n * E));
@@ -1122,26 +1428,53 @@ void ens_vcycle(EnsPlan* P, const float* v, int which, float* zout, cudaStream_t
   // next level's rows to their own).
   const Amg* a = P->amg;
   const int C = P->E, G = P->grid, L = a->nlev;
-  e_pc_in<<<G, kT, 0, st>>>(P->M, C, v, a->c, a->ce, a->perm0, which, a->inv_ces, P->sc,
-                            P->lr[0]);
-  for (int l = 0; l + 1 < L; ++l)
-    EW(e_pc_restrict, a->lev[l].width, a->lev[l], a->lev[l + 1].n, C, P->lr[l], P->lx[l],
-       P->lr[l + 1], P->sc);
+  EV(e_pc_in, G, C, P->M, C, v, a->c, a->ce, a->perm0, which, a->inv_ces, P->sc, P->lr[0]);
+  const bool v4 = C % 4 == 0;
+  for (int l = 0; l + 1 < L; ++l) {
+    if (v4)
+      EWV(e_pc_restrict, 4, a->lev[l].width, , a->lev[l], a->lev[l + 1].n, C, P->lr[l], P->lx[l],
+          P->lr[l + 1], P->sc);
+    else
+      EWV(e_pc_restrict, 1, a->lev[l].width, , a->lev[l], a->lev[l + 1].n, C, P->lr[l], P->lx[l],
+          P->lr[l + 1], P->sc);
+  }
   const AmgLevel none{};
   const bool fine = L >= 2;
-  const int TRc = kT / C > kCoarseRows ? kT / C : kCoarseRows;
-  const int Gc = (int)((a->nc + TRc - 1) / TRc);
-  e_pc_coarse<<<Gc, kT, 0, st>>>(a->nc, C, a->Xc, P->lr[L - 1], fine ? nullptr : P->lx[0],
-                                fine ? a->lev[L - 2] : none, fine ? P->lx[L - 2] : nullptr,
-                                fine ? 1 : 0, P->sc);
+  if (v4) {
+    const int TR = coarse_rows(C);
+    const dim3 gc((unsigned)((a->nc + TR - 1) / TR), kCS);
+    const size_t smem = sizeof(float) * ((size_t)TR * kCRow + (size_t)kCJ * C);
+    if (C == 64)
+      e_pc_coarse4<2><<<gc, kT, smem, st>>>(a->nc, C, TR, a->Xc, P->lr[L - 1], P->zpart, P->sc);
+    else
+      e_pc_coarse4<1><<<gc, kT, smem, st>>>(a->nc, C, TR, a->Xc, P->lr[L - 1], P->zpart, P->sc);
+    e_pc_prolong<<<G, kT, 0, st>>>(a->nc, C, P->zpart, P->lx[0], fine ? a->lev[L - 2] : none,
+                                   fine ? P->lx[L - 2] : nullptr, fine ? 1 : 0, P->sc);
+  } else {
+    const int TRc = kT / C > kCoarseRows ? kT / C : kCoarseRows;
+    const int Gc = (int)((a->nc + TRc - 1) / TRc);
+    e_pc_coarse<<<Gc, kT, 0, st>>>(a->nc, C, a->Xc, P->lr[L - 1], fine ? nullptr : P->lx[0],
+                                   fine ? a->lev[L - 2] : none, fine ? P->lx[L - 2] : nullptr,
+                                   fine ? 1 : 0, P->sc);
+  }
   if (!fine)  // the coarsest level is level 0: its z (in lx[0]) is the result
     e_pc_fin<<<G, kT, 0, st>>>(P->M, C, P->lx[0], a->perm0, zout, which, a->inv_ces, a->inv_R,
                                P->sc, P->rd);
-  for (int l = L - 2; l >= 0; --l)
-    EW(e_pc_up, a->lev[l].width, a->lev[l], C, P->lr[l], P->lx[l], l ? a->lev[l - 1] : none,
-       l ? P->lx[l - 1] : nullptr, l == 0 ? 1 : 0, a->perm0, zout, which, a->inv_ces,
-       a->inv_R, P->sc, P->rd);
-  P->launches += 2 + 2 * (L - 1) + (fine ? 0 : 1);
+  for (int l = L - 2; l >= 0; --l) {
+    const AmgLevel& F = a->lev[l];
+    const AmgLevel& Fine = l ? a->lev[l - 1] : none;
+    float* xf = l ? P->lx[l - 1] : nullptr;
+#define ENS_UP(V, L0)                                                                           \
+  EWV(e_pc_up, V, F.width, ENS_COMMA L0, F, C, P->lr[l], P->lx[l], Fine, xf, a->perm0, zout,     \
+      which, a->inv_ces, a->inv_R, P->sc, P->rd)
+    if (v4) {
+      if (l) ENS_UP(4, false); else ENS_UP(4, true);
+    } else {
+      if (l) ENS_UP(1, false); else ENS_UP(1, true);
+    }
+#undef ENS_UP
+  }
+  P->launches += 2 + 2 * (L - 1) + (fine ? 0 : 1) + (v4 ? 1 : 0);
 }
 
 struct ESolve {
@@ -1160,8 +1493,7 @@ int ens_bicgstab(rbffd_ctx* ctx, EnsPlan* P, const EOp& op, const float* w32, in
         *s = P->kw[5], *t = P->kw[6], *zp = P->kw[7], *zs = P->kw[8];
   const float* cnode = pc ? P->amg->cnode : nullptr;
   const int64_t n = op.n;
-  e_init<<<G, kT, 0, st>>>(n, C, P->r32, r, rh, pp, x, cnode, P->sc, P->rd,
-                           inner_tol * inner_tol, maxit);
+  EV(e_init, G, C, n, C, P->r32, r, rh, pp, x, cnode, P->sc, P->rd, inner_tol * inner_tol, maxit);
   EScal* h = (EScal*)ctx->host_pinned;
   int issued = 0;
   for (;;) {
@@ -1173,15 +1505,15 @@ int ens_bicgstab(rbffd_ctx* ctx, EnsPlan* P, const EOp& op, const float* w32, in
         ens_vcycle(P, pp, 0, zp, st);
         zpp = zp;
       }
-      EK(e_spmv_v, G, op, w32, zpp, v, rh, P->sc, P->rd);
-      e_update_s<<<G, kT, 0, st>>>(n, r, v, s, cnode, P->sc, P->rd);
+      ESPMV(0, G, C, op, w32, zpp, v, rh, P->sc, P->rd);
+      EV(e_update_s, G, C, n, r, v, s, cnode, P->sc, P->rd);
       if (pc) {
         ens_vcycle(P, s, 1, zs, st);
         zss = zs;
       }
-      EK(e_spmv_t, G, op, w32, zss, t, s, P->sc, P->rd);
-      e_update_xr<<<G, kT, 0, st>>>(n, x, r, rh, zpp, zss, s, t, pc ? 1 : 0, P->sc, P->rd);
-      e_update_p<<<G, kT, 0, st>>>(n, pp, r, v, cnode, P->sc, P->rd);
+      ESPMV(1, G, C, op, w32, zss, t, s, P->sc, P->rd);
+      EV(e_update_xr, G, C, n, x, r, rh, zpp, zss, s, t, pc ? 1 : 0, P->sc, P->rd);
+      EV(e_update_p, G, C, n, pp, r, v, cnode, P->sc, P->rd);
       P->launches += 5;
     }
     issued += chunk;
@@ -1410,7 +1742,7 @@ int ensemble_run(rbffd_ctx* ctx, const rbffd_flow* fp, int E, const double* Re, 
       constexpr int kReps = 20;
       cudaEventRecord(e0, st);
       for (int r = 0; r < kReps; ++r)
-        EK(e_spmv_v, G, L, P->Lw32, P->kw[7], P->kw[4], P->kw[2], P->sc_t, P->rd);
+        ESPMV(0, G, E, L, P->Lw32, P->kw[7], P->kw[4], P->kw[2], P->sc_t, P->rd);
       cudaEventRecord(e1, st);
       float ms = 0.f;
       rc = check_cuda(ctx, cudaEventSynchronize(e1), "timing sync");
