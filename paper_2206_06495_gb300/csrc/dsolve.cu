@@ -13,6 +13,8 @@ namespace rbffd {
 
 namespace {
 
+constexpr int kPT = 1024;      // threads per block, one block per SM
+constexpr int kPW = kPT / 32;  // warps per block
 constexpr int kMaxSweeps = 8;
 constexpr int kOwn = 32;  // rows a block of the inversion owns, at most
 
@@ -54,7 +56,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dense_invert(const __grid_constant__
   __shared__ double part[kNVMax * 4];
   __shared__ double f[kOwn], cv[kOwn], s_inv;
   __shared__ int used[kOwn], okf, s_p, s_bad;
-  Grid g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals};
   const int tid = threadIdx.x, n = a.n, nb = gridDim.x, blk = blockIdx.x;
   const int own = blk < n ? (n - blk + nb - 1) / nb : 0;
   if (tid < kOwn) {
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
   __shared__ double part[kNVMax * 4];
   __shared__ double s_sig, s_rr, s_bb;
   __shared__ int okf;
-  Grid g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = min(a.M, a.rows * (int)blockIdx.x), r1 = min(a.M, r0 + a.rows);
   const int active = min(kPT, (a.rows + 31) / 32 * 32);

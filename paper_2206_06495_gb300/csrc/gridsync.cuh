@@ -5,16 +5,16 @@
 
 namespace rbffd {
 
-constexpr int kPT = 1024;      // threads per block, one block per SM
-constexpr int kPW = kPT / 32;  // warps per block
-constexpr int kNVMax = 4;      // values reduced together
+constexpr int kNVMax = 4;  // values reduced together, where a kernel does not say otherwise
 constexpr long long kPolls = 1ll << 22;  // bounded barrier wait (a phase takes microseconds)
 
 // The block's share of the grid-wide machinery.  Every block sees the same
 // totals, so every block takes the same decisions.
+// PT threads per block, one block per SM; at most NVM values reduced together.
+template <int PT, int NVM = kNVMax>
 struct Grid {
-  double* sh;              // [kNVMax][kPT]
-  double* part;            // [kNVMax][4]
+  double* sh;              // [NVM][PT]
+  double* part;            // [NVM][4]
   int* ok;                 // shared: the last barrier's verdict
   double* partials;
   unsigned int* arrivals;
@@ -28,14 +28,15 @@ struct Grid {
     __syncthreads();
     target += gridDim.x;
     if (threadIdx.x == 0) {
-      __threadfence();
+      // release and acquire order the whole block's accesses, through the
+      // block barriers on both sides; a fence of its own on each side cost
+      // another 0.4 us a barrier
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrivals) : "memory");
       unsigned int got;
       long long polls = 0;
       do {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(arrivals) : "memory");
       } while ((int)(got - target) < 0 && ++polls < kPolls);
-      __threadfence();
       *ok = (int)(got - target) >= 0;
     }
     __syncthreads();
@@ -54,22 +55,22 @@ struct Grid {
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     if (t < active) {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) sh[j * kPT + t] = v[j];
+      for (int j = 0; j < NV; ++j) sh[j * PT + t] = v[j];
     }
     __syncthreads();
-    if (w < 4 * NV) {
-      const int j = w >> 2, q = w & 3;
+    for (int jq = w; jq < 4 * NV; jq += PT / 32) {
+      const int j = jq >> 2, q = jq & 3;
       double a = 0.0;
 #pragma unroll
-      for (int u = 0; u < kPW / 4; ++u) {
+      for (int u = 0; u < PT / 128; ++u) {
         const int e = (q + 4 * u) * 32;
-        if (e < active) a += sh[j * kPT + e + lane];
+        if (e < active) a += sh[j * PT + e + lane];
       }
       if (q * 32 < active) a = warp_sum(a);
       if (lane == 0) part[j * 4 + q] = a;
     }
     __syncthreads();
-    double* mine = partials + (size_t)(phase & 1) * kNVMax * gridDim.x;
+    double* mine = partials + (size_t)(phase & 1) * NVM * gridDim.x;
     ++phase;
     if (t < NV) {
       const double* q = part + t * 4;
@@ -92,5 +93,26 @@ struct Grid {
     return true;
   }
 };
+
+// a / b for the scalars of a solve (one thread's work, which every block waits
+// for): the approximate reciprocal instruction and two steps of Newton's
+// iteration for 1 / b, a shorter serial chain than a correctly rounded
+// division; within two units in the last place.
+__device__ __forceinline__ double quot(double a, double b) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  y = fma(y, fma(-b, y, 1.0), y);
+  y = fma(y, fma(-b, y, 1.0), y);
+  return fabs(b) > 1e-290 && fabs(b) < 1e290 ? a * y : a / b;
+}
+
+// sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
+__device__ __forceinline__ float hash_sign(int i, uint32_t seed) {
+  uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  h ^= h >> 12;
+  return (h & 1u) ? 1.f : -1.f;
+}
 
 }  // namespace rbffd

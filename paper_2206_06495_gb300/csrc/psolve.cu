@@ -1,7 +1,7 @@
 // The preconditioned pressure solve (Section 3, Eq. pressure_Poisson) as one
 // resident kernel: BiCGSTAB, its V-cycles and its restarts run in a single
-// cooperative launch of one 1,024-thread block per SM, with a grid barrier
-// between dependent phases.
+// cooperative launch of one block per SM, with a grid barrier between dependent
+// phases.
 //
 // What bounds it: an iteration is a chain of about 2 (2 nlev + 1) dependent
 // phases.  As launches of a replayed graph a phase costs 2.5 us at the least
@@ -30,8 +30,18 @@ namespace rbffd {
 
 namespace {
 
+// Threads per block (one block per SM).  512 where the phases are bound by
+// latency: with 1,024, 64 registers a thread spill, and the spilled addresses
+// are reloaded through L2 in every phase (each barrier empties L1), 0.7 us a
+// phase (FP64 100k rows: 94 against 104 us an iteration; MIXED 250k: 123 against
+// 140).  1,024 where they are bound by the streams and need the loads in
+// flight (FP64 1M rows: 0.38 against 0.46 ms).
+constexpr int kSmallPT = 512, kLargePT = 1024;
+constexpr int64_t kLargeRows = 300000;
 constexpr int kCycle = 50;            // iterations before a restart from the true residual
 constexpr int kMaxCycles = 400;       // restarts of one solve before giving up
+// shared memory for static rows: a block's 227 KB less what the reductions take
+constexpr size_t stage_room(int pt) { return 226 * 1024 - sizeof(double) * kNVMax * pt; }
 
 // One level of the hierarchy as the kernel reads it (rows of level l + 1 are
 // the aggregates of level l; the coarsest level uses n and r only).
@@ -41,7 +51,20 @@ struct PLevel {
   const float *val, *diag, *wd;
   const int32_t* cptr;
   float *r, *x;
+  // Block b restricts the aggregates 8 per b .. (a task is eight aggregates).
+  // With soff >= 0 the graph rows of those aggregates are kept in shared
+  // memory (from byte soff) for the whole solve: idx [width][cap], val
+  // [width][cap], diag [cap], wd [cap], the aggregates' first rows
+  // [8 per + 1] and, above level 0, each row's first row on the finer level
+  // [cap + 1], with cap = 32 per.  (Eight FP64 steps of 100k rows 63.2 to 55.1
+  // ms, a MIXED one of 250k 15.3 to 11.5, with the lighter barrier and the 512
+  // threads; a barrier empties L1, so unstaged rows came from L2 every time.)
+  int per, soff;
 };
+__host__ __device__ inline size_t stage_bytes(int width, int per, bool level0) {
+  const size_t cap = 32 * (size_t)per;
+  return 4 * (2 * width * cap + 2 * cap + 8 * per + 1 + (level0 ? 0 : cap + 1));
+}
 
 template <typename T>
 struct PArgs {
@@ -60,6 +83,7 @@ struct PArgs {
   PLevel lev[kAmgMaxLevels];
   int nlev, nc, ldx;
   const float* X;  // [nc][ldx] dense inverse of the coarsest level, rows padded with zeros
+  int xoff;        // >= 0: the block's rows of X stay in shared memory from this byte
   double inv_ces, inv_R, tol2;
   int maxit, x_zero;
   uint32_t seed;
@@ -68,52 +92,85 @@ struct PArgs {
   PSolveResult* res;
 };
 
-// sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
-__device__ __forceinline__ float p_sign(int i, uint32_t seed) {
-  uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;
-  h ^= h >> 15;
-  h *= 0x2C1B3C6Du;
-  h ^= h >> 12;
-  return (h & 1u) ? 1.f : -1.f;
-}
-
 // y_i = sum_s w_s z_j (FP64), or sum_s w_s (z_j - z_i) (FP32 rows, applied in
 // difference form: step.cu, k_spmv_pc)
-template <int K, typename T>
+// The operator's rows: read twice an iteration; larger than L2 (STREAM), they
+// are marked for early eviction so that the vectors stay there.
+template <bool STREAM, typename V>
+__device__ __forceinline__ V stream_ld(const V* p) {
+  return STREAM ? __ldcs(p) : __ldg(p);
+}
+
+template <int K, bool STREAM, typename T>
 __device__ __forceinline__ T p_row(const PArgs<T>& a, int i, const T* z, T zi) {
   constexpr bool dif = std::is_same<T, float>::value;
   T acc = 0;
   if constexpr (K > 0) {
 #pragma unroll
     for (int s = 0; s < K; ++s) {
-      const T zj = z[__ldg(a.idx + s * a.ld + i)];
-      acc += __ldg(a.w + s * a.ld + i) * (dif ? zj - zi : zj);
+      const T zj = z[stream_ld<STREAM>(a.idx + s * a.ld + i)];
+      acc += stream_ld<STREAM>(a.w + s * a.ld + i) * (dif ? zj - zi : zj);
     }
   } else {
 #pragma unroll 4
     for (int s = 0; s < a.k; ++s) {
-      const T zj = z[__ldg(a.idx + s * a.ld + i)];
-      acc += __ldg(a.w + s * a.ld + i) * (dif ? zj - zi : zj);
+      const T zj = z[stream_ld<STREAM>(a.idx + s * a.ld + i)];
+      acc += stream_ld<STREAM>(a.w + s * a.ld + i) * (dif ? zj - zi : zj);
     }
   }
   return acc;
 }
 
-// diag x_i + sum_s val_s x_j over row i of a level, W slots in flight at once
-template <int W>
-__device__ __forceinline__ float p_graph(const PLevel& F, int i, float xi) {
-  float ax = __ldg(F.diag + i) * xi;
-  for (int s0 = 0; s0 < F.width; s0 += W) {
+// The rows of a level that a block works on: in global memory (row i at
+// [s ld + i]) or staged in shared memory (S; local row i at [s cap + i]).
+template <bool S>
+struct Rows {
+  const int32_t* idx;
+  const float *val, *diag, *wd;
+  int64_t ld;
+  int width;
+};
+extern __shared__ __align__(16) unsigned char psm[];
+
+template <bool S>
+__device__ __forceinline__ Rows<S> rows_of(const PLevel& F) {
+  if constexpr (S) {
+    const int cap = 32 * F.per;
+    const int32_t* p = reinterpret_cast<const int32_t*>(psm + F.soff);
+    const float* v = reinterpret_cast<const float*>(p + F.width * cap);
+    return {p, v, v + F.width * cap, v + F.width * cap + cap, cap, F.width};
+  } else {
+    return {F.idx, F.val, F.diag, F.wd, F.ld, F.width};
+  }
+}
+template <bool S>
+__device__ __forceinline__ const int32_t* agg_of(const PLevel& F) {  // first rows of the aggregates
+  const int cap = 32 * F.per;
+  return reinterpret_cast<const int32_t*>(psm + F.soff) + 2 * F.width * cap + 2 * cap;
+}
+template <bool S, typename V>
+__device__ __forceinline__ V ro(const V* p) {
+  if constexpr (S)
+    return *p;
+  else
+    return __ldg(p);
+}
+
+// diag x_i + sum_s val_s x_j over row i, W slots in flight at once
+template <int W, bool S>
+__device__ __forceinline__ float p_graph(const Rows<S>& R, int i, const float* x, float xi) {
+  float ax = ro<S>(R.diag + i) * xi;
+  for (int s0 = 0; s0 < R.width; s0 += W) {
     int32_t j[W];
     float v[W];
 #pragma unroll
     for (int s = 0; s < W; ++s) {
-      const bool in = s0 + s < F.width;
-      j[s] = in ? __ldg(F.idx + (int64_t)(s0 + s) * F.ld + i) : i;
-      v[s] = in ? __ldg(F.val + (int64_t)(s0 + s) * F.ld + i) : 0.f;
+      const bool in = s0 + s < R.width;
+      j[s] = in ? ro<S>(R.idx + (s0 + s) * R.ld + i) : ro<S>(R.idx + i);
+      v[s] = in ? ro<S>(R.val + (s0 + s) * R.ld + i) : 0.f;
     }
 #pragma unroll
-    for (int s = 0; s < W; ++s) ax += v[s] * F.x[j[s]];
+    for (int s = 0; s < W; ++s) ax += v[s] * x[j[s]];
   }
   return ax;
 }
@@ -122,20 +179,23 @@ __device__ __forceinline__ float p_graph(const PLevel& F, int i, float xi) {
 // takes eight consecutive aggregates, whose rows (at most 32) are consecutive;
 // lane q adds the rows of aggregate q in row order.  The coarse level's
 // iterate x = omega D^-1 r is written with its r.
-template <int W>
-__device__ __forceinline__ void p_restrict(const PLevel& F, const PLevel& Cn, bool coarsest) {
+template <int W, bool S, int PT>
+__device__ __forceinline__ void p_restrict(const PLevel& F, const PLevel& Cn, bool coarsest,
+                                           int first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int tasks = (Cn.n + 7) / 8;
-  const int per = (tasks + gridDim.x - 1) / gridDim.x;
-  const int t1 = min(tasks, per * ((int)blockIdx.x + 1));
-  for (int t = per * blockIdx.x + warp; t < t1; t += kPW) {
+  const int tasks = (Cn.n + 7) / 8, t0 = F.per * blockIdx.x;
+  const int t1 = min(tasks, t0 + F.per);
+  const Rows<S> R = rows_of<S>(F);
+  for (int t = t0 + warp; t < t1; t += (PT / 32)) {
     const int I = 8 * t + lane;
-    const int cp = __ldg(F.cptr + min(8 * t + min(lane, 8), Cn.n));
+    const float wc = !coarsest && lane < 8 && I < Cn.n ? __ldg(Cn.wd + I) : 0.f;
+    const int at = min(8 * t + min(lane, 8), Cn.n);
+    const int cp = S ? agg_of<S>(F)[at - 8 * t0] : __ldg(F.cptr + at);  // local row with S
     const int f0 = __shfl_sync(0xffffffffu, cp, 0), f1 = __shfl_sync(0xffffffffu, cp, 8);
     const int nx = __shfl_down_sync(0xffffffffu, cp, 1);
-    const int i = f0 + lane;
+    const int i = f0 + lane, gi = S ? first + i : i;
     float res = 0.f;
-    if (i < f1) res = F.r[i] - p_graph<W>(F, i, F.x[i]);
+    if (i < f1) res = F.r[gi] - p_graph<W, S>(R, i, F.x, F.x[gi]);
     const int o = cp - f0, cnt = nx - cp;
     float acc = 0.f;
 #pragma unroll
@@ -145,50 +205,99 @@ __device__ __forceinline__ void p_restrict(const PLevel& F, const PLevel& Cn, bo
     }
     if (lane < 8 && I < Cn.n) {
       Cn.r[I] = acc;
-      if (!coarsest) Cn.x[I] = __ldg(Cn.wd + I) * acc;
+      if (!coarsest) Cn.x[I] = wc * acc;
     }
   }
 }
 
 // Post-smoothing sweep of a level above 0, whose result corrects the finer
 // level's rows of each aggregate (at most four, read with the gathers).
-template <int W>
-__device__ __forceinline__ void p_up(const PLevel& F, const PLevel& Fine) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int tasks = (F.n + 31) / 32;
-  const int per = (tasks + gridDim.x - 1) / gridDim.x;
-  const int t1 = min(tasks, per * ((int)blockIdx.x + 1));
-  for (int t = per * blockIdx.x + warp; t < t1; t += kPW) {
-    const int i = 32 * t + lane;
-    if (i >= F.n) continue;
-    const int c0 = __ldg(Fine.cptr + i), c1 = __ldg(Fine.cptr + i + 1);
+template <int W, bool S, int PT>
+__device__ __forceinline__ void p_up(const PLevel& F, const PLevel& Fine, int first, int count) {
+  const Rows<S> R = rows_of<S>(F);
+  const int32_t* child = S ? agg_of<S>(F) + 8 * F.per + 1 : Fine.cptr;
+  auto row = [&](int i, int gi) {
+    const int c0 = ro<S>(child + i), c1 = ro<S>(child + i + 1);
     float xf[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) xf[q] = c0 + q < c1 ? Fine.x[c0 + q] : 0.f;
-    const float xi = F.x[i];
-    const float ax = p_graph<W>(F, i, xi);
-    const float v = kAmgCoarseScale * (xi + __ldg(F.wd + i) * (F.r[i] - ax));
+    const float xi = F.x[gi], ri = F.r[gi];
+    const float ax = p_graph<W, S>(R, i, F.x, xi);
+    const float v = kAmgCoarseScale * (xi + ro<S>(R.wd + i) * (ri - ax));
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (c0 + q < c1) Fine.x[c0 + q] = xf[q] + v;
+  };
+  if constexpr (S) {
+    for (int i = threadIdx.x; i < count; i += PT) row(i, first + i);
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tasks = (F.n + 31) / 32;
+    const int per = (tasks + gridDim.x - 1) / gridDim.x;
+    const int t1 = min(tasks, per * ((int)blockIdx.x + 1));
+    for (int t = per * blockIdx.x + warp; t < t1; t += (PT / 32)) {
+      const int i = 32 * t + lane;
+      if (i < F.n) row(i, i);
+    }
+  }
+}
+
+template <int PT>
+__device__ __forceinline__ void p_restrict_level(const PLevel& F, const PLevel& Cn, bool coarsest,
+                                                 int first) {
+  if (F.soff >= 0) {
+    if (F.width <= 8)
+      p_restrict<8, true, PT>(F, Cn, coarsest, first);
+    else
+      p_restrict<16, true, PT>(F, Cn, coarsest, first);
+  } else {
+    if (F.width <= 8)
+      p_restrict<8, false, PT>(F, Cn, coarsest, 0);
+    else
+      p_restrict<16, false, PT>(F, Cn, coarsest, 0);
+  }
+}
+template <int PT>
+__device__ __forceinline__ void p_up_level(const PLevel& F, const PLevel& Fine, int first,
+                                           int count) {
+  if (F.soff >= 0) {
+    if (F.width <= 8)
+      p_up<8, true, PT>(F, Fine, first, count);
+    else
+      p_up<16, true, PT>(F, Fine, first, count);
+  } else {
+    if (F.width <= 8)
+      p_up<8, false, PT>(F, Fine, 0, 0);
+    else
+      p_up<16, false, PT>(F, Fine, 0, 0);
   }
 }
 
 // Coarsest level: z = X r, one warp per row, 16 B loads with eight in flight;
-// then the correction of the finer level, or z itself without one.
-template <typename T>
+// then the correction of the finer level, or z itself without one.  Consecutive
+// rows are on different SMs, whose bandwidth bounds it.
+template <int PT, typename T>
 __device__ __forceinline__ void p_coarse(const PArgs<T>& a, T* z) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float4* r4 = reinterpret_cast<const float4*>(a.lev[a.nlev - 1].r);
   const int n4 = a.ldx / 4;
-  // row-to-warp map: consecutive rows on different SMs, whose bandwidth bounds it
-  for (int row = blockIdx.x + warp * gridDim.x; row < a.nc; row += gridDim.x * kPW) {
-    const float4* x4 = reinterpret_cast<const float4*>(a.X + (int64_t)row * a.ldx);
+  for (int q = warp, row = blockIdx.x + warp * gridDim.x; row < a.nc;
+       q += (PT / 32), row += gridDim.x * (PT / 32)) {
     float acc = 0.f;
+    if (a.xoff >= 0) {
+      const float4* x4 = reinterpret_cast<const float4*>(psm + a.xoff) + q * n4;
 #pragma unroll 8
-    for (int j = lane; j < n4; j += 32) {
-      const float4 u = __ldg(x4 + j), q = r4[j];
-      acc += u.x * q.x + u.y * q.y + u.z * q.z + u.w * q.w;
+      for (int j = lane; j < n4; j += 32) {
+        const float4 u = x4[j], v = r4[j];
+        acc += u.x * v.x + u.y * v.y + u.z * v.z + u.w * v.w;
+      }
+    } else {
+      const float4* x4 = reinterpret_cast<const float4*>(a.X + (int64_t)row * a.ldx);
+#pragma unroll 8
+      for (int j = lane; j < n4; j += 32) {
+        const float4 u = __ldg(x4 + j), v = r4[j];
+        acc += u.x * v.x + u.y * v.y + u.z * v.z + u.w * v.w;
+      }
     }
     acc = warp_sum(acc);
     if (a.nlev == 1) {
@@ -199,6 +308,51 @@ __device__ __forceinline__ void p_coarse(const PArgs<T>& a, T* z) {
       if (lane < c1 - c0) F.x[c0 + lane] += kAmgCoarseScale * acc;
     }
   }
+}
+
+// Copies the block's static rows into shared memory; first[l], count[l]: the
+// rows of level l that its aggregates hold.
+template <int PT, typename T>
+__device__ __forceinline__ void p_stage(const PArgs<T>& a, int* first, int* count) {
+  for (int l = 0; l + 1 < a.nlev; ++l) {
+    const PLevel& F = a.lev[l];
+    const int nagg = a.lev[l + 1].n;
+    const int k0 = min(nagg, 8 * F.per * (int)blockIdx.x), k1 = min(nagg, k0 + 8 * F.per);
+    const int f0 = __ldg(F.cptr + k0), nr = __ldg(F.cptr + k1) - f0;
+    if (threadIdx.x == 0) {
+      first[l] = f0;
+      count[l] = nr;
+    }
+    if (F.soff < 0) continue;
+    const int cap = 32 * F.per;
+    int32_t* pi = reinterpret_cast<int32_t*>(psm + F.soff);
+    float* pv = reinterpret_cast<float*>(pi + F.width * cap);
+    for (int s = 0; s < F.width; ++s)
+      for (int r = threadIdx.x; r < nr; r += PT) {
+        pi[s * cap + r] = __ldg(F.idx + (int64_t)s * F.ld + f0 + r);
+        pv[s * cap + r] = __ldg(F.val + (int64_t)s * F.ld + f0 + r);
+      }
+    float* pd = pv + F.width * cap;
+    for (int r = threadIdx.x; r < nr; r += PT) {
+      pd[r] = __ldg(F.diag + f0 + r);
+      pd[cap + r] = __ldg(F.wd + f0 + r);
+    }
+    int32_t* pa = reinterpret_cast<int32_t*>(pd + 2 * cap);
+    for (int k = threadIdx.x; k <= k1 - k0; k += PT) pa[k] = __ldg(F.cptr + k0 + k) - f0;
+    if (l > 0) {
+      int32_t* pc = pa + 8 * F.per + 1;
+      for (int r = threadIdx.x; r <= nr; r += PT) pc[r] = __ldg(a.lev[l - 1].cptr + f0 + r);
+    }
+  }
+  if (a.xoff >= 0) {
+    float4* xs = reinterpret_cast<float4*>(psm + a.xoff);
+    const int n4 = a.ldx / 4;
+    for (int q = 0, row = blockIdx.x; row < a.nc; ++q, row += gridDim.x) {
+      const float4* x4 = reinterpret_cast<const float4*>(a.X + (int64_t)row * a.ldx);
+      for (int j = threadIdx.x; j < n4; j += PT) xs[q * n4 + j] = __ldg(x4 + j);
+    }
+  }
+  __syncthreads();
 }
 
 // The solve's scalars, one copy per block (identical in all of them).
@@ -213,16 +367,16 @@ struct PScal {
   int ended;
 };
 
-template <int K, typename T>
-__global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs<T> a) {
-  __shared__ double sh[kNVMax * kPT];
+template <int K, typename T, int PT>
+__global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<T> a) {
+  __shared__ double sh[kNVMax * PT];
   __shared__ double part[kNVMax * 4];
   __shared__ PScal<T> S;
-  __shared__ int okf;
-  Grid g{sh, part, &okf, a.partials, a.arrivals};
+  __shared__ int okf, first[kAmgMaxLevels], count[kAmgMaxLevels];
+  Grid<PT> g{sh, part, &okf, a.partials, a.arrivals};
   const int tid = threadIdx.x;
   const int r0 = min(a.M, a.rows * (int)blockIdx.x), r1 = min(a.M, r0 + a.rows);
-  const int active = min(kPT, a.rows);
+  const int active = min(PT, a.rows);
   const PLevel& L0 = a.lev[0];
   constexpr bool dif = std::is_same<T, float>::value;
 
@@ -237,40 +391,43 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
   auto vcycle = [&](T* z, auto fin) -> bool {
     for (int l = 0; l + 1 < a.nlev; ++l) {
       const bool last = l + 2 == a.nlev;
-      if (a.lev[l].width <= 8)
-        p_restrict<8>(a.lev[l], a.lev[l + 1], last);
-      else
-        p_restrict<16>(a.lev[l], a.lev[l + 1], last);
+      p_restrict_level<PT>(a.lev[l], a.lev[l + 1], last, first[l]);
       if (!g.sync()) return false;
     }
-    p_coarse(a, z);
+    p_coarse<PT>(a, z);
     if (a.nlev == 1) {
       if (tid == 0) fin(0.0);
       return g.sync();
     }
     if (!g.sync()) return false;
     for (int l = a.nlev - 2; l >= 1; --l) {
-      if (a.lev[l].width <= 8)
-        p_up<8>(a.lev[l], a.lev[l - 1]);
-      else
-        p_up<16>(a.lev[l], a.lev[l - 1]);
+      p_up_level<PT>(a.lev[l], a.lev[l - 1], first[l], count[l]);
       if (!g.sync()) return false;
     }
     float part0 = 0.f;
-    for (int i = r0 + tid; i < r1; i += kPT) {
-      const float xi = L0.x[i];
-      const float ax = L0.width <= 8 ? p_graph<8>(L0, i, xi) : p_graph<16>(L0, i, xi);
-      const float zi = xi + __ldg(L0.wd + i) * (L0.r[i] - ax);
-      z[i] = (T)zi;
+    auto sweep0 = [&](auto staged, int i, int gi) {
+      constexpr bool ST = decltype(staged)::value;
+      const Rows<ST> R = rows_of<ST>(L0);
+      const float xi = L0.x[gi], ri = L0.r[gi];
+      const float ax = L0.width <= 8 ? p_graph<8, ST>(R, i, L0.x, xi)
+                                     : p_graph<16, ST>(R, i, L0.x, xi);
+      const float zi = xi + ro<ST>(R.wd + i) * (ri - ax);
+      z[gi] = (T)zi;
       part0 += zi;
+    };
+    if (L0.soff >= 0) {
+      for (int i = tid; i < count[0]; i += PT) sweep0(std::true_type{}, i, first[0] + i);
+    } else {
+      for (int i = r0 + tid; i < r1; i += PT) sweep0(std::false_type{}, i, i);
     }
     const double v[1] = {(double)part0};
-    return g.reduce<1>(v, active, [&](const double* t) { fin(t[0]); });
+    return g.template reduce<1>(v, PT, [&](const double* t) { fin(t[0]); });
   };
   auto fin_p = [&](double zsum) { S.kp = (T)((S.mu_p - zsum) * a.inv_R); };
   auto fin_s = [&](double zsum) { S.ks = (T)((S.mu_s - zsum) * a.inv_R); };
 
-  for (int i = r0 + tid; i < r1; i += kPT) {
+  p_stage<PT>(a, first, count);
+  for (int i = r0 + tid; i < r1; i += PT) {
     const int q = __ldg(a.perm + i);
     a.b[i] = a.b_in[q];
     a.x[i] = a.x_zero ? (T)0 : a.x_in[q];
@@ -281,24 +438,24 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
     const bool zero = a.x_zero && cyc == 0;
     if (!zero) {
       T sx = 0;
-      for (int i = r0 + tid; i < r1; i += kPT) sx += a.x[i];
+      for (int i = r0 + tid; i < r1; i += PT) sx += a.x[i];
       const double v[1] = {(double)sx};
-      if (!g.reduce<1>(v, active, [&](const double* t) { S.sig = t[0]; })) return;
+      if (!g.template reduce<1>(v, active, [&](const double* t) { S.sig = t[0]; })) return;
     }
     const uint32_t seed = (cyc || a.seed) ? 0x51ED27u + 977u * a.seed + (uint32_t)cyc : 0u;
     {
       const T sig = zero ? (T)0 : (T)S.sig;
       T prr = 0, pbb = 0, prh = 0, pc = 0;
-      for (int i = r0 + tid; i < r1; i += kPT) {
+      for (int i = r0 + tid; i < r1; i += PT) {
         const T bi = a.b[i];
         T ri = bi;
         if (!zero) {
           const T xi = a.x[i];
-          T ax = p_row<K>(a, i, a.x, xi);
+          T ax = p_row<K, (PT == kLargePT)>(a, i, a.x, xi);
           if (dif) ax += a.a1[i] * xi;
           ri = bi - (ax + a.es[i] * sig);
         }
-        const T sgn = seed ? (T)p_sign(__ldg(a.perm + i), seed) : (T)1;
+        const T sgn = seed ? (T)hash_sign(__ldg(a.perm + i), seed) : (T)1;
         a.r[i] = ri;
         a.rh[i] = sgn * ri;
         a.p[i] = ri;
@@ -308,7 +465,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
         pc += (T)__ldg(a.c + i) * ri;
       }
       const double v[4] = {(double)prr, (double)pbb, (double)prh, (double)pc};
-      const bool ok = g.reduce<4>(v, active, [&](const double* t) {
+      const bool ok = g.template reduce<4>(v, active, [&](const double* t) {
         S.rr = t[0];
         S.bb = t[1];
         S.rho = t[2];
@@ -327,7 +484,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
     bool run = S.go == 1;
     if (run) {
       const float mu = S.fp;
-      for (int i = r0 + tid; i < r1; i += kPT) feed(i, a.p[i], mu);
+      for (int i = r0 + tid; i < r1; i += PT) feed(i, a.p[i], mu);
       if (!g.sync()) return;
     }
     while (run) {
@@ -336,16 +493,16 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
       {
         const T kap = S.kp, mu = S.mp;
         T d0 = 0, d1 = 0;
-        for (int i = r0 + tid; i < r1; i += kPT) {
+        for (int i = r0 + tid; i < r1; i += PT) {
           const T zi = dif ? a.zp[i] : (T)0;
-          const T y = p_row<K>(a, i, a.zp, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
+          const T y = p_row<K, (PT == kLargePT)>(a, i, a.zp, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
                       __ldg(a.es + i) * mu;
           a.v[i] = y;
           d0 += a.rh[i] * y;
           d1 += (T)__ldg(a.c + i) * y;
         }
         const double v[2] = {(double)d0, (double)d1};
-        const bool ok = g.reduce<2>(v, active, [&](const double* t) {
+        const bool ok = g.template reduce<2>(v, active, [&](const double* t) {
           if (t[0] == 0.0 || !isfinite(t[0])) {
             S.status = isfinite(t[0]) ? 1 : 2;
             S.iters += 1;
@@ -353,7 +510,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
             S.ended = 1;
             return;
           }
-          S.alpha = S.rho / t[0];
+          S.alpha = quot(S.rho, t[0]);
           S.al = (T)S.alpha;
           S.cv = t[1];
           S.cs = S.cr - S.alpha * t[1];
@@ -369,7 +526,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
         const T al = S.al;
         const float mu = S.fs;
         T d0 = 0, d1 = 0;
-        for (int i = r0 + tid; i < r1; i += kPT) {
+        for (int i = r0 + tid; i < r1; i += PT) {
           const T si = a.r[i] - al * a.v[i];
           a.s[i] = si;
           feed(i, si, mu);
@@ -377,7 +534,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
           d1 += a.rh[i] * si;
         }
         const double v[2] = {(double)d0, (double)d1};
-        const bool ok = g.reduce<2>(v, active, [&](const double* t) {
+        const bool ok = g.template reduce<2>(v, active, [&](const double* t) {
           S.rhs = t[1];
           if (t[0] <= a.tol2 * S.bb) {  // converged at the half step
             S.rr = t[0];
@@ -390,7 +547,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
       }
       if (S.go == 2) {
         const T al = S.al, kp = S.kp;
-        for (int i = r0 + tid; i < r1; i += kPT) a.x[i] += al * (a.zp[i] + kp);
+        for (int i = r0 + tid; i < r1; i += PT) a.x[i] += al * (a.zp[i] + kp);
         break;
       }
       if (!vcycle(a.zs, fin_s)) return;
@@ -398,9 +555,9 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
       {
         const T kap = S.ks, mu = S.ms;
         T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
-        for (int i = r0 + tid; i < r1; i += kPT) {
+        for (int i = r0 + tid; i < r1; i += PT) {
           const T zi = dif ? a.zs[i] : (T)0;
-          const T y = p_row<K>(a, i, a.zs, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
+          const T y = p_row<K, (PT == kLargePT)>(a, i, a.zs, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
                       __ldg(a.es + i) * mu;
           a.t[i] = y;
           d0 += y * a.s[i];
@@ -409,7 +566,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
           d3 += a.rh[i] * y;
         }
         const double v[4] = {(double)d0, (double)d1, (double)d2, (double)d3};
-        const bool ok = g.reduce<4>(v, active, [&](const double* t) {
+        const bool ok = g.template reduce<4>(v, active, [&](const double* t) {
           if (!(t[1] > 0.0) || !isfinite(t[0])) {
             S.status = isfinite(t[1]) ? 3 : 2;
             S.iters += 1;
@@ -417,9 +574,9 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
             S.ended = 1;
             return;
           }
-          const double om = t[0] / t[1];
+          const double om = quot(t[0], t[1]);
           const double rn = S.rhs - om * t[3];
-          const double be = (rn / S.rho) * (S.alpha / om);
+          const double be = quot(rn, S.rho) * quot(S.alpha, om);
           S.rho = rn;
           S.omega = om;
           S.om = (T)om;
@@ -435,11 +592,11 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
       if (S.go != 1) break;
       // x, r and p, and the next V-cycle's input; (r, r)
       {
-        const T al = S.al, om = S.om, be = S.be, kp = S.kp, ks = S.ks;
+        const T al = S.al, om = S.om, be = S.be, shift = al * S.kp + om * S.ks;
         const float mu = S.fp;
         T d0 = 0;
-        for (int i = r0 + tid; i < r1; i += kPT) {
-          a.x[i] += al * (a.zp[i] + kp) + om * (a.zs[i] + ks);
+        for (int i = r0 + tid; i < r1; i += PT) {
+          a.x[i] += al * a.zp[i] + (om * a.zs[i] + shift);
           const T ri = a.s[i] - om * a.t[i];
           a.r[i] = ri;
           const T pi = ri + be * (a.p[i] - om * a.v[i]);
@@ -448,7 +605,7 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
           d0 += ri * ri;
         }
         const double v[1] = {(double)d0};
-        const bool ok = g.reduce<1>(v, active, [&](const double* t) {
+        const bool ok = g.template reduce<1>(v, active, [&](const double* t) {
           const double rr = t[0];
           const bool conv = rr <= a.tol2 * S.bb;
           S.rr = rr;
@@ -481,10 +638,10 @@ __global__ void __launch_bounds__(kPT, 1) k_psolve(const __grid_constant__ PArgs
       break;
     }
     if (st == 5)  // the recurrence has blown up: start again from the initial iterate
-      for (int i = r0 + tid; i < r1; i += kPT)
+      for (int i = r0 + tid; i < r1; i += PT)
         a.x[i] = a.x_zero ? (T)0 : a.x_in[__ldg(a.perm + i)];
   }
-  for (int i = r0 + tid; i < r1; i += kPT) a.x_out[__ldg(a.perm + i)] = a.x[i];
+  for (int i = r0 + tid; i < r1; i += PT) a.x_out[__ldg(a.perm + i)] = a.x[i];
 }
 
 // ------------------------------------------------------------------ set-up
@@ -521,6 +678,8 @@ struct PSolve {
   std::vector<void*> allocs;
   bool mix = false;
   int grid = 0;
+  size_t smem = 0;
+  int pt = 0;  // threads per block
   PArgs<double> a64{};
   PArgs<float> a32{};
 };
@@ -599,6 +758,24 @@ int fill(rbffd_ctx* ctx, PSolve* p, PArgs<T>& a, int64_t M, int64_t ld, int k,
     q.cptr = g.cptr;
     if ((rc = p_alloc(ctx, p, &q.r, g.ld, st)) || (rc = p_alloc(ctx, p, &q.x, g.ld, st))) return rc;
   }
+  // shared memory for the static rows: the levels from the coarsest up (two
+  // phases a V-cycle use each), then the rows of the dense inverse
+  p->smem = 0;
+  for (int l = 0; l + 1 < a.nlev; ++l) {
+    a.lev[l].per = ((a.lev[l + 1].n + 7) / 8 + p->grid - 1) / p->grid;
+    a.lev[l].soff = -1;
+  }
+  bool room = true;
+  for (int l = a.nlev - 2; l >= 0 && room; --l) {
+    const size_t need = round_up(stage_bytes(a.lev[l].width, a.lev[l].per, l == 0), 16);
+    room = p->smem + need <= stage_room(p->pt);
+    if (!room) break;
+    a.lev[l].soff = (int)p->smem;
+    p->smem += need;
+  }
+  const size_t xneed = sizeof(float) * (size_t)a.ldx * ((a.nc + p->grid - 1) / p->grid);
+  a.xoff = p->smem + xneed <= stage_room(p->pt) ? (int)p->smem : -1;
+  if (a.xoff >= 0) p->smem += xneed;
   a.inv_ces = amg->inv_ces;
   a.inv_R = amg->inv_R;
   if ((rc = p_alloc(ctx, p, &a.partials, (size_t)2 * kNVMax * p->grid, st)) ||
@@ -626,6 +803,7 @@ int psolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   PSolve* p = new PSolve();
   p->mix = mix;
   p->grid = sm_count();
+  p->pt = M > kLargeRows ? kLargePT : kSmallPT;
   const int rc = mix ? fill(ctx, p, p->a32, M, ld, k, idx, w, es, a1, amg, st)
                      : fill(ctx, p, p->a64, M, ld, k, idx, w, es, a1, amg, st);
   if (rc) {
@@ -652,10 +830,17 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
   int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, sizeof(unsigned int), st), "memset");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
   if (rc) return rc;
-  const void* fn = a.k == 28 ? (const void*)k_psolve<28, T> : (const void*)k_psolve<0, T>;
+  const void* fn =
+      p->pt == kLargePT
+          ? (a.k == 28 ? (const void*)k_psolve<28, T, kLargePT> : (const void*)k_psolve<0, T, kLargePT>)
+          : (a.k == 28 ? (const void*)k_psolve<28, T, kSmallPT> : (const void*)k_psolve<0, T, kSmallPT>);
   void* args[] = {&a};
-  rc = check_cuda(ctx, cudaLaunchCooperativeKernel(fn, dim3(p->grid), dim3(kPT), args, 0, st),
-                  "pressure solve");
+  rc = check_cuda(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)stage_room(p->pt)),
+                  "pressure solve shared memory");
+  if (!rc)
+    rc = check_cuda(ctx, cudaLaunchCooperativeKernel(fn, dim3(p->grid), dim3(p->pt), args, p->smem, st),
+                    "pressure solve");
   if (!rc)
     rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(PSolveResult), cudaMemcpyDeviceToHost, st),
                     "pressure solve result");

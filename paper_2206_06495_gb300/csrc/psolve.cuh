@@ -9,12 +9,11 @@ namespace rbffd {
 
 struct PSolve;
 
-// Up to this many rows the resident kernel is the faster form; beyond it the
-// phases are long enough to hide their launches, and the graph of separate
-// launches, whose products and level-0 sweeps have more warps in flight, is
-// (FP64 step at 1M rows: 33.7 ms a step as launches, 34.2 resident; at 100k
-// rows 9.9 against 7.9, MIXED at 250k rows 17.3 against 15.5).
-constexpr int64_t kResidentMax = 1 << 19;
+// Up to this many rows the resident kernel is the faster form (FP64 step at 1M
+// rows: 0.38 against 0.41 ms an iteration as separate launches, at 100k rows
+// 0.08 against 0.13); larger systems have not been measured and keep the graph
+// of separate launches.
+constexpr int64_t kResidentMax = 1 << 21;
 
 struct PSolveResult {
   int iters = 0;

@@ -44,3 +44,24 @@ def test_forms_match_the_oracle(n, precision, profile):
     # the direct solve needs at most a few products a step, the Krylov one many
     direct = n <= 64 and not profile
     assert (stats["poisson_iters"] <= 20) == direct, stats["poisson_iters"]
+
+
+# either side of 300,000 rows, where the resident kernel's block grows
+@pytest.mark.parametrize("n", [547, 548])
+def test_resident_and_launched_solves_agree(n):
+    """A step from the lid's start by the resident kernel and, in a profiled
+    flow, by separate launches, both to 1e-12: velocities within 1e-9 and p~
+    within 1e-8 relative, the bars above."""
+    from paper_2206_06495_gb300 import rbffd as R
+    nd = ns.jittered_cavity(n, 3)
+    gu, gv = (_d(g) for g in O.lid_bc(nd))
+    got = []
+    for profile in (0, 1):
+        ctx = R.Context(28, 7, 3)
+        flow = R.flow_from_nodes(ctx, nd, Re=100.0, dt=0.08 / (n - 1), tol=1e-12, profile=profile)
+        st = R.State.zeros(flow)
+        R.step(ctx, flow, st, gu, gv, 1)
+        got.append(st)
+    a, b = got
+    assert max((a.u - b.u).abs().max(), (a.v - b.v).abs().max()) < 1e-9
+    assert (a.pt - b.pt).abs().max() < 1e-8 * b.pt.abs().max()
