@@ -168,11 +168,18 @@ def lib():
     return _lib
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("rbffd needs a CUDA device; no CPU fallback exists")
-    return torch
+    # asked once: the availability check costs more than a small launch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("rbffd needs a CUDA device; no CPU fallback exists")
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream():
@@ -188,6 +195,15 @@ def _ptr(t):
     if not t.is_contiguous():
         raise ValueError("rbffd arrays must be contiguous")
     return C.c_void_p(t.data_ptr())
+
+
+def _addr(t) -> int:
+    """_ptr as a plain integer (0 for an empty tensor)."""
+    if not t.is_cuda:
+        raise ValueError("rbffd arrays must be CUDA tensors")
+    if not t.is_contiguous():
+        raise ValueError("rbffd arrays must be contiguous")
+    return t.data_ptr()
 
 
 def round_up(a: int, b: int = 32) -> int:
@@ -269,13 +285,17 @@ def apply_op(ctx: Context, idx, w, n_rows: int, n_cols: int, x, y=None, alpha: f
              beta: float = 0.0):
     """rbffd_apply_op: y = alpha * D x + beta * y.  w: [n, ld] float64 or float32."""
     torch = _torch()
-    if y is None:
-        y = torch.zeros(n_rows, dtype=x.dtype, device=x.device)
-    D = Ell(idx=_ptr(idx).value, w=_ptr(w).value, n_rows=n_rows, n_cols=n_cols,
-            ld=idx.shape[1], n=idx.shape[0], w_dtype=F64 if w.dtype == torch.float64 else F32)
-    xy = F64 if x.dtype == torch.float64 else F32
-    ctx.check(lib().rbffd_apply_op(ctx.handle, C.byref(D), _ptr(x), _ptr(y), alpha, beta, xy,
-                                   _stream()))
+    if y is None:  # with beta == 0 the call writes every entry and reads none
+        new = torch.empty if beta == 0.0 else torch.zeros
+        y = new(n_rows, dtype=x.dtype, device=x.device)
+    shape, f64 = idx.shape, torch.float64
+    D = Ell(_addr(idx), _addr(w), n_rows, n_cols, shape[1], shape[0],
+            F64 if w.dtype == f64 else F32)
+    rc = lib().rbffd_apply_op(ctx.handle, C.byref(D), _addr(x), _addr(y), alpha, beta,
+                              F64 if x.dtype == f64 else F32,
+                              torch.cuda.current_stream().cuda_stream)
+    if rc != OK:
+        ctx.check(rc)
     return y
 
 
