@@ -1,8 +1,12 @@
+// The two solves of a small flow's step.
+//
 // Direct pressure solve of small systems (Section 3, Eq. pressure_Poisson; the
 // paper factorises its implicit matrices once, too): the dense inverse of the
 // scaled operator A_f = A + es 1^T is built once per plan, and a solve is a
 // product with it inside iterative refinement on the sparse operator, in one
 // cooperative launch.
+//
+// Resident viscous solve: both components' BiCGSTAB in one cooperative launch.
 #include <algorithm>
 #include <cmath>
 
@@ -175,9 +179,17 @@ struct DArgs {
   double *x, *r;  // r: ldt values, zero beyond M
   double tol2;
   double* partials;
-  unsigned int* arrivals;
+  unsigned int* arrivals;  // two words, zero between launches
   PSolveResult* res;
+  int* fail;  // null, or see psolve.cuh
+  int step;
 };
+
+// a barrier that ran out of its bounded wait
+template <typename A>
+__device__ __forceinline__ void give_up(const A& a) {
+  if (a.fail && threadIdx.x == 0) *a.fail = (a.step << 4) | kFailWait;
+}
 
 // Refinement: r = b - A_f x, x += A_f^-1 r until (r, r) <= tol^2 (b, b).  A
 // block owns `rows` consecutive rows, in the residual (one thread per row) and
@@ -186,6 +198,7 @@ struct DArgs {
 // latency of its four phases.
 template <int K>
 __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs a) {
+  if (a.fail && *a.fail) return;
   __shared__ __align__(16) double sh[kNVMax * kPT];
   static_assert(kNVMax * kPT >= kDenseMax, "the residual is staged in sh");
   __shared__ double part[kNVMax * 4];
@@ -199,7 +212,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
     double sx = 0.0;
     for (int i = r0 + tid; i < r1; i += kPT) sx += a.x[i];
     const double v[1] = {sx};
-    if (!g.reduce<1>(v, active, [&](const double* t) { s_sig = t[0]; })) return;
+    if (!g.reduce<1>(v, active, [&](const double* t) { s_sig = t[0]; })) return give_up(a);
   }
   double prev = INFINITY;
   for (int sweep = 0;; ++sweep) {
@@ -226,7 +239,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
       s_rr = t[0];
       s_bb = t[1];
     });
-    if (!ok) return;
+    if (!ok) return give_up(a);
     const double rr = s_rr, bb = s_bb;
     const bool conv = rr <= a.tol2 * bb, fin = isfinite(rr);
     // a sweep that does not halve the residual has reached the rounding level
@@ -237,8 +250,9 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
         a.res->status = conv ? 0 : (fin ? 5 : 2);
         a.res->relres = bb > 0 ? sqrt(rr / bb) : sqrt(rr);
         a.res->converged = conv;
+        if (a.fail && !conv) *a.fail = (a.step << 4) | kFailPressure;
       }
-      return;
+      return leave(a.arrivals);
     }
     prev = rr;
     // x += inv r: the rows' products need all of r, read once per block
@@ -264,11 +278,337 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
     }
     __syncthreads();  // sh is reused by the reduction
     const double vx[1] = {sx};
-    if (!g.reduce<1>(vx, kPT, [&](const double* t) { s_sig = t[0]; })) return;
+    if (!g.reduce<1>(vx, kPT, [&](const double* t) { s_sig = t[0]; })) return give_up(a);
+  }
+}
+
+// ---------------------------------------------------------- viscous solves
+constexpr int kVT = 512;  // threads per block
+constexpr int kVNV = 6;
+
+struct VArgs {
+  int N, rows, k;
+  int64_t ld;
+  const int32_t* idx;
+  const double* w[2];
+  double* x[2];
+  const double* b[2];
+  double *r[2], *rh[2], *p[2], *v[2], *s[2], *t[2], *x0[2];
+  double tol2, accept2;
+  int maxit;
+  double* partials;        // [2][kVNV][gridDim.x]
+  unsigned int* arrivals;  // two words, zero between launches
+  PSolveResult* res;
+  int* fail;
+  int step;
+};
+
+struct VScal {
+  double rho[2], rr[2], bb[2], rhs[2], alpha[2], omega[2], beta[2];
+  int active[2], half[2], status, iters, total, go, iterate;
+};
+
+// y_q = x_q + sum_s w_q,s x_q,j of row i
+template <int K>
+__device__ __forceinline__ void v_row(const VArgs& a, int i, double* const* x, double (&y)[2]) {
+  const bool same = a.w[0] == a.w[1];
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll(K > 0 ? K : 4)
+  for (int s = 0; s < (K > 0 ? K : a.k); ++s) {
+    const int j = __ldg(a.idx + s * a.ld + i);
+    const double w0 = __ldg(a.w[0] + s * a.ld + i);
+    const double w1 = same ? w0 : __ldg(a.w[1] + s * a.ld + i);
+    s0 += w0 * x[0][j];
+    s1 += w1 * x[1][j];
+  }
+  y[0] = s0 + x[0][i];
+  y[1] = s1 + x[1][i];
+}
+
+// What bounds it: latency, four phases an iteration of about 5 us each.  As
+// separate launches an iteration took five kernels of 1,216 blocks (75 us with
+// cold caches at 4,641 rows) and the solve two or three waits of the host.
+// (rh, r) = (rh, s) - omega (rh, t), so x, r and p are one pass.  A component
+// that has converged keeps its x while the other one goes on.
+template <int K>
+__global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs a) {
+  if (*a.fail) return;
+  __shared__ double sh[kVNV * kVT];
+  __shared__ double part[kVNV * 4];
+  __shared__ VScal S;
+  __shared__ int okf;
+  Grid<kVT, kVNV> g{sh, part, &okf, a.partials, a.arrivals};
+  const int tid = threadIdx.x;
+  const int r0 = min(a.N, a.rows * (int)blockIdx.x), r1 = min(a.N, r0 + a.rows);
+  const int active = min(kVT, (a.rows + 31) / 32 * 32);
+  for (int i = r0 + tid; i < r1; i += kVT)
+    for (int q = 0; q < 2; ++q) a.x0[q][i] = a.x[q][i];
+  if (tid == 0) S.total = 0;
+  for (int cyc = 0;; ++cyc) {
+    const uint32_t seed = cyc ? 0x51ED27u + (uint32_t)cyc : 0u;
+    {
+      double d[6] = {};
+      for (int i = r0 + tid; i < r1; i += kVT) {
+        double y[2];
+        v_row<K>(a, i, a.x, y);
+        const double sgn = seed ? (double)hash_sign(i, seed) : 1.0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const double bi = a.b[q][i], ri = bi - y[q];
+          a.r[q][i] = ri;
+          a.rh[q][i] = sgn * ri;
+          a.p[q][i] = ri;
+          d[3 * q] += ri * ri;
+          d[3 * q + 1] += bi * bi;
+          d[3 * q + 2] += sgn * ri * ri;
+        }
+      }
+      const bool ok = g.template reduce<6>(d, active, [&](const double* t) {
+        S.status = 0;
+        S.iters = 0;
+        S.go = 0;
+        for (int q = 0; q < 2; ++q) {
+          S.rr[q] = t[3 * q];
+          S.bb[q] = t[3 * q + 1];
+          S.rho[q] = t[3 * q + 2];
+          S.half[q] = 0;
+          if (!isfinite(S.rr[q])) S.status = 2;
+          S.active[q] = isfinite(S.rr[q]) && S.rr[q] > a.tol2 * S.bb[q] && S.rho[q] != 0.0;
+          S.go |= S.active[q];
+        }
+        if (a.maxit - S.total <= 0) S.go = 0;
+      });
+      if (!ok) return give_up(a);
+    }
+    bool run = S.go != 0;
+    while (run) {
+      {  // v = H p; (rh, v)
+        double d[2] = {};
+        for (int i = r0 + tid; i < r1; i += kVT) {
+          double y[2];
+          v_row<K>(a, i, a.p, y);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            a.v[q][i] = y[q];
+            d[q] += a.rh[q][i] * y[q];
+          }
+        }
+        const bool ok = g.template reduce<2>(d, active, [&](const double* t) {
+          for (int q = 0; q < 2; ++q) {
+            if (!S.active[q]) continue;
+            if (t[q] == 0.0 || !isfinite(t[q])) {
+              S.active[q] = 0;
+              S.status = isfinite(t[q]) ? 1 : 2;
+            } else {
+              S.alpha[q] = quot(S.rho[q], t[q]);
+            }
+          }
+        });
+        if (!ok) return give_up(a);
+      }
+      {  // s = r - alpha v; (s, s), (rh, s)
+        double d[4] = {};
+        const double al[2] = {S.alpha[0], S.alpha[1]};
+        const bool act[2] = {S.active[0] != 0, S.active[1] != 0};
+        for (int i = r0 + tid; i < r1; i += kVT) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            if (!act[q]) continue;
+            const double si = a.r[q][i] - al[q] * a.v[q][i];
+            a.s[q][i] = si;
+            d[q] += si * si;
+            d[2 + q] += a.rh[q][i] * si;
+          }
+        }
+        const bool ok = g.template reduce<4>(d, active, [&](const double* t) {
+          S.iterate = 0;
+          for (int q = 0; q < 2; ++q) {
+            if (!S.active[q]) continue;
+            S.half[q] = t[q] <= a.tol2 * S.bb[q];
+            S.rhs[q] = t[2 + q];
+            if (S.half[q])
+              S.rr[q] = t[q];
+            else
+              S.iterate = 1;
+          }
+        });
+        if (!ok) return give_up(a);
+      }
+      if (S.iterate) {  // t = H s; (t, s), (t, t), (rh, t)
+        double d[6] = {};
+        for (int i = r0 + tid; i < r1; i += kVT) {
+          double y[2];
+          v_row<K>(a, i, a.s, y);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            a.t[q][i] = y[q];
+            d[3 * q] += y[q] * a.s[q][i];
+            d[3 * q + 1] += y[q] * y[q];
+            d[3 * q + 2] += a.rh[q][i] * y[q];
+          }
+        }
+        const bool ok = g.template reduce<6>(d, active, [&](const double* t) {
+          for (int q = 0; q < 2; ++q) {
+            if (!S.active[q] || S.half[q]) continue;
+            const double ts = t[3 * q], tt = t[3 * q + 1];
+            if (!(tt > 0.0) || !isfinite(ts)) {
+              S.active[q] = 0;
+              S.status = isfinite(tt) ? 3 : 2;
+              continue;
+            }
+            const double om = quot(ts, tt), rn = S.rhs[q] - om * t[3 * q + 2];
+            S.beta[q] = quot(rn, S.rho[q]) * quot(S.alpha[q], om);
+            S.omega[q] = om;
+            S.rho[q] = rn;
+          }
+        });
+        if (!ok) return give_up(a);
+      }
+      {  // x, r, p; (r, r)
+        double d[2] = {};
+        const double al[2] = {S.alpha[0], S.alpha[1]}, om[2] = {S.omega[0], S.omega[1]},
+                     be[2] = {S.beta[0], S.beta[1]};
+        const bool act[2] = {S.active[0] != 0, S.active[1] != 0};
+        const bool hf[2] = {S.half[0] != 0, S.half[1] != 0};
+        for (int i = r0 + tid; i < r1; i += kVT) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            if (!act[q]) continue;
+            const double pi = a.p[q][i], si = a.s[q][i];
+            if (hf[q]) {
+              a.x[q][i] += al[q] * pi;
+              d[q] += si * si;
+              continue;
+            }
+            a.x[q][i] += al[q] * pi + om[q] * si;
+            const double ri = si - om[q] * a.t[q][i];
+            a.r[q][i] = ri;
+            a.p[q][i] = ri + be[q] * (pi - om[q] * a.v[q][i]);
+            d[q] += ri * ri;
+          }
+        }
+        const bool ok = g.template reduce<2>(d, active, [&](const double* t) {
+          S.iters += 1;
+          int any = 0;
+          for (int q = 0; q < 2; ++q) {
+            if (!S.active[q]) continue;
+            S.rr[q] = t[q];
+            S.active[q] = 0;
+            if (!isfinite(t[q]))
+              S.status = 2;
+            else if (t[q] > 1e8 * S.bb[q] && S.bb[q] > 0.0)
+              S.status = 5;
+            else if (S.half[q] || t[q] <= a.tol2 * S.bb[q])
+              ;
+            else if (S.rho[q] == 0.0 || S.omega[q] == 0.0)
+              S.status = 4;
+            else
+              any = S.active[q] = 1;
+          }
+          S.go = any && S.total + S.iters < a.maxit;
+        });
+        if (!ok) return give_up(a);
+      }
+      run = S.go != 0;
+    }
+    bool conv = true, near = true;
+    for (int q = 0; q < 2; ++q) {
+      conv = conv && S.rr[q] <= a.tol2 * S.bb[q];
+      near = near && S.rr[q] <= a.accept2 * S.bb[q];
+    }
+    const int st = S.status, tot = S.total + S.iters;
+    const bool again = st == 1 || st == 3 || st == 4 || st == 5;
+    __syncthreads();
+    if (tid == 0) S.total = tot;
+    if (conv || !again || tot >= a.maxit || cyc >= 400) {
+      if (blockIdx.x == 0 && tid == 0) {
+        double worst = 0.0;
+        for (int q = 0; q < 2; ++q)
+          worst = fmax(worst, S.bb[q] > 0 ? sqrt(S.rr[q] / S.bb[q]) : sqrt(S.rr[q]));
+        a.res->iters = tot;
+        a.res->status = st;
+        a.res->relres = worst;
+        a.res->converged = conv;
+        if (st == 2 || (!conv && !near)) *a.fail = (a.step << 4) | kFailViscous;
+      }
+      return leave(a.arrivals);
+    }
+    if (st == 5)  // the recurrence has blown up: start again from the initial iterate
+      for (int i = r0 + tid; i < r1; i += kVT)
+        for (int q = 0; q < 2; ++q) a.x[q][i] = a.x0[q][i];
+    // the residual of the restart reads x of other blocks
+    if (!g.sync()) return give_up(a);
   }
 }
 
 }  // namespace
+
+struct VSolve {
+  std::vector<void*> allocs;
+  int grid = 0;
+  VArgs a{};
+};
+
+void vsolve_free(VSolve* v) {
+  if (!v) return;
+  for (void* q : v->allocs) cudaFree(q);
+  delete v;
+}
+
+int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* idx,
+                 const double* wu, const double* wv, VSolve** out, cudaStream_t st) {
+  *out = nullptr;
+  VSolve* v = new VSolve();
+  v->grid = sm_count();
+  VArgs& a = v->a;
+  a.N = (int)N;
+  a.rows = (int)((N + v->grid - 1) / v->grid);
+  a.k = k;
+  a.ld = ld;
+  a.idx = idx;
+  a.w[0] = wu;
+  a.w[1] = wv;
+  auto get = [&](void** p, size_t bytes) {
+    int rc = check_cuda(ctx, cudaMalloc(p, bytes), "viscous solve alloc");
+    if (rc) return rc;
+    v->allocs.push_back(*p);
+    return check_cuda(ctx, cudaMemsetAsync(*p, 0, bytes, st), "memset");
+  };
+  int rc = 0;
+  for (int q = 0; q < 2 && !rc; ++q) {
+    double** vec[] = {&a.r[q], &a.rh[q], &a.p[q], &a.v[q], &a.s[q], &a.t[q], &a.x0[q]};
+    for (double** p : vec)
+      if (!rc) rc = get((void**)p, sizeof(double) * N);
+  }
+  if (!rc) rc = get((void**)&a.partials, sizeof(double) * 2 * kVNV * v->grid);
+  if (!rc) rc = get((void**)&a.arrivals, 2 * sizeof(unsigned int));
+  if (rc) {
+    cudaStreamSynchronize(st);
+    vsolve_free(v);
+    return rc;
+  }
+  *out = v;
+  return RBFFD_OK;
+}
+
+cudaError_t vsolve_enqueue(VSolve* v, double* const* x, const double* const* b, double tol,
+                           double accept, int maxit, PSolveResult* res, int* fail, int step,
+                           cudaStream_t st) {
+  VArgs a = v->a;
+  for (int q = 0; q < 2; ++q) {
+    a.x[q] = x[q];
+    a.b[q] = b[q];
+  }
+  a.tol2 = tol * tol;
+  a.accept2 = accept * accept;
+  a.maxit = maxit;
+  a.res = res;
+  a.fail = fail;
+  a.step = step;
+  const void* fn = a.k == 28 ? (const void*)k_vsolve<28> : (const void*)k_vsolve<0>;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel(fn, dim3(v->grid), dim3(kVT), args, 0, st);
+}
 
 struct DSolve {
   std::vector<void*> allocs;
@@ -356,7 +696,7 @@ int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   if (!rc) rc = d_alloc(ctx, d, &in.cand_r, (size_t)2 * d->grid, st);
   if (!rc) rc = d_alloc(ctx, d, &in.status, 1, st);
   if (!rc) rc = d_alloc(ctx, d, &a.partials, (size_t)2 * kNVMax * d->grid, st);
-  if (!rc) rc = d_alloc(ctx, d, &a.arrivals, 1, st);
+  if (!rc) rc = d_alloc(ctx, d, &a.arrivals, 2, st);
   if (!rc) rc = d_alloc(ctx, d, &a.res, 1, st);
   if (!rc) rc = d_alloc(ctx, d, &a.r, (size_t)a.ldt, st);
   in.partials = a.partials;
@@ -379,20 +719,35 @@ int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   return RBFFD_OK;
 }
 
-int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
-               PSolveResult* res, int64_t* launches, cudaStream_t st) {
+cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PSolveResult* res,
+                           int* fail, int step, cudaStream_t st) {
   DArgs a = d->a;
   a.x = x;
   a.b = b;
   a.tol2 = tol * tol;
-  PSolveResult* h = (PSolveResult*)ctx->host_pinned;
-  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, sizeof(unsigned int), st), "memset");
-  if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
-  if (rc) return rc;
+  a.res = res;
+  a.fail = fail;
+  a.step = step;
   const void* fn = a.k == 28 ? (const void*)k_dsolve<28> : (const void*)k_dsolve<0>;
   void* args[] = {&a};
-  rc = check_cuda(ctx, cudaLaunchCooperativeKernel(fn, dim3(d->grid), dim3(kPT), args, 0, st),
-                  "direct pressure solve");
+  return cudaLaunchCooperativeKernel(fn, dim3(d->grid), dim3(kPT), args, 0, st);
+}
+
+cudaError_t small_reset(VSolve* v, DSolve* d, int* fail, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(v->a.arrivals, 0, 2 * sizeof(unsigned int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d->a.arrivals, 0, 2 * sizeof(unsigned int), st);
+  return e == cudaSuccess ? cudaMemsetAsync(fail, 0, sizeof(int), st) : e;
+}
+
+int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
+               PSolveResult* res, int64_t* launches, cudaStream_t st) {
+  PSolveResult* h = (PSolveResult*)ctx->host_pinned;
+  const DArgs& a = d->a;
+  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, 2 * sizeof(unsigned int), st), "memset");
+  if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
+  if (!rc)
+    rc = check_cuda(ctx, dsolve_enqueue(d, x, b, tol, a.res, nullptr, 0, st),
+                    "direct pressure solve");
   if (!rc)
     rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(PSolveResult), cudaMemcpyDeviceToHost, st),
                     "direct solve result");

@@ -94,6 +94,16 @@ struct Grid {
   }
 };
 
+// Ends a kernel whose arrival counter (two words) the next launch finds at
+// zero again: the last block to come here resets it.
+__device__ __forceinline__ void leave(unsigned int* arrivals) {
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(arrivals + 1, 1u) == gridDim.x - 1u) {
+    arrivals[0] = 0u;
+    arrivals[1] = 0u;
+  }
+}
+
 // a / b for the scalars of a solve (one thread's work, which every block waits
 // for): the approximate reciprocal instruction and two steps of Newton's
 // iteration for 1 / b, a shorter serial chain than a correctly rounded

@@ -62,4 +62,29 @@ void dsolve_free(DSolve* d);
 int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
                PSolveResult* res, int64_t* launches, cudaStream_t st);
 
+// The viscous systems of a small flow, both components in one resident kernel:
+// BiCGSTAB on x + w x = b with the component's weights wu or wv (the same
+// pointer in a closed flow) on shared indices.
+struct VSolve;
+int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* idx,
+                 const double* wu, const double* wv, VSolve** out, cudaStream_t st);
+void vsolve_free(VSolve* v);
+
+// The two solves of a small flow's step, enqueued without waiting for their
+// results, so that the host can run steps ahead of the GPU.  `fail` (device)
+// is 0 or what ended an earlier step: then nothing is done.  A solve that
+// misses its tolerance sets it to (step << 4) | kFail*.  *res (device) gets
+// the result.  small_reset before a run of steps.
+constexpr int kFailViscous = 1, kFailPressure = 2, kFailWait = 3;
+struct SmallStep {
+  PSolveResult visc, pres;
+};
+cudaError_t small_reset(VSolve* v, DSolve* d, int* fail, cudaStream_t st);
+// accept: a relative residual up to which a viscous solve short of tol passes
+cudaError_t vsolve_enqueue(VSolve* v, double* const* x, const double* const* b, double tol,
+                           double accept, int maxit, PSolveResult* res, int* fail, int step,
+                           cudaStream_t st);
+cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PSolveResult* res,
+                           int* fail, int step, cudaStream_t st);
+
 }  // namespace rbffd

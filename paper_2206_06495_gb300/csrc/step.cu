@@ -1289,7 +1289,9 @@ constexpr int kMaxHist = 3;  // cubic: measured best on the 1M cavity (8.9 itera
 struct History {
   double* h[kMaxHist];
 };
-__global__ void k_extrapolate(int64_t n, int ord, double* __restrict__ x, History H) {
+__global__ void k_extrapolate(int64_t n, int ord, double* __restrict__ x, History H,
+                              const int* skip) {
+  if (skip && *skip) return;
   double c[kMaxHist + 1];
   double b = ord + 1.0;  // C(ord + 1, k + 1) with alternating signs
   for (int k = 0; k <= ord; ++k) {
@@ -1368,11 +1370,15 @@ struct ConvArgs {
   float2 *us2, *vs2;
   double dt;
   int first;
+  // null, or a flag that an earlier step of a run enqueued ahead of the GPU
+  // has failed: the state then stays at the last completed step
+  const int* skip;
 };
 
 // Stage 1: C_j(q) = -[u o D_x q + v o D_y q]; u* = u_j + dt (3/2 C_j - 1/2 C_{j-1})
 template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_convect(ConvArgs a) {
+  if (a.skip && *a.skip) return;
   const void* w[2] = {a.wdx, a.wdy};
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
        i += (int64_t)gridDim.x * kThreads) {
@@ -1427,6 +1433,7 @@ struct HelmRhsArgs {
   double vc[kMaxHist + 1] = {};
   double* hu[kMaxHist] = {};
   double* hv[kMaxHist] = {};
+  const int* skip = nullptr;  // as in ConvArgs
 };
 
 // Stage 2 right side: u* + a D_Lap (u* or u_j) inside, minus dt G0 p~_j for
@@ -1434,6 +1441,7 @@ struct HelmRhsArgs {
 // projection, the Kim & Moin term
 template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_helm_rhs(HelmRhsArgs a) {
+  if (a.skip && *a.skip) return;
   const void* wl[1] = {a.lap};
   const void* wg[2] = {a.vp_dx, a.vp_dy};
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
@@ -1511,12 +1519,14 @@ struct DivArgs {
   double inv_dt;
   double* b;
   int proj;  // exact projection: every row is a divergence row
+  const int* skip;
 };
 
 // Stage 3a: F = D^(P,V)_x u** + D^(P,V)_y v**; scaled Poisson right side
 // (0 on the Neumann rows of the paper's projection)
 template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_divergence(DivArgs a) {
+  if (a.skip && *a.skip) return;
   const void* wx[1] = {a.wdx};
   const void* wy[1] = {a.wdy};
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
@@ -1541,6 +1551,7 @@ struct PresArgs {
   float2* pt2;
   int proj;
   int nomean;  // Dirichlet pressure rows: p~ = x, no shift to mean zero
+  const int* skip;
 };
 
 // Stage 3c: p~ = x - mean(x); p = p~ - a D^(P,P)_Lap p~.  Exact projection:
@@ -1548,6 +1559,7 @@ struct PresArgs {
 // (D_Lap annihilates constants, so it is applied to x).
 template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_pressure(PresArgs a) {
+  if (a.skip && *a.skip) return;
   const void* wl[1] = {a.lap};
   const double mean = a.nomean ? 0.0 : *a.sum / (double)a.n;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
@@ -1580,12 +1592,14 @@ struct CorrArgs {
   int proj;
   const double *sum, *esn, *v_nx, *v_ny;
   const uint8_t *bcu, *bcv;  // open flows: only Dirichlet components are overwritten
+  const int* skip;
 };
 
 // Stage 3d: u_{j+1} = u** - dt D^(V,P)_x p~ (Eq. velocity_next_timestep).
 // Exact projection: u_{j+1} = u** - dt G0 phi - c w.
 template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_correct(CorrArgs a) {
+  if (a.skip && *a.skip) return;
   const void* w[2] = {a.wdx, a.wdy};
   const double c = a.proj ? -a.dt * (*a.sum) / (*a.esn) : 0.0;
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
@@ -1877,6 +1891,9 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// Steps of a small flow enqueued before the host looks at their results.
+constexpr int kSmallBatch = 32;
+
 struct StepPlan {
   rbffd_flow key;
   int k = 0;
@@ -1920,6 +1937,9 @@ struct StepPlan {
   double* dscal = nullptr;  // [0]: sum, [1..6]: residual norms
   struct AdjointPlan* adj = nullptr;  // transposed operators, built on first use
   Amg* amg = nullptr;                 // pressure preconditioner (precond = 1)
+  VSolve* vis = nullptr;              // small FP64 flows: the resident viscous solve
+  int* fail = nullptr;                // and the run's failure word and results (SmallStep)
+  SmallStep* small = nullptr;
   PSolve* ps = nullptr;               // the preconditioned solve's resident kernel
   DSolve* ds = nullptr;               // small systems: the direct solve (amg and ps are then
                                       // built when something needs the Krylov solve)
@@ -1971,6 +1991,7 @@ void step_plan_free(StepPlan* p) {
   adjoint_plan_free(p->adj);
   psolve_free(p->ps);
   dsolve_free(p->ds);
+  vsolve_free(p->vis);
   amg_free(p->amg);
   for (auto& g : p->graphs) cudaGraphExecDestroy(g.exec);
   if (p->cap) cudaStreamDestroy(p->cap);
@@ -2258,6 +2279,12 @@ int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t
       TRY(dsolve_build(ctx, f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->es, &p->ds, st));
     }
     if (!p->ds) TRY(build_precond(ctx, p, f, hd, hes, st));
+    if (p->ds && !p->mix && f.N <= 2 * kDenseMax) {
+      TRY(vsolve_build(ctx, f.N, f.ld_v, p->k, p->open ? p->Hidx : f.vv_idx, p->Hw,
+                       p->open ? p->Hw_v : p->Hw, &p->vis, st));
+      TRY(palloc(ctx, p, &p->fail, 1));
+      TRY(palloc(ctx, p, &p->small, kSmallBatch));
+    }
   }
 #undef TRY
   *out = p;
@@ -2978,16 +3005,20 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   KOp<float, float> Hv32{P->Hidx, P->Hw32_v, f.ld_v, f.N, k, 1, nullptr, nullptr};
   (MIX ? Hu32.tiles : Hu64.tiles) = P->Ht;
   (MIX ? Hv32.tiles : Hv64.tiles) = P->Ht_v;
-  for (int32_t step = 0; step < n_steps; ++step) {
+  const int GN = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.N + kThreads - 1) / kThreads));
+  const int GM = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.M + kThreads - 1) / kThreads));
+  // Stages 1 and 2 up to the viscous right side and initial guess.
+  auto front = [&](const int* skip) -> int {
     ConvArgs ca{f.N,  f.ld_v,       k,  f.vv_idx, vdx, vdy,   s->u,  s->v,  P->u2,
                 P->v2, s->cu_prev, s->cv_prev, P->us, P->vs, P->us2, P->vs2, f.dt,
-                s->j == 0 ? 1 : 0};
-    k_convect<K, MIX><<<G, kThreads, 0, st>>>(ca);
+                s->j == 0 ? 1 : 0, skip};
+    k_convect<K, MIX><<<GN, kThreads, 0, st>>>(ca);
     HelmRhsArgs ha{f.N,    f.ld_v, k,      f.vv_idx, vlap,   P->us,  P->vs,  P->us2,
                    P->vs2, f.vp_idx, gdx,  gdy,      s->pt,  P->pt2, f.v_bc, f.v_nx,
                    f.v_ny, gu,     gv,     a,        f.dt,   f.km_mode, P->ru, P->rv,
                    P->uss, P->vss, s->u,   s->v,     P->u2,  P->v2, f.cn_form, P->proj,
                    f.v_bcu, f.v_bcv};
+    ha.skip = skip;
     // the viscous solves start from the extrapolation of the previous steps'
     // solutions when this plan made them (P->px_step == s->j), as the
     // pressure solve does
@@ -3007,14 +3038,17 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     } else {
       P->vhist = 0;
     }
-    k_helm_rhs<K, MIX><<<G, kThreads, 0, st>>>(ha);
+    k_helm_rhs<K, MIX><<<GN, kThreads, 0, st>>>(ha);
     P->launches += 2 + (MIX ? 2 : 0) + 4 + (MIX ? 1 : 0);  // stage kernels of this step
-    int rc = check_cuda(ctx, cudaGetLastError(), "stage 1-2 kernels");
-    if (rc) return rc;
-    double* hx[2] = {P->uss, P->vss};
-    const double* hb[2] = {P->ru, P->rv};
+    return check_cuda(ctx, cudaGetLastError(), "stage 1-2 kernels");
+  };
+  // The viscous solves, launch by launch.
+  const double vtol = (MIX || P->open || f.tol < 1e-13) ? f.tol : std::max(f.tol * 1e-3, 1e-13);
+  double* hx[2] = {P->uss, P->vss};
+  const double* hb[2] = {P->ru, P->rv};
+  auto viscous = [&]() -> int {
+    int rc = 0, sweeps = 0;
     SolveResult hr;
-    int sweeps = 0;
     // The viscous operator is well conditioned: its FP32 inner solves go to the
     // square of the inner tolerance (each FP64 residual of the 3M-row, two-sided
     // solve costs more than a few extra FP32 iterations).
@@ -3026,7 +3060,6 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     // of it, each viscous solve 2 iterations from its extrapolated guess).  In
     // MIXED precision a tighter viscous target measured no gain (33.7 pressure
     // iterations per step at 1e-12), so the tolerance stays.
-    const double vtol = (MIX || P->open || f.tol < 1e-13) ? f.tol : std::max(f.tol * 1e-3, 1e-13);
     if (P->open) {
       // per-component operators: one solve each
       SolveResult h2[2];
@@ -3067,6 +3100,11 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       return set_error(ctx, RBFFD_ERR_NOT_CONVERGED,
                        "viscous solve: relative residual %.3e after %d iterations (status %d)",
                        hr.relres, hr.iters, hr.status);
+    return RBFFD_OK;
+  };
+  // The pressure right side and initial guess.
+  auto pressure_input = [&](const int* skip) -> int {
+    int rc = 0;
     if (MIX) {
       k_split<<<G, kThreads, 0, st>>>(f.N, P->uss, P->uss2);
       k_split<<<G, kThreads, 0, st>>>(f.N, P->vss, P->vss2);
@@ -3075,8 +3113,9 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     // FP32 weights would leave their rounding (relative to the terms, not to
     // their small sum) in p~, so both precisions take it with FP64 weights.
     DivArgs da{f.M,    f.ld_p,  k,      f.pv_idx, f.pv_dx,  f.pv_dy,      P->uss,
-               P->vss, P->uss2, P->vss2, f.p_bc,  P->scale, 1.0 / f.dt, P->pb, P->proj};
-    k_divergence<K, false><<<G, kThreads, 0, st>>>(da);
+               P->vss, P->uss2, P->vss2, f.p_bc,  P->scale, 1.0 / f.dt, P->pb, P->proj,
+               skip};
+    k_divergence<K, false><<<GM, kThreads, 0, st>>>(da);
     // Initial guess: the extrapolation in time through the previous steps'
     // solutions (up to cubic), else the state's p~.  Any guess
     // leaves the converged solution the same; a better one saves iterations
@@ -3093,17 +3132,141 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       const int ord = std::min(P->nhist, kMaxHist);
       History H;
       for (int q = 0; q < kMaxHist; ++q) H.h[q] = P->pxh[(P->hhead + q) % kMaxHist];
-      k_extrapolate<<<G, kThreads, 0, st>>>(f.M, ord, P->px, H);
+      k_extrapolate<<<GM, kThreads, 0, st>>>(f.M, ord, P->px, H, skip);
       rc = check_cuda(ctx, cudaGetLastError(), "extrapolation");
       if (rc) return rc;
       P->hhead = (P->hhead + kMaxHist - 1) % kMaxHist;  // the recycled slot is the newest
       P->nhist = std::min(P->nhist + 1, kMaxHist);
     }
+    return rc;
+  };
+  // Stage 3 after the pressure solve.
+  auto back = [&](const int* skip) -> int {
+    k_sum<double><<<GM, kThreads, 0, st>>>(P->px, f.M, P->gr, P->dscal);
+    if (MIX) k_split<<<G, kThreads, 0, st>>>(f.M, P->px, P->px2);
+    PresArgs pa{f.M,   f.ld_p, k,    f.pp_idx, plap,   P->px,  P->px2,
+                P->dscal, a,   s->pt, s->p, P->pt2,   P->proj, P->pdir > 0 ? 1 : 0, skip};
+    k_pressure<K, MIX><<<GM, kThreads, 0, st>>>(pa);
+    // The exact projection corrects with G0 x (x = phi + const) and the wall
+    // flux, with FP64 weights in both precisions (like the divergence), so
+    // that D^(P,V) u_{j+1} vanishes to the solve's accuracy.
+    CorrArgs ka{f.N,      f.ld_v, k,        f.vp_idx,       proj ? f.vp_dx : gdx,
+                proj ? f.vp_dy : gdy,       proj ? P->px : s->pt,   proj ? P->px2 : P->pt2,
+                P->uss,   P->vss, f.v_bc,   gu,             gv,   f.dt,
+                f.overwrite_bc,   s->u,     s->v,           P->u2, P->v2,
+                P->proj,  P->dscal, P->esn, f.v_nx,         f.v_ny,
+                f.v_bcu,  f.v_bcv, skip};
+    if (proj && MIX) {
+      k_correct<K, false><<<GN, kThreads, 0, st>>>(ka);
+      k_split<<<G, kThreads, 0, st>>>(f.N, s->u, P->u2);
+      k_split<<<G, kThreads, 0, st>>>(f.N, s->v, P->v2);
+    } else {
+      k_correct<K, MIX><<<GN, kThreads, 0, st>>>(ka);
+    }
+    return check_cuda(ctx, cudaGetLastError(), "stage 3 kernels");
+  };
+  // A small FP64 flow's solves decide on the GPU, so its steps are enqueued
+  // ahead, up to kSmallBatch at a time, and the host waits once for all of
+  // them; a wait after each solve was half of a 1,600-node step.  A step whose
+  // solve fails turns what follows into no-ops; the host takes its own
+  // bookkeeping back to that step and goes on with the launch by launch solve.
+  const bool ahead = !MIX && direct && P->vis;
+  struct Mark {
+    int64_t j, px_step;
+    int vhead, vhist, hhead[2], nhist[2];  // [1]: after the pressure guess
+  };
+  // kFail* of a step enqueued ahead whose solve missed its tolerance: what came
+  // before that solve stands, and the launch by launch one starts from its iterate
+  int resume = 0;
+  for (int32_t step = 0; step < n_steps;) {
+    if (ahead && !resume) {
+      const int batch = std::min<int32_t>(n_steps - step, kSmallBatch);
+      Mark marks[kSmallBatch];
+      int rc = check_cuda(ctx, small_reset(P->vis, P->ds, P->fail, st), "step reset");
+      for (int i = 0; i < batch && !rc; ++i) {
+        Mark& m = marks[i];
+        m.j = s->j;
+        m.px_step = P->px_step;
+        rc = front(P->fail);
+        m.vhead = P->vhead;
+        m.vhist = P->vhist;
+        m.hhead[0] = P->hhead;
+        m.nhist[0] = P->nhist;
+        if (!rc)
+          rc = check_cuda(ctx, vsolve_enqueue(P->vis, hx, hb, vtol, f.tol, f.max_iter,
+                                              &P->small[i].visc, P->fail, i, st),
+                          "viscous solve");
+        if (!rc) rc = pressure_input(P->fail);
+        m.hhead[1] = P->hhead;
+        m.nhist[1] = P->nhist;
+        if (!rc)
+          rc = check_cuda(ctx, dsolve_enqueue(P->ds, P->px, P->pb, f.tol, &P->small[i].pres,
+                                              P->fail, i, st),
+                          "direct pressure solve");
+        if (!rc) rc = back(P->fail);
+        P->launches += 2;
+        s->j += 1;
+        P->px_step = s->j;
+      }
+      SmallStep* h = (SmallStep*)ctx->host_pinned;
+      int* hf = (int*)(h + kSmallBatch);
+      if (!rc)
+        rc = check_cuda(ctx, cudaMemcpyAsync(h, P->small, sizeof(SmallStep) * batch,
+                                             cudaMemcpyDeviceToHost, st),
+                        "step results");
+      if (!rc)
+        rc = check_cuda(ctx, cudaMemcpyAsync(hf, P->fail, sizeof(int), cudaMemcpyDeviceToHost, st),
+                        "step results");
+      if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "step sync");
+      if (rc) return rc;
+      const int code = *hf & 15, bad = code ? *hf >> 4 : batch;
+      for (int i = 0; i < batch && i <= bad; ++i) {
+        if (stats && (i < bad || code == kFailPressure)) {
+          stats->helm_iters += h[i].visc.iters;
+          stats->helm_relres = h[i].visc.relres;
+        }
+        if (stats && (i < bad || code == kFailPressure)) {
+          stats->poisson_iters += h[i].pres.iters;
+          stats->poisson_relres = h[i].pres.relres;
+        }
+        if (stats && i < bad) stats->steps += 1;
+        if (trace_on())
+          fprintf(stderr, "[rbffd] small step: viscous %d its %.3e, pressure %d products %.3e\n",
+                  h[i].visc.iters, h[i].visc.relres, h[i].pres.iters, h[i].pres.relres);
+      }
+      step += bad;
+      if (!code) continue;
+      const Mark& m = marks[bad];
+      const int after = code == kFailPressure ? 1 : 0;
+      s->j = m.j;
+      P->px_step = m.px_step;
+      P->vhead = m.vhead;
+      P->vhist = m.vhist;
+      P->hhead = m.hhead[after];
+      P->nhist = m.nhist[after];
+      if (code == kFailWait)
+        return set_error(ctx, RBFFD_ERR_CUDA, "small solve: grid barrier not reached (bounded wait)");
+      if (code == kFailPressure && h[bad].pres.status == 2)
+        return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite pressure solve");
+      if (code == kFailPressure)  // refinement at its rounding level above the tolerance
+        rc = need_precond(ctx, P, f, st);
+      else if (h[bad].visc.status == 2)
+        for (double* x : hx)
+          if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(x, 0, sizeof(double) * f.N, st), "zero start");
+      if (rc) return rc;
+      resume = code;
+      continue;
+    }
+    int rc = 0, sweeps = 0;
+    if (!resume) rc = front(nullptr);
+    if (!rc && resume != kFailPressure) rc = viscous();
+    if (!rc && resume != kFailPressure) rc = pressure_input(nullptr);
+    if (rc) return rc;
     double* px[1] = {P->px};
     const double* pbv[1] = {P->pb};
     SolveResult pr;
     const bool prof = f.profile != 0;
-    if (direct) {
+    if (direct && !resume) {
       PSolveResult dr;
       rc = dsolve_run(ctx, P->ds, P->px, P->pb, f.tol, &dr, &P->launches, st);
       if (rc) return rc;
@@ -3116,7 +3279,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       if (!pr.converged && pr.status != 2) rc = need_precond(ctx, P, f, st);
       if (rc) return rc;
     }
-    if (direct && (pr.converged || pr.status == 2)) {
+    if (direct && !resume && (pr.converged || pr.status == 2)) {
     } else if (proj) {  // the composed operator's rows are read directly (runtime width)
       if (MIX)
         rc = refine<0, 1, true>(ctx, P, L64, L32, px, pbv, f.tol, f.inner_tol, f.max_iter, &pr,
@@ -3146,32 +3309,13 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       return set_error(ctx, RBFFD_ERR_NOT_CONVERGED,
                        "pressure solve: relative residual %.3e after %d iterations (status %d)",
                        pr.relres, pr.iters, pr.status);
-    k_sum<double><<<G, kThreads, 0, st>>>(P->px, f.M, P->gr, P->dscal);
-    if (MIX) k_split<<<G, kThreads, 0, st>>>(f.M, P->px, P->px2);
-    PresArgs pa{f.M,   f.ld_p, k,    f.pp_idx, plap,   P->px,  P->px2,
-                P->dscal, a,   s->pt, s->p, P->pt2,   P->proj, P->pdir > 0 ? 1 : 0};
-    k_pressure<K, MIX><<<G, kThreads, 0, st>>>(pa);
-    // The exact projection corrects with G0 x (x = phi + const) and the wall
-    // flux, with FP64 weights in both precisions (like the divergence), so
-    // that D^(P,V) u_{j+1} vanishes to the solve's accuracy.
-    CorrArgs ka{f.N,      f.ld_v, k,        f.vp_idx,       proj ? f.vp_dx : gdx,
-                proj ? f.vp_dy : gdy,       proj ? P->px : s->pt,   proj ? P->px2 : P->pt2,
-                P->uss,   P->vss, f.v_bc,   gu,             gv,   f.dt,
-                f.overwrite_bc,   s->u,     s->v,           P->u2, P->v2,
-                P->proj,  P->dscal, P->esn, f.v_nx,         f.v_ny,
-                f.v_bcu,  f.v_bcv};
-    if (proj && MIX) {
-      k_correct<K, false><<<G, kThreads, 0, st>>>(ka);
-      k_split<<<G, kThreads, 0, st>>>(f.N, s->u, P->u2);
-      k_split<<<G, kThreads, 0, st>>>(f.N, s->v, P->v2);
-    } else {
-      k_correct<K, MIX><<<G, kThreads, 0, st>>>(ka);
-    }
-    rc = check_cuda(ctx, cudaGetLastError(), "stage 3 kernels");
+    rc = back(nullptr);
     if (rc) return rc;
+    resume = 0;
     s->j += 1;
     P->px_step = s->j;
     if (stats) stats->steps += 1;
+    ++step;
   }
   int rc = check_cuda(ctx, cudaStreamSynchronize(st), "step sync");
   if (stats && proj && n_steps > 0 && !rc) {
