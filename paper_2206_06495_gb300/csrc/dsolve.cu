@@ -52,9 +52,9 @@ struct InvArgs {
 // rescales it while it applies step k + 1.
 //
 // What bounds it: n^2 FP64 FMAs and one pass over the matrix (in L2 up to about
-// n = 3,500) per step: 6 us a step at n = 1,600 and 13 us at 2,700, of which
-// the barrier and the pivot search are 4 us.  A blocked form would save memory
-// traffic, not FP64 instructions, which are the larger part on this GPU.
+// n = 3,500) per step, 4.1 us for the FMAs at n = 1,600, and the barrier and the
+// pivot search.  A blocked form would save memory traffic, not FP64
+// instructions.
 __global__ void __launch_bounds__(kPT, 1) k_dense_invert(const __grid_constant__ InvArgs a) {
   __shared__ double sh[kNVMax * kPT];
   __shared__ double part[kNVMax * 4];
@@ -284,6 +284,12 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
 
 // ---------------------------------------------------------- viscous solves
 constexpr int kVT = 512;  // threads per block
+constexpr int kVL = 4;    // threads per row
+// Rows of a block, where there are SMs for so few: fewer blocks make the
+// barrier lighter, fewer rows the phases (8, 16, 32, 64 rows: 20 steps of 1,600
+// nodes 5.67, 5.69, 5.63, 5.57 ms, four of the 2,700-node wake 1.47, 1.45, 1.44,
+// 1.49).
+constexpr int kVRows = 32;
 constexpr int kVNV = 6;
 
 struct VArgs {
@@ -293,7 +299,7 @@ struct VArgs {
   const double* w[2];
   double* x[2];
   const double* b[2];
-  double *r[2], *rh[2], *p[2], *v[2], *s[2], *t[2], *x0[2];
+  double *p, *s;  // [N][2], both components side by side
   double tol2, accept2;
   int maxit;
   double* partials;        // [2][kVNV][gridDim.x]
@@ -304,74 +310,103 @@ struct VArgs {
 };
 
 struct VScal {
-  double rho[2], rr[2], bb[2], rhs[2], alpha[2], omega[2], beta[2];
-  int active[2], half[2], status, iters, total, go, iterate;
+  double rho[2], rr[2], ss[2], bb[2], rhs[2], alpha[2], omega[2], beta[2];
+  int active[2], mode[2], status, iters, total, go, iterate;
 };
 
-// y_q = x_q + sum_s w_q,s x_q,j of row i
-template <int K>
-__device__ __forceinline__ void v_row(const VArgs& a, int i, double* const* x, double (&y)[2]) {
-  const bool same = a.w[0] == a.w[1];
-  double s0 = 0.0, s1 = 0.0;
-#pragma unroll(K > 0 ? K : 4)
-  for (int s = 0; s < (K > 0 ? K : a.k); ++s) {
-    const int j = __ldg(a.idx + s * a.ld + i);
-    const double w0 = __ldg(a.w[0] + s * a.ld + i);
-    const double w1 = same ? w0 : __ldg(a.w[1] + s * a.ld + i);
-    s0 += w0 * x[0][j];
-    s1 += w1 * x[1][j];
-  }
-  y[0] = s0 + x[0][i];
-  y[1] = s1 + x[1][i];
-}
-
-// What bounds it: latency, four phases an iteration of about 5 us each.  As
-// separate launches an iteration took five kernels of 1,216 blocks (75 us with
-// cold caches at 4,641 rows) and the solve two or three waits of the host.
-// (rh, r) = (rh, s) - omega (rh, t), so x, r and p are one pass.  A component
-// that has converged keeps its x while the other one goes on.
+// What bounds it: latency, four phases an iteration (a barrier of 1.3 us, the
+// reduction behind it, one gather from L2): 170 us with cold caches for the 6.5
+// iterations of a solve at 1,600 rows, 227 us with the vectors and weights in
+// memory and one thread per row.  As separate launches an iteration took five
+// kernels and the solve two or three waits of the host.
+//
+// Layout: kVL threads per row, each with its share of the row's slots in
+// registers for the whole solve (K > 0), two of them with one component's
+// vectors; only p and s, which other rows gather, are in memory, the two
+// components side by side so that a gather is one 16-byte load.
+//
+// Fewer reductions than the textbook form: (rh, r) = (rh, s) - omega (rh, t),
+// so x, r and p are one pass; (r, r) = (s, s) - omega (t, s), raised by 1e-14
+// (s, s), more than the rounding of the difference, so that it never claims a
+// convergence that the vectors do not have.  A component that has converged
+// keeps its x while the other one goes on.
 template <int K>
 __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs a) {
   if (*a.fail) return;
+  constexpr int NS = K > 0 ? (K + kVL - 1) / kVL : 1;
   __shared__ double sh[kVNV * kVT];
   __shared__ double part[kVNV * 4];
   __shared__ VScal S;
   __shared__ int okf;
   Grid<kVT, kVNV> g{sh, part, &okf, a.partials, a.arrivals};
-  const int tid = threadIdx.x;
-  const int r0 = min(a.N, a.rows * (int)blockIdx.x), r1 = min(a.N, r0 + a.rows);
-  const int active = min(kVT, (a.rows + 31) / 32 * 32);
-  for (int i = r0 + tid; i < r1; i += kVT)
-    for (int q = 0; q < 2; ++q) a.x0[q][i] = a.x[q][i];
+  const int tid = threadIdx.x, sub = tid & (kVL - 1), c = sub & 1;
+  const int i = a.rows * (int)blockIdx.x + tid / kVL;
+  const bool mine = tid / kVL < a.rows && i < a.N;
+  const bool own = mine && sub < 2;
+  const int active = min(kVT, (a.rows * kVL + 31) / 32 * 32);  // whole warps
+  const bool same = a.w[0] == a.w[1];
+  int jj[NS] = {};
+  double w0[NS] = {}, w1[NS] = {};
+  if constexpr (K > 0) {
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+      const int s = sub + kVL * t;
+      if (!mine || s >= K) continue;
+      jj[t] = a.idx[s * a.ld + i];
+      w0[t] = a.w[0][s * a.ld + i];
+      w1[t] = same ? w0[t] : a.w[1][s * a.ld + i];
+    }
+  }
+  // this thread's component of the row's off-diagonal sum; at(j) gives both
+  // components' entries of column j
+  auto row = [&](auto at) {
+    double s0 = 0.0, s1 = 0.0;
+    if constexpr (K > 0) {
+#pragma unroll
+      for (int t = 0; t < NS; ++t) {
+        const double2 q = at(jj[t]);
+        s0 = fma(w0[t], q.x, s0);
+        s1 = fma(w1[t], q.y, s1);
+      }
+    } else if (mine) {
+      for (int s = sub; s < a.k; s += kVL) {
+        const double2 q = at(__ldg(a.idx + s * a.ld + i));
+        s0 = fma(__ldg(a.w[0] + s * a.ld + i), q.x, s0);
+        s1 = fma(__ldg(a.w[1] + s * a.ld + i), q.y, s1);
+      }
+    }
+    double y = c ? s1 : s0;
+    y += __shfl_xor_sync(0xffffffffu, c ? s0 : s1, 1);
+    return y + __shfl_xor_sync(0xffffffffu, y, 2);
+  };
+  const double2* P = reinterpret_cast<const double2*>(a.p);
+  const double2* Sv = reinterpret_cast<const double2*>(a.s);
+  const double b = mine ? a.b[c][i] : 0.0, x0 = mine ? a.x[c][i] : 0.0;
+  double x = x0, r = 0.0, rh = 0.0, p = 0.0, v = 0.0, s = 0.0, t = 0.0;
   if (tid == 0) S.total = 0;
   for (int cyc = 0;; ++cyc) {
-    const uint32_t seed = cyc ? 0x51ED27u + (uint32_t)cyc : 0u;
     {
+      const uint32_t seed = cyc ? 0x51ED27u + (uint32_t)cyc : 0u;
       double d[6] = {};
-      for (int i = r0 + tid; i < r1; i += kVT) {
-        double y[2];
-        v_row<K>(a, i, a.x, y);
-        const double sgn = seed ? (double)hash_sign(i, seed) : 1.0;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const double bi = a.b[q][i], ri = bi - y[q];
-          a.r[q][i] = ri;
-          a.rh[q][i] = sgn * ri;
-          a.p[q][i] = ri;
-          d[3 * q] += ri * ri;
-          d[3 * q + 1] += bi * bi;
-          d[3 * q + 2] += sgn * ri * ri;
+      if (tid < active) {
+        r = b - (x + row([&](int j) { return make_double2(a.x[0][j], a.x[1][j]); }));
+        rh = seed ? (double)hash_sign(i, seed) * r : r;
+        p = r;
+        if (own) {
+          a.p[2 * i + c] = p;
+          d[c ? 3 : 0] = r * r;
+          d[c ? 4 : 1] = b * b;
+          d[c ? 5 : 2] = rh * r;
         }
       }
-      const bool ok = g.template reduce<6>(d, active, [&](const double* t) {
+      const bool ok = g.template reduce<6>(d, active, [&](const double* q6) {
         S.status = 0;
         S.iters = 0;
         S.go = 0;
         for (int q = 0; q < 2; ++q) {
-          S.rr[q] = t[3 * q];
-          S.bb[q] = t[3 * q + 1];
-          S.rho[q] = t[3 * q + 2];
-          S.half[q] = 0;
+          S.rr[q] = q6[3 * q];
+          S.bb[q] = q6[3 * q + 1];
+          S.rho[q] = q6[3 * q + 2];
           if (!isfinite(S.rr[q])) S.status = 2;
           S.active[q] = isfinite(S.rr[q]) && S.rr[q] > a.tol2 * S.bb[q] && S.rho[q] != 0.0;
           S.go |= S.active[q];
@@ -384,123 +419,93 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
     while (run) {
       {  // v = H p; (rh, v)
         double d[2] = {};
-        for (int i = r0 + tid; i < r1; i += kVT) {
-          double y[2];
-          v_row<K>(a, i, a.p, y);
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            a.v[q][i] = y[q];
-            d[q] += a.rh[q][i] * y[q];
-          }
+        if (tid < active) {
+          v = p + row([&](int j) { return P[j]; });
+          if (own) d[c ? 1 : 0] = rh * v;
         }
-        const bool ok = g.template reduce<2>(d, active, [&](const double* t) {
+        const bool ok = g.template reduce<2>(d, active, [&](const double* q2) {
+          S.go = 0;
           for (int q = 0; q < 2; ++q) {
+            S.mode[q] = 0;
             if (!S.active[q]) continue;
-            if (t[q] == 0.0 || !isfinite(t[q])) {
+            if (q2[q] == 0.0 || !isfinite(q2[q])) {
               S.active[q] = 0;
-              S.status = isfinite(t[q]) ? 1 : 2;
+              S.status = isfinite(q2[q]) ? 1 : 2;
             } else {
-              S.alpha[q] = quot(S.rho[q], t[q]);
+              S.alpha[q] = quot(S.rho[q], q2[q]);
+              S.go = 1;
             }
           }
         });
         if (!ok) return give_up(a);
+        if (!S.go) break;
       }
+      const double al = S.alpha[c];
       {  // s = r - alpha v; (s, s), (rh, s)
         double d[4] = {};
-        const double al[2] = {S.alpha[0], S.alpha[1]};
-        const bool act[2] = {S.active[0] != 0, S.active[1] != 0};
-        for (int i = r0 + tid; i < r1; i += kVT) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            if (!act[q]) continue;
-            const double si = a.r[q][i] - al[q] * a.v[q][i];
-            a.s[q][i] = si;
-            d[q] += si * si;
-            d[2 + q] += a.rh[q][i] * si;
-          }
+        if (own && S.active[c]) {
+          s = r - al * v;
+          a.s[2 * i + c] = s;
+          d[c ? 2 : 0] = s * s;
+          d[c ? 3 : 1] = rh * s;
         }
-        const bool ok = g.template reduce<4>(d, active, [&](const double* t) {
+        const bool ok = g.template reduce<4>(d, active, [&](const double* q4) {
           S.iterate = 0;
           for (int q = 0; q < 2; ++q) {
             if (!S.active[q]) continue;
-            S.half[q] = t[q] <= a.tol2 * S.bb[q];
-            S.rhs[q] = t[2 + q];
-            if (S.half[q])
-              S.rr[q] = t[q];
-            else
+            S.ss[q] = q4[2 * q];
+            S.rhs[q] = q4[2 * q + 1];
+            if (S.ss[q] <= a.tol2 * S.bb[q]) {
+              S.rr[q] = S.ss[q];
+              S.mode[q] = 1;
+              S.active[q] = 0;
+            } else {
+              S.mode[q] = 2;
               S.iterate = 1;
+            }
+          }
+          if (!S.iterate) {
+            S.iters += 1;
+            S.go = 0;
           }
         });
         if (!ok) return give_up(a);
       }
       if (S.iterate) {  // t = H s; (t, s), (t, t), (rh, t)
         double d[6] = {};
-        for (int i = r0 + tid; i < r1; i += kVT) {
-          double y[2];
-          v_row<K>(a, i, a.s, y);
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            a.t[q][i] = y[q];
-            d[3 * q] += y[q] * a.s[q][i];
-            d[3 * q + 1] += y[q] * y[q];
-            d[3 * q + 2] += a.rh[q][i] * y[q];
+        if (tid < active) {
+          t = s + row([&](int j) { return Sv[j]; });
+          if (own) {
+            d[c ? 3 : 0] = t * s;
+            d[c ? 4 : 1] = t * t;
+            d[c ? 5 : 2] = rh * t;
           }
         }
-        const bool ok = g.template reduce<6>(d, active, [&](const double* t) {
-          for (int q = 0; q < 2; ++q) {
-            if (!S.active[q] || S.half[q]) continue;
-            const double ts = t[3 * q], tt = t[3 * q + 1];
-            if (!(tt > 0.0) || !isfinite(ts)) {
-              S.active[q] = 0;
-              S.status = isfinite(tt) ? 3 : 2;
-              continue;
-            }
-            const double om = quot(ts, tt), rn = S.rhs[q] - om * t[3 * q + 2];
-            S.beta[q] = quot(rn, S.rho[q]) * quot(S.alpha[q], om);
-            S.omega[q] = om;
-            S.rho[q] = rn;
-          }
-        });
-        if (!ok) return give_up(a);
-      }
-      {  // x, r, p; (r, r)
-        double d[2] = {};
-        const double al[2] = {S.alpha[0], S.alpha[1]}, om[2] = {S.omega[0], S.omega[1]},
-                     be[2] = {S.beta[0], S.beta[1]};
-        const bool act[2] = {S.active[0] != 0, S.active[1] != 0};
-        const bool hf[2] = {S.half[0] != 0, S.half[1] != 0};
-        for (int i = r0 + tid; i < r1; i += kVT) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            if (!act[q]) continue;
-            const double pi = a.p[q][i], si = a.s[q][i];
-            if (hf[q]) {
-              a.x[q][i] += al[q] * pi;
-              d[q] += si * si;
-              continue;
-            }
-            a.x[q][i] += al[q] * pi + om[q] * si;
-            const double ri = si - om[q] * a.t[q][i];
-            a.r[q][i] = ri;
-            a.p[q][i] = ri + be[q] * (pi - om[q] * a.v[q][i]);
-            d[q] += ri * ri;
-          }
-        }
-        const bool ok = g.template reduce<2>(d, active, [&](const double* t) {
+        const bool ok = g.template reduce<6>(d, active, [&](const double* q6) {
           S.iters += 1;
           int any = 0;
           for (int q = 0; q < 2; ++q) {
-            if (!S.active[q]) continue;
-            S.rr[q] = t[q];
+            if (S.mode[q] != 2) continue;
+            const double ts = q6[3 * q], tt = q6[3 * q + 1];
             S.active[q] = 0;
-            if (!isfinite(t[q]))
+            if (!(tt > 0.0) || !isfinite(ts)) {
+              S.mode[q] = 0;
+              S.status = isfinite(tt) ? 3 : 2;
+              continue;
+            }
+            const double om = quot(ts, tt), rn = S.rhs[q] - om * q6[3 * q + 2];
+            const double rr = fmax(S.ss[q] - om * ts, 0.0) + 1e-14 * S.ss[q];
+            S.beta[q] = quot(rn, S.rho[q]) * quot(S.alpha[q], om);
+            S.omega[q] = om;
+            S.rho[q] = rn;
+            S.rr[q] = rr;
+            if (!isfinite(S.ss[q]) || !isfinite(om))
               S.status = 2;
-            else if (t[q] > 1e8 * S.bb[q] && S.bb[q] > 0.0)
+            else if (rr > 1e8 * S.bb[q] && S.bb[q] > 0.0)
               S.status = 5;
-            else if (S.half[q] || t[q] <= a.tol2 * S.bb[q])
+            else if (rr <= a.tol2 * S.bb[q])
               ;
-            else if (S.rho[q] == 0.0 || S.omega[q] == 0.0)
+            else if (rn == 0.0 || om == 0.0)
               S.status = 4;
             else
               any = S.active[q] = 1;
@@ -509,7 +514,19 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
         });
         if (!ok) return give_up(a);
       }
+      // x, r, p
+      const int mode = S.mode[c];
       run = S.go != 0;
+      if (mode == 1) {
+        x += al * p;
+      } else if (mode == 2) {
+        const double om = S.omega[c];
+        x += al * p + om * s;
+        r = s - om * t;
+        p = r + S.beta[c] * (p - om * v);
+        if (own) a.p[2 * i + c] = p;
+      }
+      if (run && !g.sync()) return give_up(a);
     }
     bool conv = true, near = true;
     for (int q = 0; q < 2; ++q) {
@@ -518,9 +535,10 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
     }
     const int st = S.status, tot = S.total + S.iters;
     const bool again = st == 1 || st == 3 || st == 4 || st == 5;
-    __syncthreads();
-    if (tid == 0) S.total = tot;
-    if (conv || !again || tot >= a.maxit || cyc >= 400) {
+    const bool end = conv || !again || tot >= a.maxit || cyc >= 400;
+    if (!end && st == 5) x = x0;  // the recurrence has blown up: from the initial iterate
+    if (own) a.x[c][i] = x;
+    if (end) {
       if (blockIdx.x == 0 && tid == 0) {
         double worst = 0.0;
         for (int q = 0; q < 2; ++q)
@@ -533,11 +551,9 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
       }
       return leave(a.arrivals);
     }
-    if (st == 5)  // the recurrence has blown up: start again from the initial iterate
-      for (int i = r0 + tid; i < r1; i += kVT)
-        for (int q = 0; q < 2; ++q) a.x[q][i] = a.x0[q][i];
-    // the residual of the restart reads x of other blocks
+    // the restart's residual reads x of other blocks
     if (!g.sync()) return give_up(a);
+    if (tid == 0) S.total = tot;
   }
 }
 
@@ -558,11 +574,13 @@ void vsolve_free(VSolve* v) {
 int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* idx,
                  const double* wu, const double* wv, VSolve** out, cudaStream_t st) {
   *out = nullptr;
+  // a block's threads hold its rows' vectors
+  if (N > (int64_t)sm_count() * (kVT / kVL)) return RBFFD_OK;
   VSolve* v = new VSolve();
-  v->grid = sm_count();
   VArgs& a = v->a;
   a.N = (int)N;
-  a.rows = (int)((N + v->grid - 1) / v->grid);
+  a.rows = (int)std::max<int64_t>(kVRows, (N + sm_count() - 1) / sm_count());
+  v->grid = (int)((N + a.rows - 1) / a.rows);
   a.k = k;
   a.ld = ld;
   a.idx = idx;
@@ -575,11 +593,8 @@ int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* id
     return check_cuda(ctx, cudaMemsetAsync(*p, 0, bytes, st), "memset");
   };
   int rc = 0;
-  for (int q = 0; q < 2 && !rc; ++q) {
-    double** vec[] = {&a.r[q], &a.rh[q], &a.p[q], &a.v[q], &a.s[q], &a.t[q], &a.x0[q]};
-    for (double** p : vec)
-      if (!rc) rc = get((void**)p, sizeof(double) * N);
-  }
+  if (!rc) rc = get((void**)&a.p, sizeof(double) * 2 * N);
+  if (!rc) rc = get((void**)&a.s, sizeof(double) * 2 * N);
   if (!rc) rc = get((void**)&a.partials, sizeof(double) * 2 * kVNV * v->grid);
   if (!rc) rc = get((void**)&a.arrivals, 2 * sizeof(unsigned int));
   if (rc) {

@@ -42,12 +42,11 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
 // of the scaled pressure operator, built once per plan, applied with iterative
 // refinement.
 //
-// Where the line lies: a solve takes one product with the inverse and two
-// residuals, 16 us at 1,600 rows, 30 us at 2,700 and about 60 us at 4,096
-// (16.8 M FP64 FMAs, and an inverse of 134 MB that no longer stays in L2),
-// against 40 to 55 us for EACH of the 40 to 500 Krylov iterations that these
-// sizes take; beyond it the inversion (n^3 FP64 FMAs, 0.2 s at 4,096) would
-// cost a first pass more than the hierarchy it replaces.
+// Where the line lies: a solve is one or two products with the inverse and
+// their residuals, 47 us with cold caches at 1,600 rows, against 40 to 55 us for
+// EACH of the 40 to 500 Krylov iterations that these sizes take.  At 4,096 the
+// inverse (134 MB) no longer fits L2; beyond it the inversion (n^3 FP64 FMAs)
+// would cost a first pass more than the hierarchy it replaces.
 constexpr int kDenseMax = 4096;
 struct DSolve;
 

@@ -1380,8 +1380,8 @@ template <int K, bool MIX>
 __global__ void __launch_bounds__(kThreads) k_convect(ConvArgs a) {
   if (a.skip && *a.skip) return;
   const void* w[2] = {a.wdx, a.wdy};
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * kThreads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double du[2], dv[2];
     Gather<K, MIX, 2>::run(a.idx, w, a.ld, a.k, i, a.u, a.u2, du);
     Gather<K, MIX, 2>::run(a.idx, w, a.ld, a.k, i, a.v, a.v2, dv);
@@ -1444,8 +1444,8 @@ __global__ void __launch_bounds__(kThreads) k_helm_rhs(HelmRhsArgs a) {
   if (a.skip && *a.skip) return;
   const void* wl[1] = {a.lap};
   const void* wg[2] = {a.vp_dx, a.vp_dy};
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * kThreads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double bu, bv;
     if (!a.v_bc[i]) {
       double lu, lv;
@@ -1529,8 +1529,8 @@ __global__ void __launch_bounds__(kThreads) k_divergence(DivArgs a) {
   if (a.skip && *a.skip) return;
   const void* wx[1] = {a.wdx};
   const void* wy[1] = {a.wdy};
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * kThreads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double fx, fy;
     Gather<K, MIX, 1>::run(a.idx, wx, a.ld_p, a.k, i, a.uss, a.uss2, &fx);
     Gather<K, MIX, 1>::run(a.idx, wy, a.ld_p, a.k, i, a.vss, a.vss2, &fy);
@@ -1562,8 +1562,8 @@ __global__ void __launch_bounds__(kThreads) k_pressure(PresArgs a) {
   if (a.skip && *a.skip) return;
   const void* wl[1] = {a.lap};
   const double mean = a.nomean ? 0.0 : *a.sum / (double)a.n;
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * kThreads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double l;
     Gather<K, MIX, 1>::run(a.idx, wl, a.ld_p, a.k, i, a.px, a.px2, &l);
     const double pt = (a.proj ? a.pt[i] : 0.0) + (a.px[i] - mean);
@@ -1602,8 +1602,8 @@ __global__ void __launch_bounds__(kThreads) k_correct(CorrArgs a) {
   if (a.skip && *a.skip) return;
   const void* w[2] = {a.wdx, a.wdy};
   const double c = a.proj ? -a.dt * (*a.sum) / (*a.esn) : 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * kThreads) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double un, vn;
     if (a.proj && a.v_bc[i]) {
       un = a.uss[i] - c * a.v_nx[i];
@@ -3005,14 +3005,26 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   KOp<float, float> Hv32{P->Hidx, P->Hw32_v, f.ld_v, f.N, k, 1, nullptr, nullptr};
   (MIX ? Hu32.tiles : Hu64.tiles) = P->Ht;
   (MIX ? Hv32.tiles : Hv64.tiles) = P->Ht_v;
-  const int GN = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.N + kThreads - 1) / kThreads));
-  const int GM = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.M + kThreads - 1) / kThreads));
+  // Blocks of the stage kernels: as small as it takes to reach every SM, as
+  // many as there are rows for.  A row's gathers are 100 to 200 FP64
+  // instructions, of which an SM retires a warp's in 2 to 3 us, so the rows of
+  // a small flow are spread (1,600 rows, cold caches: k_convect 31 us in seven
+  // blocks of 256, 17 us in 50 of 32).
+  auto block_of = [](int64_t n) {
+    int t = kThreads;
+    while (t > 32 && (n + t - 1) / t < sm_count()) t /= 2;
+    return t;
+  };
+  const int TN = block_of(f.N), TM = block_of(f.M);
+  const int GN = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.N + TN - 1) / TN));
+  const int GM = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.M + TM - 1) / TM));
+  const int GS = (int)std::max<int64_t>(1, std::min<int64_t>(G, (f.M + kThreads - 1) / kThreads));
   // Stages 1 and 2 up to the viscous right side and initial guess.
   auto front = [&](const int* skip) -> int {
     ConvArgs ca{f.N,  f.ld_v,       k,  f.vv_idx, vdx, vdy,   s->u,  s->v,  P->u2,
                 P->v2, s->cu_prev, s->cv_prev, P->us, P->vs, P->us2, P->vs2, f.dt,
                 s->j == 0 ? 1 : 0, skip};
-    k_convect<K, MIX><<<GN, kThreads, 0, st>>>(ca);
+    k_convect<K, MIX><<<GN, TN, 0, st>>>(ca);
     HelmRhsArgs ha{f.N,    f.ld_v, k,      f.vv_idx, vlap,   P->us,  P->vs,  P->us2,
                    P->vs2, f.vp_idx, gdx,  gdy,      s->pt,  P->pt2, f.v_bc, f.v_nx,
                    f.v_ny, gu,     gv,     a,        f.dt,   f.km_mode, P->ru, P->rv,
@@ -3038,7 +3050,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     } else {
       P->vhist = 0;
     }
-    k_helm_rhs<K, MIX><<<GN, kThreads, 0, st>>>(ha);
+    k_helm_rhs<K, MIX><<<GN, TN, 0, st>>>(ha);
     P->launches += 2 + (MIX ? 2 : 0) + 4 + (MIX ? 1 : 0);  // stage kernels of this step
     return check_cuda(ctx, cudaGetLastError(), "stage 1-2 kernels");
   };
@@ -3115,7 +3127,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     DivArgs da{f.M,    f.ld_p,  k,      f.pv_idx, f.pv_dx,  f.pv_dy,      P->uss,
                P->vss, P->uss2, P->vss2, f.p_bc,  P->scale, 1.0 / f.dt, P->pb, P->proj,
                skip};
-    k_divergence<K, false><<<GM, kThreads, 0, st>>>(da);
+    k_divergence<K, false><<<GM, TM, 0, st>>>(da);
     // Initial guess: the extrapolation in time through the previous steps'
     // solutions (up to cubic), else the state's p~.  Any guess
     // leaves the converged solution the same; a better one saves iterations
@@ -3132,7 +3144,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       const int ord = std::min(P->nhist, kMaxHist);
       History H;
       for (int q = 0; q < kMaxHist; ++q) H.h[q] = P->pxh[(P->hhead + q) % kMaxHist];
-      k_extrapolate<<<GM, kThreads, 0, st>>>(f.M, ord, P->px, H, skip);
+      k_extrapolate<<<GM, TM, 0, st>>>(f.M, ord, P->px, H, skip);
       rc = check_cuda(ctx, cudaGetLastError(), "extrapolation");
       if (rc) return rc;
       P->hhead = (P->hhead + kMaxHist - 1) % kMaxHist;  // the recycled slot is the newest
@@ -3142,11 +3154,11 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   };
   // Stage 3 after the pressure solve.
   auto back = [&](const int* skip) -> int {
-    k_sum<double><<<GM, kThreads, 0, st>>>(P->px, f.M, P->gr, P->dscal);
+    k_sum<double><<<GS, kThreads, 0, st>>>(P->px, f.M, P->gr, P->dscal);
     if (MIX) k_split<<<G, kThreads, 0, st>>>(f.M, P->px, P->px2);
     PresArgs pa{f.M,   f.ld_p, k,    f.pp_idx, plap,   P->px,  P->px2,
                 P->dscal, a,   s->pt, s->p, P->pt2,   P->proj, P->pdir > 0 ? 1 : 0, skip};
-    k_pressure<K, MIX><<<GM, kThreads, 0, st>>>(pa);
+    k_pressure<K, MIX><<<GM, TM, 0, st>>>(pa);
     // The exact projection corrects with G0 x (x = phi + const) and the wall
     // flux, with FP64 weights in both precisions (like the divergence), so
     // that D^(P,V) u_{j+1} vanishes to the solve's accuracy.
@@ -3157,19 +3169,20 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
                 P->proj,  P->dscal, P->esn, f.v_nx,         f.v_ny,
                 f.v_bcu,  f.v_bcv, skip};
     if (proj && MIX) {
-      k_correct<K, false><<<GN, kThreads, 0, st>>>(ka);
+      k_correct<K, false><<<GN, TN, 0, st>>>(ka);
       k_split<<<G, kThreads, 0, st>>>(f.N, s->u, P->u2);
       k_split<<<G, kThreads, 0, st>>>(f.N, s->v, P->v2);
     } else {
-      k_correct<K, MIX><<<GN, kThreads, 0, st>>>(ka);
+      k_correct<K, MIX><<<GN, TN, 0, st>>>(ka);
     }
     return check_cuda(ctx, cudaGetLastError(), "stage 3 kernels");
   };
   // A small FP64 flow's solves decide on the GPU, so its steps are enqueued
   // ahead, up to kSmallBatch at a time, and the host waits once for all of
-  // them; a wait after each solve was half of a 1,600-node step.  A step whose
-  // solve fails turns what follows into no-ops; the host takes its own
-  // bookkeeping back to that step and goes on with the launch by launch solve.
+  // them (a step of 1,600 nodes 0.63 ms with a wait after each solve and the
+  // launch by launch viscous solve, 0.28 enqueued ahead).  A step whose solve
+  // fails turns what follows into no-ops; the host takes its own bookkeeping
+  // back to that step and goes on with the launch by launch solve.
   const bool ahead = !MIX && direct && P->vis;
   struct Mark {
     int64_t j, px_step;
