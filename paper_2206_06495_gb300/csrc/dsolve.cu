@@ -334,11 +334,10 @@ template <int K>
 __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs a) {
   if (*a.fail) return;
   constexpr int NS = K > 0 ? (K + kVL - 1) / kVL : 1;
-  __shared__ double sh[kVNV * kVT];
-  __shared__ double part[kVNV * 4];
+  __shared__ double wsum[kVNV * (kVT / 32)];
   __shared__ VScal S;
   __shared__ int okf;
-  Grid<kVT, kVNV> g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<kVT, kVNV> g{nullptr, nullptr, &okf, a.partials, a.arrivals};
   const int tid = threadIdx.x, sub = tid & (kVL - 1), c = sub & 1;
   const int i = a.rows * (int)blockIdx.x + tid / kVL;
   const bool mine = tid / kVL < a.rows && i < a.N;
@@ -379,6 +378,29 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
     y += __shfl_xor_sync(0xffffffffu, c ? s0 : s1, 1);
     return y + __shfl_xor_sync(0xffffffffu, y, 2);
   };
+  // Grid-wide sums of n values of each component, handed to fin as
+  // [component][value]; only threads that own a component of a row hold values.
+  // In the warp they meet over the rows alone: three FP64 adds per value, where
+  // adding two components' values over all lanes would take ten.
+  auto sum = [&](auto& d, auto fin) -> bool {
+    constexpr int n = sizeof(d) / sizeof(double);
+    if (tid < active) {
+#pragma unroll
+      for (int o = kVL; o < 32; o *= 2) {
+#pragma unroll
+        for (int j = 0; j < n; ++j) d[j] += __shfl_xor_sync(0xffffffffu, d[j], o);
+      }
+      if ((tid & 31) < 2) {
+#pragma unroll
+        for (int j = 0; j < n; ++j) wsum[(c * n + j) * (kVT / 32) + tid / 32] = d[j];
+      }
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (tid < 2 * n)
+      for (int w = 0; w < active / 32; ++w) t += wsum[tid * (kVT / 32) + w];
+    return g.template spread<2 * n>(t, fin);
+  };
   const double2* P = reinterpret_cast<const double2*>(a.p);
   const double2* Sv = reinterpret_cast<const double2*>(a.s);
   const double b = mine ? a.b[c][i] : 0.0, x0 = mine ? a.x[c][i] : 0.0;
@@ -387,19 +409,19 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
   for (int cyc = 0;; ++cyc) {
     {
       const uint32_t seed = cyc ? 0x51ED27u + (uint32_t)cyc : 0u;
-      double d[6] = {};
+      double d[3] = {};
       if (tid < active) {
         r = b - (x + row([&](int j) { return make_double2(a.x[0][j], a.x[1][j]); }));
         rh = seed ? (double)hash_sign(i, seed) * r : r;
         p = r;
         if (own) {
           a.p[2 * i + c] = p;
-          d[c ? 3 : 0] = r * r;
-          d[c ? 4 : 1] = b * b;
-          d[c ? 5 : 2] = rh * r;
+          d[0] = r * r;
+          d[1] = b * b;
+          d[2] = rh * r;
         }
       }
-      const bool ok = g.template reduce<6>(d, active, [&](const double* q6) {
+      const bool ok = sum(d, [&](const double* q6) {
         S.status = 0;
         S.iters = 0;
         S.go = 0;
@@ -418,12 +440,12 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
     bool run = S.go != 0;
     while (run) {
       {  // v = H p; (rh, v)
-        double d[2] = {};
+        double d[1] = {};
         if (tid < active) {
           v = p + row([&](int j) { return P[j]; });
-          if (own) d[c ? 1 : 0] = rh * v;
+          if (own) d[0] = rh * v;
         }
-        const bool ok = g.template reduce<2>(d, active, [&](const double* q2) {
+        const bool ok = sum(d, [&](const double* q2) {
           S.go = 0;
           for (int q = 0; q < 2; ++q) {
             S.mode[q] = 0;
@@ -442,14 +464,14 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
       }
       const double al = S.alpha[c];
       {  // s = r - alpha v; (s, s), (rh, s)
-        double d[4] = {};
+        double d[2] = {};
         if (own && S.active[c]) {
           s = r - al * v;
           a.s[2 * i + c] = s;
-          d[c ? 2 : 0] = s * s;
-          d[c ? 3 : 1] = rh * s;
+          d[0] = s * s;
+          d[1] = rh * s;
         }
-        const bool ok = g.template reduce<4>(d, active, [&](const double* q4) {
+        const bool ok = sum(d, [&](const double* q4) {
           S.iterate = 0;
           for (int q = 0; q < 2; ++q) {
             if (!S.active[q]) continue;
@@ -472,16 +494,16 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
         if (!ok) return give_up(a);
       }
       if (S.iterate) {  // t = H s; (t, s), (t, t), (rh, t)
-        double d[6] = {};
+        double d[3] = {};
         if (tid < active) {
           t = s + row([&](int j) { return Sv[j]; });
           if (own) {
-            d[c ? 3 : 0] = t * s;
-            d[c ? 4 : 1] = t * t;
-            d[c ? 5 : 2] = rh * t;
+            d[0] = t * s;
+            d[1] = t * t;
+            d[2] = rh * t;
           }
         }
-        const bool ok = g.template reduce<6>(d, active, [&](const double* q6) {
+        const bool ok = sum(d, [&](const double* q6) {
           S.iters += 1;
           int any = 0;
           for (int q = 0; q < 2; ++q) {

@@ -70,14 +70,23 @@ struct Grid {
       if (lane == 0) part[j * 4 + q] = a;
     }
     __syncthreads();
-    double* mine = partials + (size_t)(phase & 1) * NVM * gridDim.x;
-    ++phase;
+    double mine = 0.0;
     if (t < NV) {
       const double* q = part + t * 4;
-      mine[t * gridDim.x + blockIdx.x] = (q[0] + q[1]) + (q[2] + q[3]);
+      mine = (q[0] + q[1]) + (q[2] + q[3]);
     }
+    return spread<NV>(mine, fin);
+  }
+
+  // The second half of reduce(): the block's sum j is in thread j.
+  template <int NV, typename Fin>
+  __device__ __forceinline__ bool spread(double sum, Fin fin) {
+    const int t = threadIdx.x, lane = t & 31;
+    double* mine = partials + (size_t)(phase & 1) * NVM * gridDim.x;
+    ++phase;
+    if (t < NV) mine[t * gridDim.x + blockIdx.x] = sum;
     if (!sync()) return false;
-    if (w == 0) {
+    if (t < 32) {
       double a[NV];
 #pragma unroll
       for (int j = 0; j < NV; ++j) a[j] = 0.0;

@@ -17,7 +17,7 @@ def _d(a):
 def _flow(kind, **kw):
     from paper_2206_06495_gb300 import rbffd as R
     from paper_2206_06495_gb300 import wake
-    ctx = R.Context(28, 7, 3)
+    ctx = R.Context(30 if kind == "21 n30" else 28, 7, 3)
     if kind == "wake":
         nd = ns.cylinder_wake(h_wall=0.06, h_wake=0.08, h_far=0.5, x0=-3.0, x1=6.0, y0=-3.0,
                               y1=3.0)
@@ -25,7 +25,7 @@ def _flow(kind, **kw):
         gu, gv = wake.wake_data(nd)
         u0 = torch.ones(nd.N, dtype=torch.float64, device="cuda")
         return R, ctx, flow, gu, gv, u0
-    n = int(kind)
+    n = int(kind.split()[0])
     nd = ns.jittered_cavity(n, 3)
     flow = R.flow_from_nodes(ctx, nd, **{**dict(Re=100.0, dt=0.08 / (n - 1), tol=1e-12), **kw})
     gu, gv = (_d(g) for g in O.lid_bc(nd))
@@ -38,8 +38,9 @@ def _same(a, b):
                for x, y in ((a.u, b.u), (a.v, b.v), (a.pt, b.pt), (a.p, b.p)))
 
 
-# 81 nodes: fewer than the SMs; 1,089 and 4,096 (the largest); an open flow
-@pytest.mark.parametrize("kind", ["9", "33", "64", "wake"])
+# 81 nodes: fewer than the SMs; 1,089 and 4,096 (the largest); a stencil of
+# other than 28 nodes; an open flow
+@pytest.mark.parametrize("kind", ["9", "33", "64", "21 n30", "wake"])
 @pytest.mark.parametrize("steps", [1, 32, 33])
 def test_grouping_of_steps(kind, steps):
     """One call of n steps gives the bits of n calls, and the launch by launch
