@@ -586,8 +586,11 @@ __global__ void __launch_bounds__(kT)
 }
 
 // x += alpha zp + omega zs; r = s - omega t; reduce (rh, r), (r, r); beta
+// Four blocks per SM, as the grid has: with the 88 registers that four columns
+// take otherwise, half of the grid ran after the other half (94 against 76 us a
+// launch at 100k nodes x 64 members, mean of both solves).
 template <int V>
-__global__ void __launch_bounds__(kT)
+__global__ void __launch_bounds__(kT, 4)
     e_update_xr(int64_t n, float* __restrict__ x, float* __restrict__ r,
                 const float* __restrict__ rh, const float* __restrict__ zp,
                 const float* __restrict__ zs, const float* __restrict__ s,
@@ -960,9 +963,11 @@ __device__ __forceinline__ void e_finish(EScal* sc, int which, int c, double zsu
 // Post-smoothing z = x + omega D^-1 (r - G x) on a level whose x holds the
 // coarse correction; above level 0 it corrects the finer level's rows of each
 // aggregate (x_fine += scale z), on level 0 it writes z in P-node order and
-// reduces its per-column sum (for B v = z - mean(z) + mu / M)
+// reduces its per-column sum (for B v = z - mean(z) + mu / M).  Four blocks per
+// SM, as the grid has: at 69 registers three fit, and a quarter of the grid ran
+// alone afterwards (level 0, 100k rows x 64 members: 83 against 56 us).
 template <int W, int V, bool LEVEL0>
-__global__ void __launch_bounds__(kT)
+__global__ void __launch_bounds__(kT, 4)
     e_pc_up(AmgLevel F, int C, const float* __restrict__ r, const float* __restrict__ x,
             AmgLevel Fine, float* __restrict__ xfine, const int32_t* __restrict__ perm0,
             float* __restrict__ zout, int which, double inv_ces, double inv_R, EScal* sc,
