@@ -288,7 +288,7 @@ constexpr int kVL = 4;    // threads per row
 // Rows of a block, where there are SMs for so few: fewer blocks make the
 // barrier lighter, fewer rows the phases (8, 16, 32, 64 rows: 20 steps of 1,600
 // nodes 5.67, 5.69, 5.63, 5.57 ms, four of the 2,700-node wake 1.47, 1.45, 1.44,
-// 1.49).
+// 1.49; 5.13 and 1.37 since the sums of a warp meet before those of a block).
 constexpr int kVRows = 32;
 constexpr int kVNV = 6;
 

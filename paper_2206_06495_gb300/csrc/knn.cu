@@ -3,11 +3,11 @@
 // A uniform bucket grid over the bounding box of both node sets holds about
 // two beta-nodes per cell.  Buckets are built with a counting sort (count,
 // exclusive scan, scatter).  Each alpha-node (a warp, or one thread for more
-// than 32 neighbours) then scans rings of cells around its own cell, keeping the k best candidates ordered by
-// (squared distance, index); it stops once no point outside the rings seen so
-// far can beat the current k-th candidate.  Squared distances are formed as
-// dx*dx + dy*dy with each operation rounded on its own, so the ordering
-// (including ties) is reproducible on any IEEE machine.
+// than 32 neighbours) then scans rings of cells around its own cell, keeping the
+// k best candidates ordered by (squared distance, index); it stops once no point
+// outside the rings seen so far can beat the current k-th candidate.  Squared
+// distances are formed as dx*dx + dy*dy with each operation rounded on its own,
+// so the ordering (including ties) is reproducible on any IEEE machine.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>

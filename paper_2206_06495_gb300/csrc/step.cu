@@ -3180,7 +3180,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   // A small FP64 flow's solves decide on the GPU, so its steps are enqueued
   // ahead, up to kSmallBatch at a time, and the host waits once for all of
   // them (a step of 1,600 nodes 0.63 ms with a wait after each solve and the
-  // launch by launch viscous solve, 0.28 enqueued ahead).  A step whose solve
+  // launch by launch viscous solve, 0.26 enqueued ahead).  A step whose solve
   // fails turns what follows into no-ops; the host takes its own bookkeeping
   // back to that step and goes on with the launch by launch solve.
   const bool ahead = !MIX && direct && P->vis;
