@@ -315,7 +315,7 @@ struct VScal {
 };
 
 // What bounds it: latency, four phases an iteration (a barrier of 1.3 us, the
-// reduction behind it, one gather from L2): 170 us with cold caches for the 6.5
+// reduction behind it, one gather from L2): 141 us with cold caches for the 6.5
 // iterations of a solve at 1,600 rows, 227 us with the vectors and weights in
 // memory and one thread per row.  As separate launches an iteration took five
 // kernels and the solve two or three waits of the host.

@@ -43,7 +43,7 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
 // refinement.
 //
 // Where the line lies: a solve is one or two products with the inverse and
-// their residuals, 47 us with cold caches at 1,600 rows, against 40 to 55 us for
+// their residuals, 50 us with cold caches at 1,600 rows, against 40 to 55 us for
 // EACH of the 40 to 500 Krylov iterations that these sizes take.  At 4,096 the
 // inverse (134 MB) no longer fits L2; beyond it the inversion (n^3 FP64 FMAs)
 // would cost a first pass more than the hierarchy it replaces.

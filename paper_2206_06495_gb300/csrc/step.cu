@@ -3195,6 +3195,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     if (ahead && !resume) {
       const int batch = std::min<int32_t>(n_steps - step, kSmallBatch);
       Mark marks[kSmallBatch];
+      const int64_t j0 = s->j;
       int rc = check_cuda(ctx, small_reset(P->vis, P->ds, P->fail, st), "step reset");
       for (int i = 0; i < batch && !rc; ++i) {
         Mark& m = marks[i];
@@ -3231,7 +3232,11 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
         rc = check_cuda(ctx, cudaMemcpyAsync(hf, P->fail, sizeof(int), cudaMemcpyDeviceToHost, st),
                         "step results");
       if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "step sync");
-      if (rc) return rc;
+      if (rc) {  // none of these steps is known to have run
+        s->j = j0;
+        P->px_step = -1;
+        return rc;
+      }
       const int code = *hf & 15, bad = code ? *hf >> 4 : batch;
       for (int i = 0; i < batch && i <= bad; ++i) {
         if (stats && (i < bad || code == kFailPressure)) {
