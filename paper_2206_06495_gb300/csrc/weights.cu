@@ -288,6 +288,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32)
         break;
       }
       const double inv = recip(Am[kk * LD + br]);
+      __syncwarp();  // every lane has the pivot before the exchange overwrites it
       if (br != kk) {
         for (int c = (COND ? 0 : kk) + lane; c < NC; c += 32) {
           const double t = Am[c * LD + kk];
