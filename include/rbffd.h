@@ -449,6 +449,16 @@ int rbffd_stencil_error(rbffd_ctx* ctx, const rbffd_ell* D, uint32_t op, const d
 int rbffd_debug_set_wait_limit(rbffd_ctx* ctx, int64_t polls);
 
 /*
+ * rbffd_debug_set_solver_bytes - test hook (no counterpart in the paper): in
+ * plans that this context builds from now on, an allocation of more than
+ * `bytes` bytes for the direct or a resident solve is refused as if the
+ * device were out of memory; the solve as separate launches then takes its
+ * place.  bytes < 0 restores the default (no limit).
+ * Errors: INVALID_ARG (null ctx).
+ */
+int rbffd_debug_set_solver_bytes(rbffd_ctx* ctx, int64_t bytes);
+
+/*
  * rbffd_ensemble_step - advance an ensemble of independent flows that share
  * one node set and its operators (the batching of many flows at once; the
  * paper runs one flow at a time).  Member e is the step of rbffd_step

@@ -35,6 +35,30 @@ int check_cuda(rbffd_ctx* ctx, cudaError_t e, const char* what) {
   return set_error(ctx, RBFFD_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+cudaError_t solver_malloc(const rbffd_ctx* ctx, void** out, size_t bytes) {
+  if (ctx->solver_bytes >= 0 && bytes > (size_t)ctx->solver_bytes)
+    bytes = (size_t)1 << 60;  // the runtime's own refusal, with what it leaves behind
+  return cudaMalloc(out, bytes);
+}
+
+int solver_left_out(rbffd_ctx* ctx, int rc) {
+  if (rc != RBFFD_ERR_OOM) return rc;
+  cudaGetLastError();
+  ctx->err.clear();
+  return RBFFD_OK;
+}
+
+bool coop_fits(const void* fn, int grid, int threads, size_t smem) {
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (int64_t)per_sm * sm_count() >= grid;
+}
+
 int ctx_scratch(rbffd_ctx* ctx, size_t bytes, void** out) {
   if (bytes > ctx->scratch_bytes) {
     if (ctx->scratch) cudaFree(ctx->scratch);
@@ -329,6 +353,13 @@ int rbffd_stencil_error(rbffd_ctx* ctx, const rbffd_ell* D, uint32_t op, const d
   if (D->n_rows == 0) return RBFFD_OK;
   if (!ax || !ay || !bx || !by || !err) return set_error(ctx, RBFFD_ERR_INVALID_ARG, "null pointer");
   return analysis_error(ctx, D, opi, ax, ay, bx, by, dr, err, err_mean, stream);
+}
+
+int rbffd_debug_set_solver_bytes(rbffd_ctx* ctx, int64_t bytes) {
+  if (!ctx) return RBFFD_ERR_INVALID_ARG;
+  ctx->err.clear();
+  ctx->solver_bytes = bytes < 0 ? -1 : bytes;
+  return RBFFD_OK;
 }
 
 int rbffd_debug_set_wait_limit(rbffd_ctx* ctx, int64_t polls) {

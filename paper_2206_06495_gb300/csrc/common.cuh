@@ -107,6 +107,7 @@ struct rbffd_ctx {
   void* host_pinned = nullptr;  // small pinned buffer for status words
   rbffd::StepPlan* plan = nullptr;
   rbffd::EnsPlan* ens = nullptr;  // ensemble step plan (rbffd_ensemble_step)
+  int64_t solver_bytes = -1;      // rbffd_debug_set_solver_bytes: largest allocation (-1: any)
   // launch shapes the SpMV autotuner picked, per operator shape key
   std::vector<std::pair<uint64_t, int>> spmv_shapes;
 };
@@ -115,6 +116,13 @@ namespace rbffd {
 
 int set_error(rbffd_ctx* ctx, int code, const char* fmt, ...);
 int check_cuda(rbffd_ctx* ctx, cudaError_t e, const char* what);
+// Device memory of a solver that another form stands in for (the direct and
+// the resident solves), and what its builder returns for `rc`: out of memory
+// leaves no trace in the context or the runtime, the other form takes over.
+cudaError_t solver_malloc(const rbffd_ctx* ctx, void** out, size_t bytes);
+int solver_left_out(rbffd_ctx* ctx, int rc);
+// whether `grid` blocks of a cooperative kernel fit the device at once
+bool coop_fits(const void* fn, int grid, int threads, size_t smem);
 // grow-only device scratch of the context
 int ctx_scratch(rbffd_ctx* ctx, size_t bytes, void** out);
 

@@ -593,6 +593,10 @@ void vsolve_free(VSolve* v) {
   delete v;
 }
 
+static const void* vsolve_kernel(int k) {
+  return k == 28 ? (const void*)k_vsolve<28> : (const void*)k_vsolve<0>;
+}
+
 int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* idx,
                  const double* wu, const double* wv, VSolve** out, cudaStream_t st) {
   *out = nullptr;
@@ -609,20 +613,19 @@ int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* id
   a.w[0] = wu;
   a.w[1] = wv;
   auto get = [&](void** p, size_t bytes) {
-    int rc = check_cuda(ctx, cudaMalloc(p, bytes), "viscous solve alloc");
+    int rc = check_cuda(ctx, solver_malloc(ctx, p, bytes), "viscous solve alloc");
     if (rc) return rc;
     v->allocs.push_back(*p);
     return check_cuda(ctx, cudaMemsetAsync(*p, 0, bytes, st), "memset");
   };
-  int rc = 0;
-  if (!rc) rc = get((void**)&a.p, sizeof(double) * 2 * N);
+  int rc = get((void**)&a.p, sizeof(double) * 2 * N);
   if (!rc) rc = get((void**)&a.s, sizeof(double) * 2 * N);
   if (!rc) rc = get((void**)&a.partials, sizeof(double) * 2 * kVNV * v->grid);
   if (!rc) rc = get((void**)&a.arrivals, 2 * sizeof(unsigned int));
-  if (rc) {
+  if (rc || !coop_fits(vsolve_kernel(k), v->grid, kVT, 0)) {
     cudaStreamSynchronize(st);
     vsolve_free(v);
-    return rc;
+    return solver_left_out(ctx, rc);
   }
   *out = v;
   return RBFFD_OK;
@@ -642,9 +645,8 @@ cudaError_t vsolve_enqueue(VSolve* v, double* const* x, const double* const* b, 
   a.res = res;
   a.fail = fail;
   a.step = step;
-  const void* fn = a.k == 28 ? (const void*)k_vsolve<28> : (const void*)k_vsolve<0>;
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel(fn, dim3(v->grid), dim3(kVT), args, 0, st);
+  return cudaLaunchCooperativeKernel(vsolve_kernel(a.k), dim3(v->grid), dim3(kVT), args, 0, st);
 }
 
 struct DSolve {
@@ -664,11 +666,16 @@ namespace {
 template <typename T>
 int d_alloc(rbffd_ctx* ctx, DSolve* d, T** out, size_t count, cudaStream_t st) {
   void* ptr = nullptr;
-  const int rc = check_cuda(ctx, cudaMalloc(&ptr, sizeof(T) * count), "direct solve alloc");
+  const int rc =
+      check_cuda(ctx, solver_malloc(ctx, &ptr, sizeof(T) * count), "direct solve alloc");
   if (rc) return rc;
   d->allocs.push_back(ptr);
   *out = (T*)ptr;
   return check_cuda(ctx, cudaMemsetAsync(ptr, 0, sizeof(T) * count, st), "memset");
+}
+
+const void* dsolve_kernel(int k) {
+  return k == 28 ? (const void*)k_dsolve<28> : (const void*)k_dsolve<0>;
 }
 
 int invert(rbffd_ctx* ctx, DSolve* d, const InvArgs& in, const double* es, double* out, int* h_status,
@@ -723,29 +730,31 @@ int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   const size_t nn = (size_t)M * a.ldt;
   double* inv = nullptr;
   int rc = 0, bad = 0;
-  if (a.rows > kOwn)  // fewer SMs than the ownership tables assume
-    rc = -1;
-  if (!rc) rc = d_alloc(ctx, d, &inv, nn, st);
-  if (!rc) rc = d_alloc(ctx, d, &in.T, nn, st);
+  // fewer SMs than the ownership tables assume, or than the grids need
+  if (a.rows > kOwn || !coop_fits((const void*)k_dense_invert, d->grid, kPT, 0) ||
+      !coop_fits(dsolve_kernel(k), d->grid, kPT, 0))
+    bad = 1;
+  if (!bad) rc = d_alloc(ctx, d, &inv, nn, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &in.T, nn, st);
   void* work = in.T;
-  if (!rc) rc = d_alloc(ctx, d, &in.prow, (size_t)M, st);
-  if (!rc) rc = d_alloc(ctx, d, &in.cand_v, (size_t)2 * d->grid, st);
-  if (!rc) rc = d_alloc(ctx, d, &in.cand_r, (size_t)2 * d->grid, st);
-  if (!rc) rc = d_alloc(ctx, d, &in.status, 1, st);
-  if (!rc) rc = d_alloc(ctx, d, &a.partials, (size_t)2 * kNVMax * d->grid, st);
-  if (!rc) rc = d_alloc(ctx, d, &a.arrivals, 2, st);
-  if (!rc) rc = d_alloc(ctx, d, &a.res, 1, st);
-  if (!rc) rc = d_alloc(ctx, d, &a.r, (size_t)a.ldt, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &in.prow, (size_t)M, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &in.cand_v, (size_t)2 * d->grid, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &in.cand_r, (size_t)2 * d->grid, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &in.status, 1, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &a.partials, (size_t)2 * kNVMax * d->grid, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &a.arrivals, 2, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &a.res, 1, st);
+  if (!rc && !bad) rc = d_alloc(ctx, d, &a.r, (size_t)a.ldt, st);
   in.partials = a.partials;
   in.arrivals = a.arrivals;
   a.inv = inv;
-  if (!rc) rc = invert(ctx, d, in, es, inv, &bad, st);
+  if (!rc && !bad) rc = invert(ctx, d, in, es, inv, &bad, st);
   if (!rc && !bad) rc = check_cuda(ctx, cudaStreamSynchronize(st), "dense inverse sync");
   if (rc || bad) {
     cudaStreamSynchronize(st);
     dsolve_free(d);
     // singular to working precision, or no room: the Krylov solve takes over
-    return rc == RBFFD_ERR_CUDA ? rc : RBFFD_OK;
+    return solver_left_out(ctx, rc);
   }
   for (void*& q : d->allocs)  // the inversion's matrix is not needed any more
     if (q == work) {
@@ -765,9 +774,8 @@ cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PS
   a.res = res;
   a.fail = fail;
   a.step = step;
-  const void* fn = a.k == 28 ? (const void*)k_dsolve<28> : (const void*)k_dsolve<0>;
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel(fn, dim3(d->grid), dim3(kPT), args, 0, st);
+  return cudaLaunchCooperativeKernel(dsolve_kernel(a.k), dim3(d->grid), dim3(kPT), args, 0, st);
 }
 
 cudaError_t small_reset(VSolve* v, DSolve* d, int* fail, cudaStream_t st) {

@@ -695,7 +695,8 @@ namespace {
 template <typename T>
 int p_alloc(rbffd_ctx* ctx, PSolve* p, T** out, size_t count, cudaStream_t st) {
   void* ptr = nullptr;
-  int rc = check_cuda(ctx, cudaMalloc(&ptr, sizeof(T) * (count ? count : 1)), "pressure solve alloc");
+  int rc = check_cuda(ctx, solver_malloc(ctx, &ptr, sizeof(T) * (count ? count : 1)),
+                      "pressure solve alloc");
   if (rc) return rc;
   p->allocs.push_back(ptr);
   *out = (T*)ptr;
@@ -785,6 +786,13 @@ int fill(rbffd_ctx* ctx, PSolve* p, PArgs<T>& a, int64_t M, int64_t ld, int k,
 }
 
 template <typename T>
+const void* kernel_of(int k, int pt) {
+  if (pt == kLargePT)
+    return k == 28 ? (const void*)k_psolve<28, T, kLargePT> : (const void*)k_psolve<0, T, kLargePT>;
+  return k == 28 ? (const void*)k_psolve<28, T, kSmallPT> : (const void*)k_psolve<0, T, kSmallPT>;
+}
+
+template <typename T>
 PArgs<T>& args_of(PSolve* p);
 template <>
 PArgs<double>& args_of<double>(PSolve* p) {
@@ -806,10 +814,11 @@ int psolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   p->pt = M > kLargeRows ? kLargePT : kSmallPT;
   const int rc = mix ? fill(ctx, p, p->a32, M, ld, k, idx, w, es, a1, amg, st)
                      : fill(ctx, p, p->a64, M, ld, k, idx, w, es, a1, amg, st);
-  if (rc) {
+  const void* fn = mix ? kernel_of<float>(k, p->pt) : kernel_of<double>(k, p->pt);
+  if (rc || !coop_fits(fn, p->grid, p->pt, stage_room(p->pt))) {
     cudaStreamSynchronize(st);
     psolve_free(p);
-    return rc;
+    return solver_left_out(ctx, rc);
   }
   *out = p;
   return RBFFD_OK;
@@ -830,10 +839,7 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
   int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, sizeof(unsigned int), st), "memset");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
   if (rc) return rc;
-  const void* fn =
-      p->pt == kLargePT
-          ? (a.k == 28 ? (const void*)k_psolve<28, T, kLargePT> : (const void*)k_psolve<0, T, kLargePT>)
-          : (a.k == 28 ? (const void*)k_psolve<28, T, kSmallPT> : (const void*)k_psolve<0, T, kSmallPT>);
+  const void* fn = kernel_of<T>(a.k, p->pt);
   void* args[] = {&a};
   rc = check_cuda(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)stage_room(p->pt)),

@@ -24,7 +24,9 @@ struct PSolveResult {
 
 // Build the solve's copies for one plan: the scaled pressure operator (idx, w
 // [k][ld], rank-one column es, row sums a1; M rows) in the hierarchy's level-0
-// order, in FP64, or in FP32 when `mix` is set, and its work vectors.
+// order, in FP64, or in FP32 when `mix` is set, and its work vectors.  *out
+// stays null when the memory or the SMs do not suffice (the caller then solves
+// as separate launches), as in the builders below.
 int psolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* idx,
                  const double* w, const double* es, const double* a1, const Amg* amg, bool mix,
                  PSolve** out, cudaStream_t st);
@@ -50,8 +52,8 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
 constexpr int kDenseMax = 4096;
 struct DSolve;
 
-// *out stays null when the operator is numerically singular (the caller then
-// takes the Krylov solve).  Synchronises `st`.
+// *out stays null when the operator is numerically singular, too (the caller
+// then takes the Krylov solve).  Synchronises `st`.
 int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* idx,
                  const double* w, const double* es, DSolve** out, cudaStream_t st);
 void dsolve_free(DSolve* d);

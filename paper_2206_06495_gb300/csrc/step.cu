@@ -2282,8 +2282,10 @@ int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t
     if (p->ds && !p->mix && f.N <= 2 * kDenseMax) {
       TRY(vsolve_build(ctx, f.N, f.ld_v, p->k, p->open ? p->Hidx : f.vv_idx, p->Hw,
                        p->open ? p->Hw_v : p->Hw, &p->vis, st));
-      TRY(palloc(ctx, p, &p->fail, 1));
-      TRY(palloc(ctx, p, &p->small, kSmallBatch));
+      if (p->vis) {
+        TRY(palloc(ctx, p, &p->fail, 1));
+        TRY(palloc(ctx, p, &p->small, kSmallBatch));
+      }
     }
   }
 #undef TRY

@@ -123,6 +123,7 @@ PROTOTYPES = {
     "rbffd_probe_fma": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.POINTER(C.c_double),
                                   C.c_void_p]),
     "rbffd_debug_set_wait_limit": (C.c_int, [C.c_void_p, C.c_int64]),
+    "rbffd_debug_set_solver_bytes": (C.c_int, [C.c_void_p, C.c_int64]),
     "rbffd_ensemble_step": (C.c_int, [C.c_void_p, C.POINTER(FlowC), C.c_int32,
                                       C.POINTER(C.c_double), C.POINTER(StateC), C.c_void_p,
                                       C.c_void_p, C.c_int32, C.POINTER(Stats), C.c_void_p]),
@@ -518,6 +519,12 @@ def debug_set_wait_limit(ctx: Context, polls: int) -> None:
     """rbffd_debug_set_wait_limit (test hook): polls of the first staged-copy
     wait; 0 gives up at once, a negative value restores the default."""
     ctx.check(lib().rbffd_debug_set_wait_limit(ctx.handle, polls))
+
+
+def debug_set_solver_bytes(ctx: Context, nbytes: int) -> None:
+    """rbffd_debug_set_solver_bytes (test hook): allocations of the direct and
+    resident solves above nbytes are refused; a negative value lifts the limit."""
+    ctx.check(lib().rbffd_debug_set_solver_bytes(ctx.handle, nbytes))
 
 
 @dataclass

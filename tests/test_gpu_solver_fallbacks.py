@@ -1,0 +1,46 @@
+"""What stands in for a solve that cannot run: no memory for the direct or the
+resident solve, and a direct solve that does not reach the tolerance."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import rbffd_oracle as O  # noqa: E402
+from paper_2206_06495_gb300 import nodesets as ns  # noqa: E402
+
+
+def _d(a):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def _flow(n, limit=None, **kw):
+    from paper_2206_06495_gb300 import rbffd as R
+    nd = ns.jittered_cavity(n, 3)
+    ctx = R.Context(28, 7, 3)
+    if limit is not None:
+        R.debug_set_solver_bytes(ctx, limit)
+    tol = 1e-11 if kw.get("precision") else 1e-12
+    flow = R.flow_from_nodes(ctx, nd, **{**dict(Re=100.0, dt=0.08 / (n - 1), tol=tol), **kw})
+    gu, gv = (_d(g) for g in O.lid_bc(nd))
+    return R, ctx, flow, gu, gv
+
+
+# 20: a dense inverse of 1.28 MB, resident copies of at most 94 KB; 65: no
+# direct solve; a limit of 0 refuses every solver's memory, 500,000 the inverse
+@pytest.mark.parametrize("n,limit", [(20, 0), (20, 500000), (65, 0)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_out_of_memory_leaves_the_launched_solve(n, limit, precision):
+    """Three steps with the solvers' memory refused and without: velocities
+    within 1e-9 (MIXED 1e-6) and p~ within 1e-8 (1e-5), the bars between the
+    forms of the solve elsewhere."""
+    got = []
+    for lim in (limit, None):
+        R, ctx, flow, gu, gv = _flow(n, lim, precision=precision)
+        st = R.State.zeros(flow)
+        assert R.step(ctx, flow, st, gu, gv, 3)["steps"] == 3
+        got.append(st)
+    a, b = got
+    tu, tp = (1e-6, 1e-5) if precision else (1e-9, 1e-8)
+    assert max((a.u - b.u).abs().max(), (a.v - b.v).abs().max()) < tu
+    assert (a.pt - b.pt).abs().max() < tp * b.pt.abs().max()
