@@ -2988,17 +2988,24 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   // except where the launches of that one are profiled or its iterations
   // capped below a single cycle
   const bool direct = P->ds && !f.profile && f.max_iter >= kRestartLen;
-  if (f.precond && !direct) {
-    const int rc = need_precond(ctx, P, f, st);
+  KOp<double, double> H64{f.vv_idx, P->Hw, f.ld_v, f.N, k, 1, nullptr};
+  KOp<double, double> L64{P->Lidx, P->Lw, f.ld_p, f.M, P->kL, 0, P->es, nullptr};
+  KOp<float, float> H32{f.vv_idx, P->Hw32, f.ld_v, f.N, k, 1, nullptr, nullptr};
+  KOp<float, float> L32{P->Lidx, P->Lw32, f.ld_p, f.M, P->kL, 0, P->es32, nullptr};
+  const bool proj = P->proj != 0;
+  // what the Krylov pressure solve needs, built when a solve first asks for it
+  auto krylov = [&]() -> int {
+    const int rc = f.precond ? need_precond(ctx, P, f, st) : RBFFD_OK;
+    L64.a1 = P->a1;
+    L32.a1 = P->a1_32;
+    L32.diff = P->a1_32 ? 1 : 0;
+    if (MIX && f.precond && !proj) L32.tiles = P->Lt;
+    return rc;
+  };
+  if (!direct) {
+    const int rc = krylov();
     if (rc) return rc;
   }
-  KOp<double, double> H64{f.vv_idx, P->Hw, f.ld_v, f.N, k, 1, nullptr};
-  KOp<double, double> L64{P->Lidx, P->Lw, f.ld_p, f.M, P->kL, 0, P->es, nullptr, P->a1};
-  KOp<float, float> H32{f.vv_idx, P->Hw32, f.ld_v, f.N, k, 1, nullptr, nullptr};
-  KOp<float, float> L32{P->Lidx, P->Lw32, f.ld_p, f.M, P->kL, 0, P->es32, nullptr, P->a1_32};
-  L32.diff = P->a1_32 ? 1 : 0;
-  const bool proj = P->proj != 0;
-  if (MIX && f.precond && !proj) L32.tiles = P->Lt;
   (MIX ? H32.tiles : H64.tiles) = P->Ht;
   // open flows: one viscous operator per component on the shared index array
   KOp<double, double> Hu64{P->Hidx, P->Hw, f.ld_v, f.N, k, 1, nullptr};
@@ -3269,7 +3276,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       if (code == kFailPressure && h[bad].pres.status == 2)
         return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite pressure solve");
       if (code == kFailPressure)  // refinement at its rounding level above the tolerance
-        rc = need_precond(ctx, P, f, st);
+        rc = krylov();
       else if (h[bad].visc.status == 2)
         for (double* x : hx)
           if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(x, 0, sizeof(double) * f.N, st), "zero start");
@@ -3296,7 +3303,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       pr.converged = dr.converged;
       sweeps = dr.iters;
       // refinement at its rounding level above the tolerance: Krylov from here
-      if (!pr.converged && pr.status != 2) rc = need_precond(ctx, P, f, st);
+      if (!pr.converged && pr.status != 2) rc = krylov();
       if (rc) return rc;
     }
     if (direct && !resume && (pr.converged || pr.status == 2)) {

@@ -44,3 +44,28 @@ def test_out_of_memory_leaves_the_launched_solve(n, limit, precision):
     tu, tp = (1e-6, 1e-5) if precision else (1e-9, 1e-8)
     assert max((a.u - b.u).abs().max(), (a.v - b.v).abs().max()) < tu
     assert (a.pt - b.pt).abs().max() < tp * b.pt.abs().max()
+
+
+@pytest.mark.parametrize("limit", [None, 0])
+@pytest.mark.parametrize("group", [1, 6])
+def test_krylov_takes_over_from_a_stalled_direct_solve(limit, group):
+    """A tolerance of 1e-15 is below what the refinement's residual reaches;
+    the Krylov recurrence goes on from its iterate through all six steps, with
+    the hierarchy built then, whether or not there is memory for the resident
+    form.  Within 1e-9 and 1e-8 of the launched form alone: both solve to the
+    rounding level."""
+    got = []
+    for profile in (0, 1):
+        R, ctx, flow, gu, gv = _flow(20, profile=profile)
+        st = R.State.zeros(flow)
+        R.step(ctx, flow, st, gu, gv, 1)  # builds the plan, with its direct solve
+        if limit is not None:
+            R.debug_set_solver_bytes(ctx, limit)
+        flow.tol = 1e-15
+        for _ in range(6 // group):
+            assert R.step(ctx, flow, st, gu, gv, group)["steps"] == group
+        assert st.j == 7
+        got.append(st)
+    a, b = got
+    assert max((a.u - b.u).abs().max(), (a.v - b.v).abs().max()) < 1e-9
+    assert (a.pt - b.pt).abs().max() < 1e-8 * b.pt.abs().max()
