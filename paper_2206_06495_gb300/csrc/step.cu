@@ -3067,6 +3067,11 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   const double vtol = (MIX || P->open || f.tol < 1e-13) ? f.tol : std::max(f.tol * 1e-3, 1e-13);
   double* hx[2] = {P->uss, P->vss};
   const double* hb[2] = {P->ru, P->rv};
+  auto viscous_failed = [&](double relres, int iters, int status) {
+    return set_error(ctx, RBFFD_ERR_NOT_CONVERGED,
+                     "viscous solve: relative residual %.3e after %d iterations (status %d)",
+                     relres, iters, status);
+  };
   auto viscous = [&]() -> int {
     int rc = 0, sweeps = 0;
     SolveResult hr;
@@ -3118,9 +3123,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     if (hr.status == 2) return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite viscous solve");
     // a solve short of the tighter target but within the tolerance is accepted
     if (!hr.converged && !(hr.relres <= f.tol))
-      return set_error(ctx, RBFFD_ERR_NOT_CONVERGED,
-                       "viscous solve: relative residual %.3e after %d iterations (status %d)",
-                       hr.relres, hr.iters, hr.status);
+      return viscous_failed(hr.relres, hr.iters, hr.status);
     return RBFFD_OK;
   };
   // The pressure right side and initial guess.
@@ -3277,9 +3280,16 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
         return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite pressure solve");
       if (code == kFailPressure)  // refinement at its rounding level above the tolerance
         rc = krylov();
-      else if (h[bad].visc.status == 2)
+      else if (h[bad].visc.status == 2) {  // the guess may be what is not finite
         for (double* x : hx)
           if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(x, 0, sizeof(double) * f.N, st), "zero start");
+      } else {  // max_iter or the restarts are used up
+        if (stats) {
+          stats->helm_iters += h[bad].visc.iters;
+          stats->helm_relres = h[bad].visc.relres;
+        }
+        return viscous_failed(h[bad].visc.relres, h[bad].visc.iters, h[bad].visc.status);
+      }
       if (rc) return rc;
       resume = code;
       continue;
@@ -3293,7 +3303,8 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     const double* pbv[1] = {P->pb};
     SolveResult pr;
     const bool prof = f.profile != 0;
-    if (direct && !resume) {
+    bool done = false;  // by the direct solve
+    if (direct && resume != kFailPressure) {
       PSolveResult dr;
       rc = dsolve_run(ctx, P->ds, P->px, P->pb, f.tol, &dr, &P->launches, st);
       if (rc) return rc;
@@ -3303,10 +3314,11 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       pr.converged = dr.converged;
       sweeps = dr.iters;
       // refinement at its rounding level above the tolerance: Krylov from here
-      if (!pr.converged && pr.status != 2) rc = krylov();
+      done = pr.converged || pr.status == 2;
+      if (!done) rc = krylov();
       if (rc) return rc;
     }
-    if (direct && !resume && (pr.converged || pr.status == 2)) {
+    if (done) {
     } else if (proj) {  // the composed operator's rows are read directly (runtime width)
       if (MIX)
         rc = refine<0, 1, true>(ctx, P, L64, L32, px, pbv, f.tol, f.inner_tol, f.max_iter, &pr,

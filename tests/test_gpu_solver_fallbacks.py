@@ -69,3 +69,24 @@ def test_krylov_takes_over_from_a_stalled_direct_solve(limit, group):
     a, b = got
     assert max((a.u - b.u).abs().max(), (a.v - b.v).abs().max()) < 1e-9
     assert (a.pt - b.pt).abs().max() < 1e-8 * b.pt.abs().max()
+
+
+@pytest.mark.parametrize("profile", [0, 1])
+def test_iteration_cap_holds_for_the_viscous_solve(profile):
+    """A stiff viscous system that takes more than 84 iterations fails with 0.6
+    times as many (50 at least, so that the direct solve stays in place), in
+    the resident form and as separate launches, and leaves the state."""
+    its = None
+    for cap in (20000, None):
+        R, ctx, flow, gu, gv = _flow(33, Re=0.5, dt=0.05, profile=profile)
+        st = R.State.zeros(flow)
+        flow.max_iter = cap or int(0.6 * its)
+        if cap:
+            its = R.step(ctx, flow, st, gu, gv, 1)["helm_iters"]
+            assert its > 84
+            continue
+        with pytest.raises(R.RbffdError) as e:
+            R.step(ctx, flow, st, gu, gv, 1)
+        assert e.value.code == R.ERR_NOT_CONVERGED and "viscous" in str(e.value)
+        assert e.value.stats["steps"] == 0 and st.j == 0 and not st.u.any()
+        assert flow.max_iter <= e.value.stats["helm_iters"] <= flow.max_iter + 1
