@@ -1893,6 +1893,7 @@ __global__ void __launch_bounds__(kThreads)
 
 // Steps of a small flow enqueued before the host looks at their results.
 constexpr int kSmallBatch = 32;
+constexpr int kMaxHold = 64;
 
 struct StepPlan {
   rbffd_flow key;
@@ -1943,6 +1944,11 @@ struct StepPlan {
   PSolve* ps = nullptr;               // the preconditioned solve's resident kernel
   DSolve* ds = nullptr;               // small systems: the direct solve (amg and ps are then
                                       // built when something needs the Krylov solve)
+  // A direct solve that stalls above its tolerance is not tried again for
+  // `hold` steps, twice as many after each further stall (at most kMaxHold), as
+  // long as the tolerance is not loosened.
+  int hold = 0, hold_len = 0;
+  double hold_tol = 0.0;
   double* a1 = nullptr;    // row sums of the FP64 pressure operator
   float* a1_32 = nullptr;  // the same in FP32 (complement of the difference-form FP32 rows)
   // tile records of the pressure and viscous operators the Krylov solves
@@ -3002,7 +3008,14 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     if (MIX && f.precond && !proj) L32.tiles = P->Lt;
     return rc;
   };
-  if (!direct) {
+  if (f.tol > P->hold_tol) P->hold = P->hold_len = 0;
+  auto stalled = [&]() {
+    P->hold_len = std::min(std::max(1, 2 * P->hold_len), kMaxHold);
+    P->hold = P->hold_len;
+    P->hold_tol = f.tol;
+    return krylov();
+  };
+  if (!direct || P->hold > 0) {
     const int rc = krylov();
     if (rc) return rc;
   }
@@ -3204,8 +3217,10 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
   // before that solve stands, and the launch by launch one starts from its iterate
   int resume = 0;
   for (int32_t step = 0; step < n_steps;) {
-    if (ahead && !resume) {
-      const int batch = std::min<int32_t>(n_steps - step, kSmallBatch);
+    const bool held = P->hold > 0, now = direct && !held;
+    if (ahead && now && !resume) {
+      // after a stall one step at a time, until one passes
+      const int batch = P->hold_len ? 1 : std::min<int32_t>(n_steps - step, kSmallBatch);
       Mark marks[kSmallBatch];
       const int64_t j0 = s->j;
       int rc = check_cuda(ctx, small_reset(P->vis, P->ds, P->fail, st), "step reset");
@@ -3265,6 +3280,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
                   h[i].visc.iters, h[i].visc.relres, h[i].pres.iters, h[i].pres.relres);
       }
       step += bad;
+      if (bad > 0) P->hold_len = 0;
       if (!code) continue;
       const Mark& m = marks[bad];
       const int after = code == kFailPressure ? 1 : 0;
@@ -3279,7 +3295,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       if (code == kFailPressure && h[bad].pres.status == 2)
         return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite pressure solve");
       if (code == kFailPressure)  // refinement at its rounding level above the tolerance
-        rc = krylov();
+        rc = stalled();
       else if (h[bad].visc.status == 2) {  // the guess may be what is not finite
         for (double* x : hx)
           if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(x, 0, sizeof(double) * f.N, st), "zero start");
@@ -3304,7 +3320,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
     SolveResult pr;
     const bool prof = f.profile != 0;
     bool done = false;  // by the direct solve
-    if (direct && resume != kFailPressure) {
+    if (now) {
       PSolveResult dr;
       rc = dsolve_run(ctx, P->ds, P->px, P->pb, f.tol, &dr, &P->launches, st);
       if (rc) return rc;
@@ -3315,7 +3331,8 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       sweeps = dr.iters;
       // refinement at its rounding level above the tolerance: Krylov from here
       done = pr.converged || pr.status == 2;
-      if (!done) rc = krylov();
+      if (pr.converged) P->hold_len = 0;
+      if (!done) rc = stalled();
       if (rc) return rc;
     }
     if (done) {
@@ -3350,6 +3367,7 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
                        pr.relres, pr.iters, pr.status);
     rc = back(nullptr);
     if (rc) return rc;
+    if (held && !resume) --P->hold;
     resume = 0;
     s->j += 1;
     P->px_step = s->j;

@@ -90,3 +90,35 @@ def test_iteration_cap_holds_for_the_viscous_solve(profile):
         assert e.value.code == R.ERR_NOT_CONVERGED and "viscous" in str(e.value)
         assert e.value.stats["steps"] == 0 and st.j == 0 and not st.u.any()
         assert flow.max_iter <= e.value.stats["helm_iters"] <= flow.max_iter + 1
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_stalled_direct_solve_is_not_tried_at_every_step(precision):
+    """32 steps in one call launch no more than 1.5 times what 32 calls do (a
+    batch of 32 steps enqueued again after each stall launches three times as
+    much), give their bits, and a loosened tolerance has the direct solve back
+    at once (at most 8 products a step).  MIXED flows stall at the rounding level of
+    the FP64 residual, where the Krylov solve stalls, too: the call reports it."""
+    runs = []
+    for group in (32, 1):
+        R, ctx, flow, gu, gv = _flow(20, precision=precision)
+        st = R.State.zeros(flow)
+        R.step(ctx, flow, st, gu, gv, 1)
+        flow.tol = 1e-16
+        if precision:
+            with pytest.raises(R.RbffdError) as e:
+                R.step(ctx, flow, st, gu, gv, group)
+            assert e.value.code == R.ERR_NOT_CONVERGED and st.j == 1
+        launches = 0
+        if not precision:
+            flow.tol = 1e-15
+            for _ in range(32 // group):
+                launches += R.step(ctx, flow, st, gu, gv, group)["launches"]
+            assert st.j == 33
+        runs.append((launches, st))
+        flow.tol = 1e-11
+        other = R.State.zeros(flow)
+        assert R.step(ctx, flow, other, gu, gv, 4)["poisson_iters"] <= 4 * 8
+    (a, x), (b, y) = runs
+    assert a <= 1.5 * b
+    assert torch.equal(x.u, y.u) and torch.equal(x.pt, y.pt)
