@@ -207,12 +207,31 @@ void permute(const HostCsr& A, const std::vector<int32_t>& old, const std::vecto
   }
 }
 
-// Dense inverse of (A + sigma 1 1^T + eps diag(A)) by Cholesky, row-major.
+// The hierarchy's levels from (*L)[0] down, and the aggregates of each.
+void coarsen(std::vector<HostCsr>* L, std::vector<std::vector<int32_t>>* aggs) {
+  while (L->back().n > kAmgCoarse && (int)L->size() < kAmgMaxLevels) {
+    const HostCsr& A = L->back();
+    std::vector<int32_t> a1, a2;
+    HostCsr A1, A2;
+    const int32_t n1 = pairwise(A, &a1);
+    galerkin(A, a1, n1, &A1);
+    const int32_t n2 = pairwise(A1, &a2);
+    galerkin(A1, a2, n2, &A2);
+    if ((double)n2 > 0.85 * (double)A.n) break;  // no longer coarsening
+    for (auto& v : a1) v = a2[v];
+    aggs->push_back(std::move(a1));
+    L->push_back(std::move(A2));
+  }
+}
+
+// Lower Cholesky factor, row-major, of the dense A + sigma 1 1^T + eps diag(A).
 // sigma lifts the constant null vector of the Laplacian to the mean diagonal;
-// eps = 1e-10 keeps the factorisation defined if the graph falls apart.
-bool coarse_inverse(const HostCsr& A, std::vector<double>* X, bool singular) {
+// eps = 1e-10 keeps the factorisation defined if the graph falls apart.  False
+// if a pivot is not positive.
+bool coarse_factor(const HostCsr& A, std::vector<double>* out, bool singular) {
   const int64_t n = A.n;
-  std::vector<double> B(n * n, 0.0);
+  std::vector<double>& B = *out;
+  B.assign(n * n, 0.0);
   double dm = 0.0;
   for (int64_t i = 0; i < n; ++i) dm += A.diag[i];
   dm /= (double)n;
@@ -238,6 +257,14 @@ bool coarse_inverse(const HostCsr& A, std::vector<double>* X, bool singular) {
       B[i * n + j] = s / ljj;
     }
   }
+  return true;
+}
+
+// Dense inverse of the matrix that coarse_factor factors, row-major.
+bool coarse_inverse(const HostCsr& A, std::vector<double>* X, bool singular) {
+  const int64_t n = A.n;
+  std::vector<double> B;
+  if (!coarse_factor(A, &B, singular)) return false;
   // W = L^-1 (stored transposed: WT[c][i] = W[i][c]), then X = W^T W
   std::vector<double> WT(n * n, 0.0), t(n);
   for (int64_t c = 0; c < n; ++c) {
@@ -367,22 +394,48 @@ bool has_dirichlet(const std::vector<uint8_t>& bc) {
   return std::find(bc.begin(), bc.end(), (uint8_t)RBFFD_PBC_DIRICHLET) != bc.end();
 }
 
+int not_positive(rbffd_ctx* ctx) {
+  return set_error(ctx, RBFFD_ERR_INVALID_ARG, "coarsest pressure graph matrix is not positive");
+}
+
+int check_coarsest(rbffd_ctx* ctx, const HostCsr& A) {
+  if (A.n <= 8 * kAmgCoarse) return RBFFD_OK;
+  return set_error(ctx, RBFFD_ERR_INVALID_ARG,
+                   "pressure graph does not coarsen below %lld nodes (disconnected?)",
+                   (long long)A.n);
+}
+
 }  // namespace
 
 int amg_check(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const double* es,
               cudaStream_t st) {
-  HostCsr G;
+  std::vector<HostCsr> L(1);
   std::vector<uint8_t> bc;
-  const int rc = load_graph(ctx, f, &G, &bc, st);
+  int rc = load_graph(ctx, f, &L[0], &bc, st);
   if (rc) return rc;
+  const HostCsr& G = L[0];
   double ces = 0.0;
   for (int64_t i = 0; i < f.M; ++i) {
-    if (!std::isfinite(G.diag[i]))
-      return set_error(ctx, RBFFD_ERR_INVALID_ARG, "coarsest pressure graph matrix is not positive");
+    if (!std::isfinite(G.diag[i])) return not_positive(ctx);
     ces += (diag_a[i] != 0.0 ? G.diag[i] / diag_a[i] : G.diag[i]) * es[i];
   }
-  if (!has_dirichlet(bc) && (!(ces != 0.0) || !std::isfinite(ces)))
+  const bool pdir = has_dirichlet(bc);
+  if (!pdir && (!(ces != 0.0) || !std::isfinite(ces)))
     return set_error(ctx, RBFFD_ERR_INVALID_ARG, "pressure rank-one column is zero");
+  std::vector<std::vector<int32_t>> aggs;
+  coarsen(&L, &aggs);
+  if ((rc = check_coarsest(ctx, L.back()))) return rc;
+  // The factorisation, the one check that takes long (n^3 / 3 multiply-adds), is
+  // made only where the coarsest diagonal varies enough for a pivot to be lost
+  // to rounding: the pivots are at least eps = 1e-10 of the diagonal, and the
+  // rounding of a dense row is below 1e-12 of it up to a ratio of 1e4 (node
+  // sets graded by 10 have 1e2; two P-nodes of a 20 x 20 set that almost
+  // coincide fail the factorisation from a ratio of about 1e19 on).
+  const std::vector<double>& d = L.back().diag;
+  const auto mm = std::minmax_element(d.begin(), d.end());
+  std::vector<double> B;
+  if (!(*mm.second <= 1e4 * *mm.first) && !coarse_factor(L.back(), &B, !pdir))
+    return not_positive(ctx);
   return RBFFD_OK;
 }
 
@@ -395,27 +448,11 @@ int amg_build(rbffd_ctx* ctx, const rbffd_flow& f, const double* diag_a, const d
   int rc = load_graph(ctx, f, &L[0], &bc, st);
   if (rc) return rc;
   std::vector<std::vector<int32_t>> aggs;
-  while (L.back().n > kAmgCoarse && (int)L.size() < kAmgMaxLevels) {
-    const HostCsr& A = L.back();
-    std::vector<int32_t> a1, a2;
-    HostCsr A1, A2;
-    const int32_t n1 = pairwise(A, &a1);
-    galerkin(A, a1, n1, &A1);
-    const int32_t n2 = pairwise(A1, &a2);
-    galerkin(A1, a2, n2, &A2);
-    if ((double)n2 > 0.85 * (double)A.n) break;  // no longer coarsening
-    for (auto& v : a1) v = a2[v];
-    aggs.push_back(std::move(a1));
-    L.push_back(std::move(A2));
-  }
-  if (L.back().n > 8 * kAmgCoarse)
-    return set_error(ctx, RBFFD_ERR_INVALID_ARG,
-                     "pressure graph does not coarsen below %lld nodes (disconnected?)",
-                     (long long)L.back().n);
+  coarsen(&L, &aggs);
+  if ((rc = check_coarsest(ctx, L.back()))) return rc;
   const bool pdir = has_dirichlet(bc);
   std::vector<double> Xd;
-  if (!coarse_inverse(L.back(), &Xd, !pdir))
-    return set_error(ctx, RBFFD_ERR_INVALID_ARG, "coarsest pressure graph matrix is not positive");
+  if (!coarse_inverse(L.back(), &Xd, !pdir)) return not_positive(ctx);
 
   // Nested ordering, coarsest to finest: the coarsest level keeps its order,
   // and each finer level lists its rows aggregate by aggregate in the coarser

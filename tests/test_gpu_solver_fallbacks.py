@@ -122,3 +122,22 @@ def test_a_stalled_direct_solve_is_not_tried_at_every_step(precision):
     (a, x), (b, y) = runs
     assert a <= 1.5 * b
     assert torch.equal(x.u, y.u) and torch.equal(x.pt, y.pt)
+
+
+@pytest.mark.parametrize("profile", [0, 1])
+def test_pressure_graphs_are_refused_alike(profile):
+    """A graph whose coarsest matrix is not positive (two P-nodes of an edge
+    1e-14 apart, whose weight of 1e28 leaves nothing of the others) is refused
+    when the plan is built, by the hierarchy and by a flow solved directly."""
+    R, ctx, flow, gu, gv = _flow(20, profile=profile)
+    e, bc = flow.tensors["p_edges"], flow.tensors["p_bc"].bool()
+    a, b = (int(v) for v in e[~bc[e[:, 0].long()] & ~bc[e[:, 1].long()]][50])
+    for k in ("px", "py"):
+        flow.tensors[k] = flow.tensors[k].clone()
+        flow.tensors[k][b] = flow.tensors[k][a]
+    flow.tensors["px"][b] += 1e-14
+    st = R.State.zeros(flow)
+    with pytest.raises(R.RbffdError) as err:
+        R.step(ctx, flow, st, gu, gv, 1)
+    assert err.value.code == R.ERR_INVALID_ARG and "not positive" in str(err.value)
+    assert st.j == 0
