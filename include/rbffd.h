@@ -449,6 +449,17 @@ int rbffd_stencil_error(rbffd_ctx* ctx, const rbffd_ell* D, uint32_t op, const d
 int rbffd_debug_set_wait_limit(rbffd_ctx* ctx, int64_t polls);
 
 /*
+ * rbffd_debug_set_barrier_limit - test hook (no counterpart in the paper): the
+ * number of polls a block of this context's direct and resident solves spends
+ * on a grid barrier before it gives up (at least one; at most the default,
+ * 2^22).  A block that gives up sets the solve's error flag and returns; the
+ * call then fails with RBFFD_ERR_CUDA ("... bounded wait") and the context
+ * stays usable.  polls < 0 restores the default.
+ * Errors: INVALID_ARG (null ctx).
+ */
+int rbffd_debug_set_barrier_limit(rbffd_ctx* ctx, int64_t polls);
+
+/*
  * rbffd_debug_set_solver_bytes - test hook (no counterpart in the paper): in
  * plans that this context builds from now on, an allocation of more than
  * `bytes` bytes for the direct or a resident solve is refused as if the

@@ -362,6 +362,13 @@ int rbffd_debug_set_solver_bytes(rbffd_ctx* ctx, int64_t bytes) {
   return RBFFD_OK;
 }
 
+int rbffd_debug_set_barrier_limit(rbffd_ctx* ctx, int64_t polls) {
+  if (!ctx) return RBFFD_ERR_INVALID_ARG;
+  ctx->err.clear();
+  ctx->barrier_limit = polls < 0 ? -1 : polls;
+  return RBFFD_OK;
+}
+
 int rbffd_debug_set_wait_limit(rbffd_ctx* ctx, int64_t polls) {
   if (!ctx) return RBFFD_ERR_INVALID_ARG;
   ctx->err.clear();

@@ -107,6 +107,7 @@ struct rbffd_ctx {
   void* host_pinned = nullptr;  // small pinned buffer for status words
   rbffd::StepPlan* plan = nullptr;
   rbffd::EnsPlan* ens = nullptr;  // ensemble step plan (rbffd_ensemble_step)
+  int64_t barrier_limit = -1;     // rbffd_debug_set_barrier_limit (-1: the default)
   int64_t solver_bytes = -1;      // rbffd_debug_set_solver_bytes: largest allocation (-1: any)
   // launch shapes the SpMV autotuner picked, per operator shape key
   std::vector<std::pair<uint64_t, int>> spmv_shapes;

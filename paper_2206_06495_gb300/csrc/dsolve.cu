@@ -41,7 +41,8 @@ struct InvArgs {
   double* cand_v;        // [2][gridDim.x] each block's best pivot candidate
   int* cand_r;           // [2][gridDim.x]
   double* partials;
-  unsigned int* arrivals;  // zero at launch
+  unsigned int* arrivals;  // [kBarrierWords], zero at launch
+  long long polls;
   int* status;             // 0 on entry; 1: singular, 2: non-finite
 };
 
@@ -60,7 +61,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dense_invert(const __grid_constant__
   __shared__ double part[kNVMax * 4];
   __shared__ double f[kOwn], cv[kOwn], s_inv;
   __shared__ int used[kOwn], okf, s_p, s_bad;
-  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals, a.polls};
   const int tid = threadIdx.x, n = a.n, nb = gridDim.x, blk = blockIdx.x;
   const int own = blk < n ? (n - blk + nb - 1) / nb : 0;
   if (tid < kOwn) {
@@ -179,16 +180,22 @@ struct DArgs {
   double *x, *r;  // r: ldt values, zero beyond M
   double tol2;
   double* partials;
-  unsigned int* arrivals;  // two words, zero between launches
+  unsigned int* arrivals;  // [kBarrierWords], zero between launches
+  long long polls;
   PSolveResult* res;
   int* fail;  // null, or see psolve.cuh
   int step;
 };
 
+// what ended the step: the code of a wait outranks the others
+template <typename A>
+__device__ __forceinline__ void set_fail(const A& a, int code) {
+  atomicMax(a.fail, (a.step << 4) | code);
+}
 // a barrier that ran out of its bounded wait
 template <typename A>
 __device__ __forceinline__ void give_up(const A& a) {
-  if (a.fail && threadIdx.x == 0) *a.fail = (a.step << 4) | kFailWait;
+  if (a.fail && threadIdx.x == 0) set_fail(a, kFailWait);
 }
 
 // Refinement: r = b - A_f x, x += A_f^-1 r until (r, r) <= tol^2 (b, b).  A
@@ -204,7 +211,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
   __shared__ double part[kNVMax * 4];
   __shared__ double s_sig, s_rr, s_bb;
   __shared__ int okf;
-  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<kPT> g{sh, part, &okf, a.partials, a.arrivals, a.polls};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = min(a.M, a.rows * (int)blockIdx.x), r1 = min(a.M, r0 + a.rows);
   const int active = min(kPT, (a.rows + 31) / 32 * 32);
@@ -250,7 +257,7 @@ __global__ void __launch_bounds__(kPT, 1) k_dsolve(const __grid_constant__ DArgs
         a.res->status = conv ? 0 : (fin ? 5 : 2);
         a.res->relres = bb > 0 ? sqrt(rr / bb) : sqrt(rr);
         a.res->converged = conv;
-        if (a.fail && !conv) *a.fail = (a.step << 4) | kFailPressure;
+        if (a.fail && !conv) set_fail(a, kFailPressure);
       }
       return leave(a.arrivals);
     }
@@ -303,7 +310,8 @@ struct VArgs {
   double tol2, accept2;
   int maxit;
   double* partials;        // [2][kVNV][gridDim.x]
-  unsigned int* arrivals;  // two words, zero between launches
+  unsigned int* arrivals;  // [kBarrierWords], zero between launches
+  long long polls;
   PSolveResult* res;
   int* fail;
   int step;
@@ -337,7 +345,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
   __shared__ double wsum[kVNV * (kVT / 32)];
   __shared__ VScal S;
   __shared__ int okf;
-  Grid<kVT, kVNV> g{nullptr, nullptr, &okf, a.partials, a.arrivals};
+  Grid<kVT, kVNV> g{nullptr, nullptr, &okf, a.partials, a.arrivals, a.polls};
   const int tid = threadIdx.x, sub = tid & (kVL - 1), c = sub & 1;
   const int i = a.rows * (int)blockIdx.x + tid / kVL;
   const bool mine = tid / kVL < a.rows && i < a.N;
@@ -569,7 +577,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
         a.res->status = st;
         a.res->relres = worst;
         a.res->converged = conv;
-        if (st == 2 || (!conv && !near)) *a.fail = (a.step << 4) | kFailViscous;
+        if (st == 2 || (!conv && !near)) set_fail(a, kFailViscous);
       }
       return leave(a.arrivals);
     }
@@ -580,6 +588,10 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
 }
 
 }  // namespace
+
+long long barrier_polls(const rbffd_ctx* ctx) {
+  return ctx->barrier_limit < 0 ? kPolls : std::min<long long>(ctx->barrier_limit, kPolls);
+}
 
 struct VSolve {
   std::vector<void*> allocs;
@@ -621,7 +633,7 @@ int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* id
   int rc = get((void**)&a.p, sizeof(double) * 2 * N);
   if (!rc) rc = get((void**)&a.s, sizeof(double) * 2 * N);
   if (!rc) rc = get((void**)&a.partials, sizeof(double) * 2 * kVNV * v->grid);
-  if (!rc) rc = get((void**)&a.arrivals, 2 * sizeof(unsigned int));
+  if (!rc) rc = get((void**)&a.arrivals, kBarrierWords * sizeof(unsigned int));
   if (rc || !coop_fits(vsolve_kernel(k), v->grid, kVT, 0)) {
     cudaStreamSynchronize(st);
     vsolve_free(v);
@@ -633,8 +645,9 @@ int vsolve_build(rbffd_ctx* ctx, int64_t N, int64_t ld, int k, const int32_t* id
 
 cudaError_t vsolve_enqueue(VSolve* v, double* const* x, const double* const* b, double tol,
                            double accept, int maxit, PSolveResult* res, int* fail, int step,
-                           cudaStream_t st) {
+                           long long polls, cudaStream_t st) {
   VArgs a = v->a;
+  a.polls = polls;
   for (int q = 0; q < 2; ++q) {
     a.x[q] = x[q];
     a.b[q] = b[q];
@@ -690,16 +703,16 @@ int invert(rbffd_ctx* ctx, DSolve* d, const InvArgs& in, const double* es, doubl
                                                    dim3(kPT), args, 0, st), "dense inverse");
   if (rc) return rc;
   int* h = (int*)ctx->host_pinned;
-  unsigned int* arrived = (unsigned int*)(h + 1);
+  unsigned int* gave_up = (unsigned int*)(h + 1);
   rc = check_cuda(ctx, cudaMemcpyAsync(h, in.status, sizeof(int), cudaMemcpyDeviceToHost, st),
                   "inverse status");
   if (!rc)
-    rc = check_cuda(ctx, cudaMemcpyAsync(arrived, in.arrivals, sizeof(unsigned int),
+    rc = check_cuda(ctx, cudaMemcpyAsync(gave_up, in.arrivals + 2, sizeof(unsigned int),
                                          cudaMemcpyDeviceToHost, st), "inverse status");
   if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "dense inverse sync");
   if (rc) return rc;
   *h_status = *h;
-  if (*h == 0 && *arrived != (unsigned int)d->grid * ((unsigned int)a.M + 1u))
+  if (*gave_up)
     return set_error(ctx, RBFFD_ERR_CUDA, "dense inverse: grid barrier not reached (bounded wait)");
   if (*h == 0) {
     k_dense_order<<<a.M, 256, 0, st>>>(a.M, a.ldt, in.prow, in.T, out);
@@ -742,11 +755,16 @@ int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
   if (!rc && !bad) rc = d_alloc(ctx, d, &in.cand_r, (size_t)2 * d->grid, st);
   if (!rc && !bad) rc = d_alloc(ctx, d, &in.status, 1, st);
   if (!rc && !bad) rc = d_alloc(ctx, d, &a.partials, (size_t)2 * kNVMax * d->grid, st);
-  if (!rc && !bad) rc = d_alloc(ctx, d, &a.arrivals, 2, st);
-  if (!rc && !bad) rc = d_alloc(ctx, d, &a.res, 1, st);
+  SolveStatus* status = nullptr;
+  if (!rc && !bad) rc = d_alloc(ctx, d, &status, 1, st);
   if (!rc && !bad) rc = d_alloc(ctx, d, &a.r, (size_t)a.ldt, st);
+  if (status) {
+    a.res = &status->res;
+    a.arrivals = status->bar;
+  }
   in.partials = a.partials;
   in.arrivals = a.arrivals;
+  in.polls = barrier_polls(ctx);
   a.inv = inv;
   if (!rc && !bad) rc = invert(ctx, d, in, es, inv, &bad, st);
   if (!rc && !bad) rc = check_cuda(ctx, cudaStreamSynchronize(st), "dense inverse sync");
@@ -766,8 +784,9 @@ int dsolve_build(rbffd_ctx* ctx, int64_t M, int64_t ld, int k, const int32_t* id
 }
 
 cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PSolveResult* res,
-                           int* fail, int step, cudaStream_t st) {
+                           int* fail, int step, long long polls, cudaStream_t st) {
   DArgs a = d->a;
+  a.polls = polls;
   a.x = x;
   a.b = b;
   a.tol2 = tol * tol;
@@ -779,29 +798,30 @@ cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PS
 }
 
 cudaError_t small_reset(VSolve* v, DSolve* d, int* fail, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(v->a.arrivals, 0, 2 * sizeof(unsigned int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d->a.arrivals, 0, 2 * sizeof(unsigned int), st);
+  constexpr size_t words = kBarrierWords * sizeof(unsigned int);
+  cudaError_t e = cudaMemsetAsync(v->a.arrivals, 0, words, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d->a.arrivals, 0, words, st);
   return e == cudaSuccess ? cudaMemsetAsync(fail, 0, sizeof(int), st) : e;
 }
 
 int dsolve_run(rbffd_ctx* ctx, DSolve* d, double* x, const double* b, double tol,
                PSolveResult* res, int64_t* launches, cudaStream_t st) {
-  PSolveResult* h = (PSolveResult*)ctx->host_pinned;
+  SolveStatus* h = (SolveStatus*)ctx->host_pinned;
   const DArgs& a = d->a;
-  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, 2 * sizeof(unsigned int), st), "memset");
-  if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
+  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, kBarrierWords * sizeof(unsigned int), st),
+                      "memset");
   if (!rc)
-    rc = check_cuda(ctx, dsolve_enqueue(d, x, b, tol, a.res, nullptr, 0, st),
+    rc = check_cuda(ctx, dsolve_enqueue(d, x, b, tol, a.res, nullptr, 0, barrier_polls(ctx), st),
                     "direct pressure solve");
   if (!rc)
-    rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(PSolveResult), cudaMemcpyDeviceToHost, st),
+    rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(SolveStatus), cudaMemcpyDeviceToHost, st),
                     "direct solve result");
   if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "direct solve sync");
   if (rc) return rc;
   *launches += 1;
-  if (h->iters < 0)  // the kernel gave up before it could write its result
+  if (h->bar[2])
     return set_error(ctx, RBFFD_ERR_CUDA, "direct solve: grid barrier not reached (bounded wait)");
-  *res = *h;
+  *res = h->res;
   return RBFFD_OK;
 }
 

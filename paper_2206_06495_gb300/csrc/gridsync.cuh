@@ -6,7 +6,11 @@
 namespace rbffd {
 
 constexpr int kNVMax = 4;  // values reduced together, where a kernel does not say otherwise
-constexpr long long kPolls = 1ll << 22;  // bounded barrier wait (a phase takes microseconds)
+// bounded barrier wait (a phase takes microseconds), where a test does not
+// lower it through rbffd_debug_set_barrier_limit
+constexpr long long kPolls = 1ll << 22;
+// The barrier's three words, `arrivals`: blocks arrived, blocks that have left
+// (see leave()), and 1 once a block has given up a wait.
 
 // The block's share of the grid-wide machinery.  Every block sees the same
 // totals, so every block takes the same decisions.
@@ -18,12 +22,14 @@ struct Grid {
   int* ok;                 // shared: the last barrier's verdict
   double* partials;
   unsigned int* arrivals;
+  long long limit;  // polls of a wait
   unsigned int target = 0;
   int phase = 0;
 
   // All blocks' writes before it are visible to all blocks after it.  Returns
   // false (in every thread of the block) if the other blocks did not arrive
-  // within the bounded wait.
+  // within the bounded wait.  The block then sets arrivals[2]: at the last
+  // barrier of a kernel the others may have passed.
   __device__ __forceinline__ bool sync() {
     __syncthreads();
     target += gridDim.x;
@@ -36,8 +42,9 @@ struct Grid {
       long long polls = 0;
       do {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(arrivals) : "memory");
-      } while ((int)(got - target) < 0 && ++polls < kPolls);
+      } while ((int)(got - target) < 0 && ++polls < limit);
       *ok = (int)(got - target) >= 0;
+      if (!*ok) arrivals[2] = 1u;
     }
     __syncthreads();
     return *ok != 0;
@@ -103,8 +110,8 @@ struct Grid {
   }
 };
 
-// Ends a kernel whose arrival counter (two words) the next launch finds at
-// zero again: the last block to come here resets it.
+// Ends a kernel whose arrival counter the next launch finds at zero again: the
+// last block to come here resets it.
 __device__ __forceinline__ void leave(unsigned int* arrivals) {
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(arrivals + 1, 1u) == gridDim.x - 1u) {

@@ -88,7 +88,8 @@ struct PArgs {
   int maxit, x_zero;
   uint32_t seed;
   double* partials;        // [2][kNVMax][gridDim.x], alternating
-  unsigned int* arrivals;  // zero at launch
+  unsigned int* arrivals;  // [kBarrierWords], zero at launch
+  long long polls;
   PSolveResult* res;
 };
 
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
   __shared__ double part[kNVMax * 4];
   __shared__ PScal<T> S;
   __shared__ int okf, first[kAmgMaxLevels], count[kAmgMaxLevels];
-  Grid<PT> g{sh, part, &okf, a.partials, a.arrivals};
+  Grid<PT> g{sh, part, &okf, a.partials, a.arrivals, a.polls};
   const int tid = threadIdx.x;
   const int r0 = min(a.M, a.rows * (int)blockIdx.x), r1 = min(a.M, r0 + a.rows);
   const int active = min(PT, a.rows);
@@ -738,6 +739,7 @@ int fill(rbffd_ctx* ctx, PSolve* p, PArgs<T>& a, int64_t M, int64_t ld, int k,
   a.nlev = amg->nlev;
   a.nc = (int)amg->nc;
   a.ldx = (int)round_up(amg->nc, 4);
+  SolveStatus* status = nullptr;
   float* X = nullptr;
   if ((rc = p_alloc(ctx, p, &X, (size_t)a.nc * a.ldx, st))) return rc;
   if ((rc = check_cuda(ctx, cudaMemcpy2DAsync(X, sizeof(float) * a.ldx, amg->Xc,
@@ -780,8 +782,10 @@ int fill(rbffd_ctx* ctx, PSolve* p, PArgs<T>& a, int64_t M, int64_t ld, int k,
   a.inv_ces = amg->inv_ces;
   a.inv_R = amg->inv_R;
   if ((rc = p_alloc(ctx, p, &a.partials, (size_t)2 * kNVMax * p->grid, st)) ||
-      (rc = p_alloc(ctx, p, &a.arrivals, 1, st)) || (rc = p_alloc(ctx, p, &a.res, 1, st)))
+      (rc = p_alloc(ctx, p, &status, 1, st)))
     return rc;
+  a.res = &status->res;
+  a.arrivals = status->bar;
   return RBFFD_OK;
 }
 
@@ -835,9 +839,10 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
   a.maxit = maxit;
   a.seed = seed;
   a.x_zero = x_zero ? 1 : 0;
-  PSolveResult* h = (PSolveResult*)ctx->host_pinned;
-  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, sizeof(unsigned int), st), "memset");
-  if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(a.res, 0xff, sizeof(PSolveResult), st), "memset");
+  a.polls = barrier_polls(ctx);
+  SolveStatus* h = (SolveStatus*)ctx->host_pinned;
+  int rc = check_cuda(ctx, cudaMemsetAsync(a.arrivals, 0, kBarrierWords * sizeof(unsigned int), st),
+                      "memset");
   if (rc) return rc;
   const void* fn = kernel_of<T>(a.k, p->pt);
   void* args[] = {&a};
@@ -848,14 +853,14 @@ int psolve_run(rbffd_ctx* ctx, PSolve* p, T* x, const T* b, double tol, int maxi
     rc = check_cuda(ctx, cudaLaunchCooperativeKernel(fn, dim3(p->grid), dim3(p->pt), args, p->smem, st),
                     "pressure solve");
   if (!rc)
-    rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(PSolveResult), cudaMemcpyDeviceToHost, st),
+    rc = check_cuda(ctx, cudaMemcpyAsync(h, a.res, sizeof(SolveStatus), cudaMemcpyDeviceToHost, st),
                     "pressure solve result");
   if (!rc) rc = check_cuda(ctx, cudaStreamSynchronize(st), "pressure solve sync");
   if (rc) return rc;
   *launches += 1;
-  if (h->iters < 0)  // the kernel gave up before it could write its result
+  if (h->bar[2])  // given up by any block: some of the solution may not have been written
     return set_error(ctx, RBFFD_ERR_CUDA, "pressure solve: grid barrier not reached (bounded wait)");
-  *res = *h;
+  *res = h->res;
   return RBFFD_OK;
 }
 

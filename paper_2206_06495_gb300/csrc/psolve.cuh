@@ -9,6 +9,9 @@ namespace rbffd {
 
 struct PSolve;
 
+// polls of a grid barrier's wait in the kernels that `ctx` launches
+long long barrier_polls(const rbffd_ctx* ctx);
+
 // Up to this many rows the resident kernel is the faster form (FP64 step at 1M
 // rows: 0.38 against 0.41 ms an iteration as separate launches, at 100k rows
 // 0.08 against 0.13); larger systems have not been measured and keep the graph
@@ -20,6 +23,13 @@ struct PSolveResult {
   int status = 0;  // as KScal::status of step.cu
   double relres = 0.0;
   bool converged = false;
+};
+
+// A solve's result and, behind it, its barrier's words: one copy to the host.
+constexpr int kBarrierWords = 3;
+struct SolveStatus {
+  PSolveResult res;
+  unsigned int bar[kBarrierWords];
 };
 
 // Build the solve's copies for one plan: the scaled pressure operator (idx, w
@@ -84,8 +94,8 @@ cudaError_t small_reset(VSolve* v, DSolve* d, int* fail, cudaStream_t st);
 // accept: a relative residual up to which a viscous solve short of tol passes
 cudaError_t vsolve_enqueue(VSolve* v, double* const* x, const double* const* b, double tol,
                            double accept, int maxit, PSolveResult* res, int* fail, int step,
-                           cudaStream_t st);
+                           long long polls, cudaStream_t st);
 cudaError_t dsolve_enqueue(DSolve* d, double* x, const double* b, double tol, PSolveResult* res,
-                           int* fail, int step, cudaStream_t st);
+                           int* fail, int step, long long polls, cudaStream_t st);
 
 }  // namespace rbffd

@@ -3235,14 +3235,15 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
         m.nhist[0] = P->nhist;
         if (!rc)
           rc = check_cuda(ctx, vsolve_enqueue(P->vis, hx, hb, vtol, f.tol, f.max_iter,
-                                              &P->small[i].visc, P->fail, i, st),
+                                              &P->small[i].visc, P->fail, i,
+                                              barrier_polls(ctx), st),
                           "viscous solve");
         if (!rc) rc = pressure_input(P->fail);
         m.hhead[1] = P->hhead;
         m.nhist[1] = P->nhist;
         if (!rc)
           rc = check_cuda(ctx, dsolve_enqueue(P->ds, P->px, P->pb, f.tol, &P->small[i].pres,
-                                              P->fail, i, st),
+                                              P->fail, i, barrier_polls(ctx), st),
                           "direct pressure solve");
         if (!rc) rc = back(P->fail);
         P->launches += 2;
@@ -3290,8 +3291,10 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
       P->vhist = m.vhist;
       P->hhead = m.hhead[after];
       P->nhist = m.nhist[after];
-      if (code == kFailWait)
+      if (code == kFailWait) {  // the guesses' rings may have been turned
+        P->px_step = -1;
         return set_error(ctx, RBFFD_ERR_CUDA, "small solve: grid barrier not reached (bounded wait)");
+      }
       if (code == kFailPressure && h[bad].pres.status == 2)
         return set_error(ctx, RBFFD_ERR_NONFINITE, "non-finite pressure solve");
       if (code == kFailPressure)  // refinement at its rounding level above the tolerance

@@ -123,6 +123,7 @@ PROTOTYPES = {
     "rbffd_probe_fma": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.POINTER(C.c_double),
                                   C.c_void_p]),
     "rbffd_debug_set_wait_limit": (C.c_int, [C.c_void_p, C.c_int64]),
+    "rbffd_debug_set_barrier_limit": (C.c_int, [C.c_void_p, C.c_int64]),
     "rbffd_debug_set_solver_bytes": (C.c_int, [C.c_void_p, C.c_int64]),
     "rbffd_ensemble_step": (C.c_int, [C.c_void_p, C.POINTER(FlowC), C.c_int32,
                                       C.POINTER(C.c_double), C.POINTER(StateC), C.c_void_p,
@@ -519,6 +520,12 @@ def debug_set_wait_limit(ctx: Context, polls: int) -> None:
     """rbffd_debug_set_wait_limit (test hook): polls of the first staged-copy
     wait; 0 gives up at once, a negative value restores the default."""
     ctx.check(lib().rbffd_debug_set_wait_limit(ctx.handle, polls))
+
+
+def debug_set_barrier_limit(ctx: Context, polls: int) -> None:
+    """rbffd_debug_set_barrier_limit (test hook): polls of a grid barrier's wait;
+    a negative value restores the default."""
+    ctx.check(lib().rbffd_debug_set_barrier_limit(ctx.handle, polls))
 
 
 def debug_set_solver_bytes(ctx: Context, nbytes: int) -> None:
