@@ -110,6 +110,29 @@ struct Grid {
   }
 };
 
+// A thread's share of a sum over its rows.  FP32 values are added as an
+// unevaluated pair (Knuth's two-sum), exact to 2^-40 for the 13 rows a thread
+// has at most, so that the sum over a grid is as good as one whose FP32 shares
+// are single rows; FP64 additions would take the pipe that retires one warp in
+// 16 cycles.  The intrinsics keep the compiler from fusing a product into the
+// additions.
+template <typename T>
+struct Part {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct Part<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = __fadd_rn(hi, v), b = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(v, b)));
+    hi = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 // Ends a kernel whose arrival counter the next launch finds at zero again: the
 // last block to come here resets it.
 __device__ __forceinline__ void leave(unsigned int* arrivals) {

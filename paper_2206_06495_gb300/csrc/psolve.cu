@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
       p_up_level<PT>(a.lev[l], a.lev[l - 1], first[l], count[l]);
       if (!g.sync()) return false;
     }
-    float part0 = 0.f;
+    Part<float> part0;
     auto sweep0 = [&](auto staged, int i, int gi) {
       constexpr bool ST = decltype(staged)::value;
       const Rows<ST> R = rows_of<ST>(L0);
@@ -414,14 +414,14 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
                                      : p_graph<16, ST>(R, i, L0.x, xi);
       const float zi = xi + ro<ST>(R.wd + i) * (ri - ax);
       z[gi] = (T)zi;
-      part0 += zi;
+      part0.add(zi);
     };
     if (L0.soff >= 0) {
       for (int i = tid; i < count[0]; i += PT) sweep0(std::true_type{}, i, first[0] + i);
     } else {
       for (int i = r0 + tid; i < r1; i += PT) sweep0(std::false_type{}, i, i);
     }
-    const double v[1] = {(double)part0};
+    const double v[1] = {part0.value()};
     return g.template reduce<1>(v, PT, [&](const double* t) { fin(t[0]); });
   };
   auto fin_p = [&](double zsum) { S.kp = (T)((S.mu_p - zsum) * a.inv_R); };
@@ -438,15 +438,15 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
     // r = b - A x; shadow residual rh = r (seed 0) or r with seeded signs; p = r
     const bool zero = a.x_zero && cyc == 0;
     if (!zero) {
-      T sx = 0;
-      for (int i = r0 + tid; i < r1; i += PT) sx += a.x[i];
-      const double v[1] = {(double)sx};
+      Part<T> sx;
+      for (int i = r0 + tid; i < r1; i += PT) sx.add(a.x[i]);
+      const double v[1] = {sx.value()};
       if (!g.template reduce<1>(v, active, [&](const double* t) { S.sig = t[0]; })) return;
     }
     const uint32_t seed = (cyc || a.seed) ? 0x51ED27u + 977u * a.seed + (uint32_t)cyc : 0u;
     {
       const T sig = zero ? (T)0 : (T)S.sig;
-      T prr = 0, pbb = 0, prh = 0, pc = 0;
+      Part<T> prr, pbb, prh, pc;
       for (int i = r0 + tid; i < r1; i += PT) {
         const T bi = a.b[i];
         T ri = bi;
@@ -460,12 +460,12 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
         a.r[i] = ri;
         a.rh[i] = sgn * ri;
         a.p[i] = ri;
-        prr += ri * ri;
-        pbb += bi * bi;
-        prh += sgn * ri * ri;
-        pc += (T)__ldg(a.c + i) * ri;
+        prr.add(ri * ri);
+        pbb.add(bi * bi);
+        prh.add(sgn * ri * ri);
+        pc.add((T)__ldg(a.c + i) * ri);
       }
-      const double v[4] = {(double)prr, (double)pbb, (double)prh, (double)pc};
+      const double v[4] = {prr.value(), pbb.value(), prh.value(), pc.value()};
       const bool ok = g.template reduce<4>(v, active, [&](const double* t) {
         S.rr = t[0];
         S.bb = t[1];
@@ -493,16 +493,16 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
       // v = A p^, p^ = zp + kap_p; (rh, v), (c . v)
       {
         const T kap = S.kp, mu = S.mp;
-        T d0 = 0, d1 = 0;
+        Part<T> d0, d1;
         for (int i = r0 + tid; i < r1; i += PT) {
           const T zi = dif ? a.zp[i] : (T)0;
           const T y = p_row<K, (PT == kLargePT)>(a, i, a.zp, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
                       __ldg(a.es + i) * mu;
           a.v[i] = y;
-          d0 += a.rh[i] * y;
-          d1 += (T)__ldg(a.c + i) * y;
+          d0.add(a.rh[i] * y);
+          d1.add((T)__ldg(a.c + i) * y);
         }
-        const double v[2] = {(double)d0, (double)d1};
+        const double v[2] = {d0.value(), d1.value()};
         const bool ok = g.template reduce<2>(v, active, [&](const double* t) {
           if (t[0] == 0.0 || !isfinite(t[0])) {
             S.status = isfinite(t[0]) ? 1 : 2;
@@ -526,15 +526,15 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
       {
         const T al = S.al;
         const float mu = S.fs;
-        T d0 = 0, d1 = 0;
+        Part<T> d0, d1;
         for (int i = r0 + tid; i < r1; i += PT) {
           const T si = a.r[i] - al * a.v[i];
           a.s[i] = si;
           feed(i, si, mu);
-          d0 += si * si;
-          d1 += a.rh[i] * si;
+          d0.add(si * si);
+          d1.add(a.rh[i] * si);
         }
-        const double v[2] = {(double)d0, (double)d1};
+        const double v[2] = {d0.value(), d1.value()};
         const bool ok = g.template reduce<2>(v, active, [&](const double* t) {
           S.rhs = t[1];
           if (t[0] <= a.tol2 * S.bb) {  // converged at the half step
@@ -555,18 +555,18 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
       // t = A s^, s^ = zs + kap_s; (t, s), (t, t), (c . t), (rh, t)
       {
         const T kap = S.ks, mu = S.ms;
-        T d0 = 0, d1 = 0, d2 = 0, d3 = 0;
+        Part<T> d0, d1, d2, d3;
         for (int i = r0 + tid; i < r1; i += PT) {
           const T zi = dif ? a.zs[i] : (T)0;
           const T y = p_row<K, (PT == kLargePT)>(a, i, a.zs, zi) + (dif ? zi + kap : kap) * __ldg(a.a1 + i) +
                       __ldg(a.es + i) * mu;
           a.t[i] = y;
-          d0 += y * a.s[i];
-          d1 += y * y;
-          d2 += (T)__ldg(a.c + i) * y;
-          d3 += a.rh[i] * y;
+          d0.add(y * a.s[i]);
+          d1.add(y * y);
+          d2.add((T)__ldg(a.c + i) * y);
+          d3.add(a.rh[i] * y);
         }
-        const double v[4] = {(double)d0, (double)d1, (double)d2, (double)d3};
+        const double v[4] = {d0.value(), d1.value(), d2.value(), d3.value()};
         const bool ok = g.template reduce<4>(v, active, [&](const double* t) {
           if (!(t[1] > 0.0) || !isfinite(t[0])) {
             S.status = isfinite(t[1]) ? 3 : 2;
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
       {
         const T al = S.al, om = S.om, be = S.be, shift = al * S.kp + om * S.ks;
         const float mu = S.fp;
-        T d0 = 0;
+        Part<T> d0;
         for (int i = r0 + tid; i < r1; i += PT) {
           a.x[i] += al * a.zp[i] + (om * a.zs[i] + shift);
           const T ri = a.s[i] - om * a.t[i];
@@ -603,9 +603,9 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
           const T pi = ri + be * (a.p[i] - om * a.v[i]);
           a.p[i] = pi;
           feed(i, pi, mu);
-          d0 += ri * ri;
+          d0.add(ri * ri);
         }
-        const double v[1] = {(double)d0};
+        const double v[1] = {d0.value()};
         const bool ok = g.template reduce<1>(v, active, [&](const double* t) {
           const double rr = t[0];
           const bool conv = rr <= a.tol2 * S.bb;
