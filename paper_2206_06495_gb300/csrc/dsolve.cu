@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
               S.active[q] = 0;
               S.status = isfinite(q2[q]) ? 1 : 2;
             } else {
-              S.alpha[q] = quot(S.rho[q], q2[q]);
+              S.alpha[q] = S.rho[q] / q2[q];
               S.go = 1;
             }
           }
@@ -523,9 +523,9 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
               S.status = isfinite(tt) ? 3 : 2;
               continue;
             }
-            const double om = quot(ts, tt), rn = S.rhs[q] - om * q6[3 * q + 2];
+            const double om = ts / tt, rn = S.rhs[q] - om * q6[3 * q + 2];
             const double rr = fmax(S.ss[q] - om * ts, 0.0) + 1e-14 * S.ss[q];
-            S.beta[q] = quot(rn, S.rho[q]) * quot(S.alpha[q], om);
+            S.beta[q] = (rn / S.rho[q]) * (S.alpha[q] / om);
             S.omega[q] = om;
             S.rho[q] = rn;
             S.rr[q] = rr;

@@ -143,18 +143,6 @@ __device__ __forceinline__ void leave(unsigned int* arrivals) {
   }
 }
 
-// a / b for the scalars of a solve (one thread's work, which every block waits
-// for): the approximate reciprocal instruction and two steps of Newton's
-// iteration for 1 / b, a shorter serial chain than a correctly rounded
-// division; within two units in the last place.
-__device__ __forceinline__ double quot(double a, double b) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  y = fma(y, fma(-b, y, 1.0), y);
-  y = fma(y, fma(-b, y, 1.0), y);
-  return fabs(b) > 1e-290 && fabs(b) < 1e290 ? a * y : a / b;
-}
-
 // sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
 __device__ __forceinline__ float hash_sign(int i, uint32_t seed) {
   uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;

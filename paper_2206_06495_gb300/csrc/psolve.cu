@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
             S.ended = 1;
             return;
           }
-          S.alpha = quot(S.rho, t[0]);
+          S.alpha = S.rho / t[0];
           S.al = (T)S.alpha;
           S.cv = t[1];
           S.cs = S.cr - S.alpha * t[1];
@@ -575,9 +575,9 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
             S.ended = 1;
             return;
           }
-          const double om = quot(t[0], t[1]);
+          const double om = t[0] / t[1];
           const double rn = S.rhs - om * t[3];
-          const double be = quot(rn, S.rho) * quot(S.alpha, om);
+          const double be = (rn / S.rho) * (S.alpha / om);
           S.rho = rn;
           S.omega = om;
           S.om = (T)om;

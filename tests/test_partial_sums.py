@@ -39,3 +39,10 @@ def test_fp32_shares_lose_nothing_that_fp64_sums_keep(n, tmp_path):
         assert abs(total(v) - math.fsum(v.tolist())) <= 2.0 ** -40 * np.abs(v).sum(dtype=float)
     v[0] = np.inf
     assert not math.isfinite(total(v))
+
+
+def test_solve_scalars_are_correctly_rounded_quotients():
+    """alpha, omega and beta of the resident solves are the compiler's divisions:
+    no approximate FP64 instruction in their sources."""
+    for f in ("gridsync.cuh", "psolve.cu", "dsolve.cu"):
+        assert ".approx" not in open(build.CSRC + "/" + f).read(), f
