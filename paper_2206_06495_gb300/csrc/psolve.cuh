@@ -12,11 +12,16 @@ struct PSolve;
 // polls of a grid barrier's wait in the kernels that `ctx` launches
 long long barrier_polls(const rbffd_ctx* ctx);
 
-// Up to this many rows the resident kernel is the faster form (FP64 step at 1M
-// rows: 0.38 against 0.41 ms an iteration as separate launches, at 100k rows
-// 0.08 against 0.13); larger systems have not been measured and keep the graph
-// of separate launches.
-constexpr int64_t kResidentMax = 1 << 21;
+// Up to this many rows the resident kernel is the faster form.  Milliseconds of
+// a step for each of its pressure iterations, resident against launched, of two
+// flows: rows of 28 entries, FP64, 0.69 and 0.63 against 0.71 and 0.66 at 1.10M
+// rows, 0.71 and 0.81 against 0.66 and 0.74 at 1.21M, 0.90 and 0.89 against
+// 0.83 and 0.83 at 1.32M, 1.24 against 1.11 at 2.0M (1.69M alone is even);
+// MIXED 0.53 against 0.53 and 0.54 at 1.10M, 0.58 and 0.57 against 0.56 and
+// 0.55 at 1.21M, 0.87 against 0.83 at 2.0M.  Rows of another width, whose
+// products are loops, FP64 at 2.0M: 1.51 against 1.54 (21 entries) and 1.66
+// against 1.95 (composed); larger systems have not been measured.
+constexpr int64_t kResidentMax28 = 1150000, kResidentMax = 1 << 21;
 
 struct PSolveResult {
   int iters = 0;

@@ -2089,7 +2089,7 @@ int build_precond(rbffd_ctx* ctx, StepPlan* p, const rbffd_flow& f, const std::v
       return rc;
   }
   if ((rc = amg_build(ctx, f, hd.data(), hes.data(), &p->amg, st))) return rc;
-  if (f.M > kResidentMax) return RBFFD_OK;
+  if (f.M > (p->kL == 28 ? kResidentMax28 : kResidentMax)) return RBFFD_OK;
   return psolve_build(ctx, f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->es, p->a1, p->amg, p->mix,
                       &p->ps, st);
 }

@@ -141,3 +141,21 @@ def test_pressure_graphs_are_refused_alike(profile):
         R.step(ctx, flow, st, gu, gv, 1)
     assert err.value.code == R.ERR_INVALID_ARG and "not positive" in str(err.value)
     assert st.j == 0
+
+
+# 1.10M and 1.21M rows: either side of the limit for rows of 28 entries; another
+# width stays resident
+@pytest.mark.parametrize("n,stencil,resident", [(1050, (28, 7, 3), True),
+                                                (1100, (28, 7, 3), False),
+                                                (1100, (21, 5, 2), True)])
+def test_large_systems_take_the_faster_form(n, stencil, resident):
+    """A resident solve is one launch, a launched one some 25 an iteration."""
+    from paper_2206_06495_gb300 import rbffd as R
+    nd = ns.jittered_cavity(n, 3)
+    ctx = R.Context(*stencil)
+    flow = R.flow_from_nodes(ctx, nd, Re=1000.0, dt=0.08 / (n - 1), tol=1e-6)
+    gu, gv = (_d(g) for g in O.lid_bc(nd))
+    st = R.State.zeros(flow)
+    stats = R.step(ctx, flow, st, gu, gv, 1)
+    assert stats["poisson_iters"] >= 10
+    assert (stats["launches"] < 10 * stats["poisson_iters"]) == resident, stats
