@@ -335,9 +335,13 @@ typedef struct rbffd_state {
 /* Per-call statistics (host struct, filled by rbffd_step). */
 typedef struct rbffd_stats {
   int64_t steps;            /* steps taken                                    */
-  int64_t helm_iters;       /* Krylov iterations of the viscous solves        */
-  int64_t poisson_iters;    /* Krylov iterations of the pressure solves      */
-  int64_t refinements;      /* FP64 refinement sweeps (MIXED)                 */
+  int64_t helm_iters;       /* Krylov iterations of the viscous solves (closed
+                               flows: one count for both components)          */
+  int64_t poisson_iters;    /* iterations of the pressure solves: Krylov
+                               iterations, or products with the inverse where
+                               the solve is direct (at most 4,096 P-nodes)    */
+  int64_t refinements;      /* MIXED: FP64 refinement sweeps of both solves (a
+                               direct solve's are its products)               */
   double helm_relres;       /* last relative residual, viscous solve         */
   double poisson_relres;    /* last relative residual, pressure solve        */
   int64_t launches;         /* kernels launched by this call                  */

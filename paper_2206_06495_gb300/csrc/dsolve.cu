@@ -320,6 +320,7 @@ struct VArgs {
 struct VScal {
   double rho[2], rr[2], ss[2], bb[2], rhs[2], alpha[2], omega[2], beta[2];
   int active[2], mode[2], status, iters, total, go, iterate;
+  int its[2];  // iterations of each component, over all restarts
 };
 
 // What bounds it: latency, four phases an iteration (a barrier of 1.3 us, the
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
   const double2* Sv = reinterpret_cast<const double2*>(a.s);
   const double b = mine ? a.b[c][i] : 0.0, x0 = mine ? a.x[c][i] : 0.0;
   double x = x0, r = 0.0, rh = 0.0, p = 0.0, v = 0.0, s = 0.0, t = 0.0;
-  if (tid == 0) S.total = 0;
+  if (tid == 0) S.total = S.its[0] = S.its[1] = 0;
   for (int cyc = 0;; ++cyc) {
     {
       const uint32_t seed = cyc ? 0x51ED27u + (uint32_t)cyc : 0u;
@@ -487,6 +488,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
             S.rhs[q] = q4[2 * q + 1];
             if (S.ss[q] <= a.tol2 * S.bb[q]) {
               S.rr[q] = S.ss[q];
+              S.its[q] += 1;
               S.mode[q] = 1;
               S.active[q] = 0;
             } else {
@@ -516,6 +518,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
           int any = 0;
           for (int q = 0; q < 2; ++q) {
             if (S.mode[q] != 2) continue;
+            S.its[q] += 1;
             const double ts = q6[3 * q], tt = q6[3 * q + 1];
             S.active[q] = 0;
             if (!(tt > 0.0) || !isfinite(ts)) {
@@ -573,7 +576,9 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
         double worst = 0.0;
         for (int q = 0; q < 2; ++q)
           worst = fmax(worst, S.bb[q] > 0 ? sqrt(S.rr[q] / S.bb[q]) : sqrt(S.rr[q]));
-        a.res->iters = tot;
+        // an open flow's components are systems of their own, whose iterations
+        // add up; a closed flow's are two right sides of one
+        a.res->iters = same ? tot : S.its[0] + S.its[1];
         a.res->status = st;
         a.res->relres = worst;
         a.res->converged = conv;
