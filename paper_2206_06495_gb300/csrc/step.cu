@@ -2285,6 +2285,11 @@ int build_plan(rbffd_ctx* ctx, const rbffd_flow& f, StepPlan** out, cudaStream_t
       TRY(dsolve_build(ctx, f.M, f.ld_p, p->kL, p->Lidx, p->Lw, p->es, &p->ds, st));
     }
     if (!p->ds) TRY(build_precond(ctx, p, f, hd, hes, st));
+    // Up to 8,192 V-nodes, the set on which the form was measured first.  It is the
+    // faster one beyond, too, up to the largest flow with a direct pressure solve
+    // (20 FP64 steps of cavities with 53, 58 and 64 P-nodes a side: 9.3, 9.9 and
+    // 11.0 ms launched, 5.0, 5.5 and 6.6 enqueued), and MIXED flows have not been
+    // measured in it: the line has not been moved yet.
     if (p->ds && !p->mix && f.N <= 2 * kDenseMax) {
       TRY(vsolve_build(ctx, f.N, f.ld_v, p->k, p->open ? p->Hidx : f.vv_idx, p->Hw,
                        p->open ? p->Hw_v : p->Hw, &p->vis, st));
