@@ -90,6 +90,15 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NV], GridReduce gr, doub
   }
 }
 
+// sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
+__device__ __forceinline__ float shadow_sign(int64_t i, uint32_t seed) {
+  uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  h ^= h >> 12;
+  return (h & 1u) ? 1.f : -1.f;
+}
+
 }  // namespace rbffd
 
 // ------------------------------------------------------------------ context

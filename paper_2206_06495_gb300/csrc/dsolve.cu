@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kVT, 1) k_vsolve(const __grid_constant__ VArgs
       double d[3] = {};
       if (tid < active) {
         r = b - (x + row([&](int j) { return make_double2(a.x[0][j], a.x[1][j]); }));
-        rh = seed ? (double)hash_sign(i, seed) * r : r;
+        rh = seed ? (double)shadow_sign(i, seed) * r : r;
         p = r;
         if (own) {
           a.p[2 * i + c] = p;

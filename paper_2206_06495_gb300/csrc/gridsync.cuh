@@ -143,13 +143,4 @@ __device__ __forceinline__ void leave(unsigned int* arrivals) {
   }
 }
 
-// sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
-__device__ __forceinline__ float hash_sign(int i, uint32_t seed) {
-  uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;
-  h ^= h >> 15;
-  h *= 0x2C1B3C6Du;
-  h ^= h >> 12;
-  return (h & 1u) ? 1.f : -1.f;
-}
-
 }  // namespace rbffd

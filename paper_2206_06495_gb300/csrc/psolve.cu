@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(PT, 1) k_psolve(const __grid_constant__ PArgs<
           if (dif) ax += a.a1[i] * xi;
           ri = bi - (ax + a.es[i] * sig);
         }
-        const T sgn = seed ? (T)hash_sign(__ldg(a.perm + i), seed) : (T)1;
+        const T sgn = seed ? (T)shadow_sign(__ldg(a.perm + i), seed) : (T)1;
         a.r[i] = ri;
         a.rh[i] = sgn * ri;
         a.p[i] = ri;

@@ -302,15 +302,6 @@ __global__ void __launch_bounds__(kThreads) k_sum(const TV* __restrict__ x, int6
   grid_reduce<NU_>(v, gr, sh, [&](double* t) { *out = t[0]; });
 }
 
-// sign pattern of a restarted shadow residual (a 32-bit integer hash of i and the seed)
-__device__ __forceinline__ float shadow_sign(int64_t i, uint32_t seed) {
-  uint32_t h = (uint32_t)i * 0x9E3779B1u ^ seed * 0x85EBCA77u;
-  h ^= h >> 15;
-  h *= 0x2C1B3C6Du;
-  h ^= h >> 12;
-  return (h & 1u) ? 1.f : -1.f;
-}
-
 // r = b - A x ; p = r ; shadow residual rh = r (seed 0) or r with seeded signs
 template <int K, int NRHS, bool RANK1, typename TW, typename TV>
 __global__ void __launch_bounds__(kThreads)
@@ -3275,8 +3266,6 @@ int run_steps(rbffd_ctx* ctx, StepPlan* P, const rbffd_flow& f, rbffd_state* s, 
         if (stats && (i < bad || code == kFailPressure)) {
           stats->helm_iters += h[i].visc.iters;
           stats->helm_relres = h[i].visc.relres;
-        }
-        if (stats && (i < bad || code == kFailPressure)) {
           stats->poisson_iters += h[i].pres.iters;
           stats->poisson_relres = h[i].pres.relres;
         }
