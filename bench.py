@@ -630,7 +630,10 @@ def run_ours(args):
     # of a k = 28 stencil SpMV row (k column indices, k weights, the operand
     # read once, the output written: 232 B in FP32, 352 B in FP64); the
     # kernel also streams three fused per-row vectors (the dot-product
-    # partner, the row sum A 1 and the rank-one column), listed apart
+    # partner, the row sum A 1 and the rank-one column), listed apart.  It is
+    # the product of the launched solve, which a profiled step takes; the timed
+    # steps form the same product inside the resident solve k_psolve (up to
+    # 1.15M rows), where it cannot be timed by events
     k = 28
     if head == "mixed":
         bytes_row, fused, key = 8 * k + 2 * 4, 3 * 4, "k_spmv_pc_fp32"  # FP32 inner solves
@@ -646,7 +649,9 @@ def run_ours(args):
     in_step = (nd.M * bytes_row / (in_step_ms * 1e-3) / 1e9
                if r["spmv_launches"] > 0 and in_step_ms > 0 else None)
     traffic = profiled_traffic(key, nd.M)
-    pres_roof = {"kernel": key, "bound": "hbm", "achieved": achieved, "peak": hbm,
+    pres_roof = {"kernel": key, "form": "launched solve of a profiled step; the timed steps "
+                                        "solve in the resident kernel k_psolve",
+                 "bound": "hbm", "achieved": achieved, "peak": hbm,
                  "unit": "GB/s", "frac": achieved / hbm if achieved else None,
                  "traffic": traffic,
                  "bytes_per_row": bytes_row, "fused_bytes_per_row": fused,
@@ -811,7 +816,7 @@ def ensemble_record(R, args, hbm, peak_kind):
                 "sequential_fp64_steps_per_s": seq["fp64"][0],
                 "sequential_fp64_poisson_iters_per_step": seq["fp64"][1],
                 "speedup_vs_best_sequential": rate / max(seq_rate, seq["fp64"][0]),
-                "spmm_roofline": {"kernel": "e_spmv_v (batched pressure SpMV)", "bound": "hbm",
+                "spmm_roofline": {"kernel": "e_spmv (batched pressure SpMV)", "bound": "hbm",
                                   "bytes_per_member_row": (k * 8) / E + 8,
                                   "us_per_launch": per_ms * 1e3, "achieved": achieved,
                                   "peak": hbm, "unit": "GB/s", "peak_kind": peak_kind,
