@@ -35,7 +35,10 @@ namespace {
 // are reloaded through L2 in every phase (each barrier empties L1), 0.7 us a
 // phase (FP64 100k rows: 94 against 104 us an iteration; MIXED 250k: 123 against
 // 140).  1,024 where they are bound by the streams and need the loads in
-// flight (FP64 1M rows: 0.38 against 0.46 ms).
+// flight (FP64 1M rows: 0.38 against 0.46 ms).  The line: milliseconds of a step
+// for each pressure iteration with 512 and with 1,024, FP64 0.161 and 0.182 at
+// 200k rows, 0.195 and 0.189 at 250k, 0.228 and 0.203 at 300k; MIXED 0.142 and
+// 0.161, 0.152 and 0.169, 0.189 and 0.176.
 constexpr int kSmallPT = 512, kLargePT = 1024;
 constexpr int64_t kLargeRows = 300000;
 constexpr int kCycle = 50;            // iterations before a restart from the true residual

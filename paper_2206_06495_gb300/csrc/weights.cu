@@ -20,7 +20,7 @@
 // right-hand sides share one root per node: 1,200 FP64 instructions a stencil
 // against 1,890 before, with the same weights bit for bit, but for a reciprocal
 // or a root in some 2e9 that misses the correct rounding (1.08M stencils with
-// three operators: 77.7 against 89.6 ms; the pipe is 88 % busy).
+// three operators: 77.7 against 89.6 ms; the pipe is 85 % busy).
 //
 // Local coordinates (the "shift and scale" of the implementation the paper
 // follows): stencil nodes are shifted to the alpha-node and divided by the
